@@ -370,10 +370,13 @@ mpm_status decoder_status_word(mpm_decoder* dec, uint32_t* out, int clear, void*
 /*
  * Arithmetic of the square hidden layers in decoder_eval and in the reduced
  * step's decoder calls (training always uses the tensor cores).  fp32 = 0
- * (default): BF16 x BF16 -> FP32 tcgen05 GEMMs.  fp32 = 1: FP32 GEMMs on the
- * CUDA cores from the FP32 master weights; for the reduced step's small calls,
- * whose time is set by per-tile latency rather than throughput, this costs
- * little and removes the BF16 rounding of positions and gradients.  fp32 = 2:
+ * (default): BF16 x BF16 -> FP32 tcgen05 GEMMs.  fp32 = 1: FP32 accuracy from
+ * the FP32 master weights, on the tensor cores with every operand the exact sum
+ * of three BF16 numbers (six products, FP32 accumulation), or as FP32 GEMMs on
+ * the CUDA cores where those are faster or their rounding is kept (mixed rows,
+ * a lone caller's small calls with secant rows, gradients measured against a
+ * reference configuration); it removes the BF16 rounding of positions and
+ * gradients.  fp32 = 2:
  * split BF16 on the tensor cores: activations and weights are each the sum of
  * two BF16 numbers (hi = bf16(v), lo = bf16(v - hi)) and every product is
  * A_hi W_hi + A_hi W_lo + A_lo W_hi accumulated in FP32, so each product keeps

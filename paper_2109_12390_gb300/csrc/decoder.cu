@@ -1031,6 +1031,522 @@ __global__ void __launch_bounds__(kF32Threads, 1) decoder_f32(DecArgs a) {
   cp_async_wait_all();
 }
 
+// --------------------------------------------------------------------------
+// FP32-accurate decoder on the tensor cores (decoder_tc3).  Every FP32 operand is held as the
+// exact sum of three BF16 numbers, v = hi + mid + lo (8 + 8 + 8 significand bits; weights split by
+// rounding, activations by truncation), and a layer is the six products of weight 2^-16 and above,
+//   A W ~ Ah Wl + Am Wm + Ah Wm + Al Wh + Am Wh + Ah Wh,
+// accumulated in FP32 in that order (small terms first, so that the accumulator holds its final
+// magnitude for the eight K steps of Ah Wh only); the dropped products are below 2^-23 of each term
+// with signs of their own.  All layers but the output layer (N = d, FP32 on the CUDA cores) run
+// this way, the first one with K = d + r padded to a multiple of 16.
+//
+// A tile is 128 rows: four lane groups of 32 rows, each owned by four warps (32 columns apiece).
+// Rows are taken in (point, kind) order, so that a derivative row finds its point's primal
+// pre-activation in another lane of its warp (one shuffle per feature; no exchange through shared
+// memory and no block barrier):
+//   tc3_U = 32   32 % R == 0: a lane group holds whole points;
+//   tc3_U = 31   any R: 31 consecutive rows, lane 0 recomputing the primal row of the first one's
+//                point (not written out).
+// NS tile slots per CTA: the sixteen epilogue warps take the slots in turn, so that one slot's
+// epilogue overlaps the other's MMAs (NS = 1: calls of at most one tile per SM).  The A operand's
+// high and middle images sit in tensor memory (written by the epilogue with tcgen05.st), the low
+// image in shared memory; the accumulator takes 128 more columns.  One warp streams the weights
+// (atoms of 128 rows x 64 K, 16 KB) through a ring of kRing slots with bulk copies, one warp per
+// tile slot issues its MMAs.  A ring slot is refilled once both tile slots' MMAs on it completed.
+// What bounds it: per tile and layer the tensor core takes 48 MMAs (about 65 cycles each), the sixteen
+// epilogue warps about 3.8k cycles (21 instructions per element, 2.2 of 4 issue slots), the two
+// overlapped.  262,144 points x 4 rows, r = 16: 0.71 ms (decoder_f32: 5.07 ms), distance from 64 bits
+// 4e-8 .. 7e-8 (6.5e-8); 256 points x 17 rows: 27 us (31 us).
+// After a wait that ran out nothing waits on the copies or MMAs any more: the pass runs to its end
+// (in bounds, its results void) with the TIMEOUT status raised.
+// --------------------------------------------------------------------------
+constexpr int kTc3Epi = 512;              // epilogue threads
+constexpr int kAtomBytes = kW * 128;      // 128 rows x 64 BF16
+constexpr int kRing = 9;
+template <int NS>
+constexpr int tc3_threads() { return kTc3Epi + 32 + 32 * NS; }
+
+struct __align__(8) Tc3Tail {
+  uint64_t full[kRing];
+  uint64_t empty[kRing];
+  uint64_t bar_mma[2];
+  uint64_t drain;
+  uint32_t tmem;
+  int abort;      // a wait ran out
+};
+
+// Bounded wait; after a timeout anywhere in the CTA no further waits are made.
+__device__ __forceinline__ void tc3_wait(const DecArgs& a, int* abort, uint64_t* bar, uint32_t phase) {
+  if (*(volatile int*)abort) return;
+  if (!tc::mbar_wait(bar, phase)) {
+    raise_status(a.status, STATUS_TIMEOUT);
+    atomicExch(abort, 1);
+  }
+}
+
+// Barriers 1 + s: the epilogue warps arrive when slot s's next operand is complete (and its
+// accumulator read), the slot's issuer warp waits.  Barriers 3 + s: the issuer arrives when the
+// accumulator is complete, the epilogue warps wait (blocked, where polling the MMA barrier would
+// take issue slots).  Barrier 5: the epilogue warps among themselves.
+__device__ __forceinline__ void tc3_arrive(int id) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kTc3Epi + 32) : "memory");
+}
+__device__ __forceinline__ void tc3_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kTc3Epi + 32) : "memory");
+}
+__device__ __forceinline__ void tc3_epi_sync() { asm volatile("bar.sync 5, %0;" ::"n"(kTc3Epi) : "memory"); }
+
+// 2^x on the special-function unit, results below the normal range flushed to zero
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x));
+  return e;
+}
+// Pairs of FP32 operations in one instruction (each rounded as the scalar operation)
+__device__ __forceinline__ void add2(float& a0, float& a1, float b0, float b1) {
+  asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n add.rn.f32x2 a, a, b;\n"
+      " mov.b64 {%0, %1}, a;\n}\n"
+      : "+f"(a0), "+f"(a1)
+      : "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void mul2(float& a0, float& a1, float b) {
+  asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %2};\n mul.rn.f32x2 a, a, b;\n"
+      " mov.b64 {%0, %1}, a;\n}\n"
+      : "+f"(a0), "+f"(a1)
+      : "f"(b));
+}
+__device__ __forceinline__ void fma2(float& a0, float& a1, float b0, float b1, float c) {   // a += b c
+  asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n mov.b64 c, {%4, %4};\n"
+      " fma.rn.f32x2 a, b, c, a;\n mov.b64 {%0, %1}, a;\n}\n"
+      : "+f"(a0), "+f"(a1)
+      : "f"(b0), "f"(b1), "f"(c));
+}
+constexpr float kLog2e = 1.4426950408889634f;   // __expf(z) is 2^(z kLog2e)
+
+// hi, mid and lo words (two BF16 values each, first value in the low half) of an FP32 pair: each
+// image the truncation of what the previous ones leave, so the three hold the 24 bits exactly
+__device__ __forceinline__ void split3(float v0, float v1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  constexpr uint32_t top = 0xffff0000u, neg = 0x80000000u;
+  uint32_t u0 = __float_as_uint(v0), u1 = __float_as_uint(v1);
+  hi = __byte_perm(u0, u1, 0x7632);
+  add2(v0, v1, __uint_as_float((u0 & top) ^ neg), __uint_as_float((u1 & top) ^ neg));
+  u0 = __float_as_uint(v0);
+  u1 = __float_as_uint(v1);
+  mid = __byte_perm(u0, u1, 0x7632);
+  add2(v0, v1, __uint_as_float((u0 & top) ^ neg), __uint_as_float((u1 & top) ^ neg));
+  lo = __byte_perm(__float_as_uint(v0), __float_as_uint(v1), 0x7632);
+}
+
+// One thread's row of a tile slot.
+struct Tc3Row {
+  int cls, psrc, kidx;   // class, lane of the point's primal row, output block (-1: not written)
+  int64_t p;             // point
+};
+
+template <int NS>
+__global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  // 1024-byte alignment by an offset, so that the pointers stay known as shared memory
+  uint8_t* smem = smem_raw + ((1024u - (tc::smem_addr(smem_raw) & 1023u)) & 1023u);
+  uint8_t* ring = smem;                                  // kRing x 16 KB weight atoms
+  uint8_t* lotile = ring + kRing * kAtomBytes;           // NS x 32 KB low images
+  float* ypart = (float*)(lotile + NS * kLayerBytes);    // [3][128][3]
+  float* sb0 = ypart + 3 * 128 * 3;                      // [128]
+  float* sbh = sb0 + kW;                                 // [kMaxTC][128]
+  float* sWout = sbh + kMaxTC * kW;                      // [3][128]
+  Tc3Tail* tail = (Tc3Tail*)(sWout + 3 * kW);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+
+  if (t == 0) {
+    for (int i = 0; i < kRing; ++i) {
+      tc::mbar_init(&tail->full[i], 1);
+      tc::mbar_init(&tail->empty[i], NS);
+    }
+    tc::mbar_init(&tail->bar_mma[0], 1);
+    tc::mbar_init(&tail->bar_mma[1], 1);
+    tc::mbar_init(&tail->drain, NS);
+    tail->abort = 0;
+    tc::fence_mbar_init();
+  }
+  if (warp == 0) tc::tmem_alloc<256 * NS>(&tail->tmem);
+  for (int e = t; e < kW; e += tc3_threads<NS>()) sb0[e] = a.b0[e];
+  for (int e = t; e < a.n_tc * kW; e += tc3_threads<NS>()) sbh[e] = a.bh[e];
+  for (int e = t; e < 3 * kW; e += tc3_threads<NS>()) sWout[e] = e < a.d * kW ? a.Wout[e] : 0.f;
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+
+  const int64_t n_pts = dec_count(a);
+  const int64_t n_rows = n_pts * a.R;
+  const int U = a.tc3_U;
+  const int64_t n_tiles = (n_rows + 4 * U - 1) / (4 * U);
+  // tiles per pass: one while every tile has a CTA of its own (slot 1 then has none)
+  const int NT = n_tiles <= gridDim.x ? 1 : NS;
+  const int64_t n_iter = (n_tiles + NT - 1) / NT;
+  const int K0 = a.d + a.r;
+  const int KS0 = (K0 + 15) / 16;                         // first-layer K steps
+  const int atoms = 3 + 6 * a.n_tc;
+
+  if (warp == kTc3Epi / 32) {
+    // ---- weight stream
+    if (lane == 0) {
+      uint32_t i = 0;
+      for (int64_t it = blockIdx.x; it < n_iter; it += gridDim.x)
+        for (int j = 0; j < atoms; ++j, ++i) {
+          const uint32_t slot = i % kRing, use = i / kRing;
+          if (use > 0) tc3_wait(a, &tail->abort, &tail->empty[slot], (use - 1) & 1u);
+          tc::mbar_expect_tx(&tail->full[slot], (uint32_t)kAtomBytes);
+          tc::bulk_g2s(ring + slot * kAtomBytes, a.wstream + (size_t)j * kAtomBytes, kAtomBytes, &tail->full[slot]);
+        }
+      // the last copies land before the CTA exits (only a timed-out pass leaves any in flight)
+      if (*(volatile int*)&tail->abort)
+        for (uint32_t k = i > kRing ? i - kRing : 0; k < i; ++k)
+          (void)tc::mbar_wait(&tail->full[k % kRing], (k / kRing) & 1u);
+    }
+    __syncwarp();
+  } else if (warp > kTc3Epi / 32) {
+    // ---- MMA issuer of slot s.  The whole warp runs the loop; one elected lane issues.
+    const int s = warp - kTc3Epi / 32 - 1;
+    const bool leader = tc::elect_one();
+    const uint32_t tD = tail->tmem + (uint32_t)(s * 256), tAh = tD + 128, tAm = tD + 192;
+    const uint32_t lo_desc = tc::smem_desc_sw128_lo(tc::smem_addr(lotile + s * kLayerBytes));
+    const uint32_t ring_desc = tc::smem_desc_sw128_lo(tc::smem_addr(ring));
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW), kAtomDesc = kAtomBytes >> 4;
+    uint32_t atom = 0, mma_phase = 0;
+    // waits for the next atom of the stream, returns its ring slot
+    auto take = [&]() {
+      const uint32_t slot = atom % kRing;
+      tc3_wait(a, &tail->abort, &tail->full[slot], (atom / kRing) & 1u);
+      __syncwarp();
+      ++atom;
+      return slot;
+    };
+    for (int64_t it = blockIdx.x; it < n_iter; it += gridDim.x) {
+      if (s >= NT || it * NT + s >= n_tiles) {
+        // no tile: the slot only releases the pass's atoms
+        for (int j = 0; j < atoms; ++j) {
+          const uint32_t r = take();
+          if (leader) tc::mbar_arrive(&tail->empty[r]);
+        }
+        continue;
+      }
+      for (int l = -1; l < a.n_tc; ++l) {
+        tc3_sync(1 + s);
+        tc::tc_fence_after();
+        if (l < 0) {
+          // first layer: one atom per image, KS0 K steps
+          for (int img = 0; img < 3; ++img) {
+            const uint32_t r = take();
+            if (leader) {
+              const uint32_t bd = ring_desc + r * kAtomDesc;
+              auto desc = [](uint32_t lo) { return ((uint64_t)tc::kDescSw128Hi << 32) | lo; };
+              if (img == 2)
+                for (int k = 0; k < KS0; ++k)
+                  tc::mma_bf16(tD, desc(lo_desc + 2 * k), desc(bd + 2 * k), idesc, 1u);
+              if (img > 0)
+                for (int k = 0; k < KS0; ++k) tc::mma_bf16_ts(tD, tAm + 8 * k, desc(bd + 2 * k), idesc, 1u);
+              for (int k = 0; k < KS0; ++k)
+                tc::mma_bf16_ts(tD, tAh + 8 * k, desc(bd + 2 * k), idesc, img > 0 || k > 0 ? 1u : 0u);
+              tc::mma_commit(&tail->empty[r]);
+            }
+            __syncwarp();
+          }
+        } else {
+#pragma unroll
+          for (int kh = 0; kh < 2; ++kh) {               // low weight image
+            const uint32_t r = take();
+            if (leader) {
+              tc::mma4_bf16_ts(tD, tAh + kh * 32, ring_desc + r * kAtomDesc, idesc, kh);
+              tc::mma_commit(&tail->empty[r]);
+            }
+          }
+#pragma unroll
+          for (int kh = 0; kh < 2; ++kh) {               // middle
+            const uint32_t r = take();
+            if (leader) {
+              tc::mma4_bf16_ts(tD, tAm + kh * 32, ring_desc + r * kAtomDesc, idesc, 1u);
+              tc::mma4_bf16_ts(tD, tAh + kh * 32, ring_desc + r * kAtomDesc, idesc, 1u);
+              tc::mma_commit(&tail->empty[r]);
+            }
+          }
+          uint32_t rh[2];
+#pragma unroll
+          for (int kh = 0; kh < 2; ++kh) {               // high: the small products of both atoms first
+            rh[kh] = take();
+            if (leader) {
+              tc::mma4_bf16_ss(tD, lo_desc + kh * kAtomDesc, ring_desc + rh[kh] * kAtomDesc, idesc);
+              tc::mma4_bf16_ts(tD, tAm + kh * 32, ring_desc + rh[kh] * kAtomDesc, idesc, 1u);
+            }
+          }
+          if (leader) {
+#pragma unroll
+            for (int kh = 0; kh < 2; ++kh) {
+              tc::mma4_bf16_ts(tD, tAh + kh * 32, ring_desc + rh[kh] * kAtomDesc, idesc, 1u);
+              tc::mma_commit(&tail->empty[rh[kh]]);
+            }
+          }
+        }
+        if (leader) tc::mma_commit(&tail->bar_mma[s]);
+        __syncwarp();
+        tc3_wait(a, &tail->abort, &tail->bar_mma[s], mma_phase);
+        mma_phase ^= 1u;
+        __syncwarp();
+        tc::tc_fence_after();
+        tc::tc_fence_before();
+        tc3_arrive(3 + s);
+      }
+    }
+    // MMAs of a timed-out pass complete (bounded) before the tensor memory is freed
+    if (leader) tc::mma_commit(&tail->drain);
+    __syncwarp();
+    (void)tc::mbar_wait(&tail->drain, 0);
+    __syncwarp();
+  } else {
+    // ---- epilogue warps: rows 32 (warp % 4) + lane, columns 32 h .. 32 h + 31
+    const int h = warp >> 2;
+    const int rw = (warp & 3) * 32 + lane;                 // tile row / tensor-memory lane
+    const uint32_t tbase = tail->tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const bool deriv = a.R > 1;
+    bool secants = false;
+    for (int k = 1; k < a.R; ++k) secants |= kind_class(a.kinds[k]) == 2;
+
+    // The row of this thread in a tile, and its first-layer operand: inputs of primal rows,
+    // directions of the others (a one-hot entry, or a latent direction), 8 inputs per column part.
+    // load() reads the row's inputs (ahead of the last layer's accumulator wait, so that their
+    // latency is hidden), put() writes the operand once the slot is free.
+    auto load = [&](int64_t tile, float v[8], float v2[8]) {
+      const int64_t g0 = (tile * 4 + (warp & 3)) * U;
+      Tc3Row rs;
+      int kind = -1;
+      {
+        // point of the lane group's first row
+        const int64_t p0 = g0 < (int64_t)1 << 31 ? (int64_t)((uint32_t)g0 / (uint32_t)a.R) : g0 / a.R;
+        const int64_t row = U == 32 ? g0 + lane : lane == 0 ? p0 * a.R : g0 + lane - 1;
+        const int off = (int)(row - p0 * a.R);             // 0 .. R + 30
+        const int dp = off / a.R, k = off - dp * a.R;
+        rs.p = p0 + dp;
+        rs.cls = -1;
+        rs.psrc = lane;
+        rs.kidx = -1;
+        if (row < n_rows) {
+          kind = a.kinds[k];
+          rs.cls = kind_class(kind);
+          rs.kidx = (U != 32 && lane == 0) ? -1 : k;
+          rs.psrc = U == 32 ? lane - k : max(lane - k, 0);   // before the group's first row: lane 0's copy
+        }
+      }
+      const int d = a.d;
+      const float *vec = nullptr, *xp = nullptr;           // latent part, coordinates
+      int hot = -1;
+      if (rs.cls >= 0) {
+        RowInfo ri;
+        ri.p = rs.p;
+        int64_t xrow;
+        int li;
+        row_source(a, ri, xrow, li);
+        if (rs.cls == 0) {
+          vec = a.latents + (int64_t)li * a.r;
+          xp = a.X + xrow * d;
+        } else if (rs.cls == 1 && kind != KIND_JVP) {
+          hot = kind - 1;
+        } else {
+          vec = a.dirs + dir_offset(a, kind, li);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int i = 8 * h + j;
+        v[j] = (vec != nullptr && i >= d && i < K0) ? vec[i - d] : 0.f;
+        if (i == hot) v[j] = 1.f;
+      }
+      if (h == 0) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          if (j < d) {
+            const float range = a.norm[d + j];
+            if (xp != nullptr) v[j] = (xp[j] - a.norm[j]) / range;
+            if (j == hot) v[j] = 1.f / range;
+          }
+        }
+      }
+      if (K0 > 32) {                                       // inputs 32 .. 39 (d + r <= 40), column part 0
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int i = 32 + j;
+          v2[j] = (vec != nullptr && i < K0) ? vec[i - d] : 0.f;
+          if (i == hot) v2[j] = 1.f;
+        }
+      }
+      return rs;
+    };
+    auto put8 = [&](int s, int c, const float v[8]) {      // inputs 8 c .. 8 c + 7 of the slot's operand row
+      uint32_t wh[4], wm[4], wl[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) split3(v[2 * j], v[2 * j + 1], wh[j], wm[j], wl[j]);
+      __syncwarp();
+      tc::tmem_st4(tbase + s * 256 + 128 + 4 * c, wh);
+      tc::tmem_st4(tbase + s * 256 + 192 + 4 * c, wm);
+      *reinterpret_cast<uint4*>(lotile + s * kLayerBytes + tc::sw128_offset(rw, 8 * c, kW)) =
+          make_uint4(wl[0], wl[1], wl[2], wl[3]);
+    };
+    auto put = [&](int s, const float v[8], const float v2[8]) {
+      if (h < 2 * KS0) put8(s, h, v);
+      if (K0 > 32 && h < 2) {
+        const float zero[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        put8(s, 4 + h, h == 0 ? v2 : zero);
+      }
+    };
+    // the slot's operand is complete and its accumulator read: its issuer may go on
+    auto ready = [&](int s) {
+      tc::tmem_wait_st();
+      tc::fence_async_smem();
+      tc::tc_fence_before();
+      tc3_arrive(1 + s);
+    };
+
+    Tc3Row rows[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int64_t tile = (int64_t)blockIdx.x * NT + s;
+      if (blockIdx.x < n_iter && s < NT && tile < n_tiles) {
+        float v[8], v2[8];
+        rows[s] = load(tile, v, v2);
+        put(s, v, v2);
+        ready(s);
+      }
+    }
+    for (int64_t it = blockIdx.x; it < n_iter; it += gridDim.x) {
+      for (int l = -1; l < a.n_tc; ++l) {
+        const bool last = l == a.n_tc - 1;
+        const float* bl = l < 0 ? sb0 : sbh + l * kW;
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+          if (s >= NT || it * NT + s >= n_tiles) break;
+          const Tc3Row rs = rows[s];
+          const bool primal = rs.cls == 0;
+          // per-lane constants that make one expression of both row classes: below zero a primal row
+          // is e^z 1 - 1, a tangent row e^z zd + 0; the factor is (zd & keep) | one
+          const float neg_c = primal ? -1.0f : 0.0f, one_p = primal ? 1.0f : 0.0f;
+          const uint32_t keep = primal ? 0u : 0xffffffffu, one = __float_as_uint(one_p);
+          const uint32_t ts = tbase + s * 256;
+          uint8_t* lo_t = lotile + s * kLayerBytes;
+          float y[3] = {0.f, 0.f, 0.f};
+          // the slot's next tile: its inputs load while the last accumulator completes
+          float v[8], v2[8];
+          const int64_t next = it + gridDim.x;
+          const bool more = last && next < n_iter && next * NT + s < n_tiles;
+          if (more) rows[s] = load(next * NT + s, v, v2);
+          tc3_sync(3 + s);
+          tc::tc_fence_after();
+#pragma unroll 1
+          for (int c0 = 32 * h; c0 < 32 * h + 32; c0 += 16) {
+            float z[16];
+            tc::tmem_ld16(ts + c0, z);
+            // the bias of primal rows (a factor 0 on the others)
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) {
+              const float4 b4 = *reinterpret_cast<const float4*>(bl + c0 + i);
+              fma2(z[i], z[i + 1], b4.x, b4.y, one_p);
+              fma2(z[i + 2], z[i + 3], b4.z, b4.w, one_p);
+            }
+            if (a.act == 0) {
+              if (!deriv) {
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                  float x0 = z[i], x1 = z[i + 1];
+                  mul2(x0, x1, kLog2e);
+                  x0 = ex2_ftz(x0);
+                  x1 = ex2_ftz(x1);
+                  add2(x0, x1, -1.0f, -1.0f);
+                  z[i] = z[i] > 0.f ? z[i] : x0;
+                  z[i + 1] = z[i + 1] > 0.f ? z[i + 1] : x1;
+                }
+              } else if (!secants) {
+                // primal rows: z, or e^z - 1 below zero; tangent rows: zd, or e^z zd
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                  const float p0 = __shfl_sync(0xffffffffu, z[i], rs.psrc);
+                  const float p1 = __shfl_sync(0xffffffffu, z[i + 1], rs.psrc);
+                  float x0 = p0, x1 = p1;
+                  mul2(x0, x1, kLog2e);
+                  x0 = fmaf(ex2_ftz(x0), __uint_as_float((__float_as_uint(z[i]) & keep) | one), neg_c);
+                  x1 = fmaf(ex2_ftz(x1), __uint_as_float((__float_as_uint(z[i + 1]) & keep) | one), neg_c);
+                  z[i] = p0 > 0.f ? z[i] : x0;
+                  z[i + 1] = p1 > 0.f ? z[i + 1] : x1;
+                }
+              } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                  const float zp = __shfl_sync(0xffffffffu, z[i], rs.psrc);
+                  const float neg = fmaf(ex2_ftz(zp * kLog2e), primal ? 1.0f : z[i], neg_c);
+                  const float pt = zp > 0.f ? z[i] : neg;
+                  z[i] = rs.cls == 2 ? elu_secant(zp, z[i]) : pt;
+                }
+              }
+            }
+            if (last) {
+              // output layer fused into the last epilogue (FP32), partial over this part's columns
+#pragma unroll
+              for (int o = 0; o < 3; ++o) {
+                if (o >= a.d) break;
+                float q0 = 0.f, q1 = 0.f, q2 = 0.f, q3 = 0.f;   // short chains, added pairwise
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                  const float4 w4 = *reinterpret_cast<const float4*>(sWout + o * kW + c0 + i);
+                  q0 = fmaf(w4.x, z[i], q0);
+                  q1 = fmaf(w4.y, z[i + 1], q1);
+                  q2 = fmaf(w4.z, z[i + 2], q2);
+                  q3 = fmaf(w4.w, z[i + 3], q3);
+                }
+                y[o] += (q0 + q1) + (q2 + q3);
+              }
+            } else {
+              uint32_t wh[8], wm[8], wl[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) split3(z[2 * j], z[2 * j + 1], wh[j], wm[j], wl[j]);
+              tc::tmem_st8(ts + 128 + c0 / 2, wh);
+              tc::tmem_st8(ts + 192 + c0 / 2, wm);
+              *reinterpret_cast<uint4*>(lo_t + tc::sw128_offset(rw, c0, kW)) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+              *reinterpret_cast<uint4*>(lo_t + tc::sw128_offset(rw, c0 + 8, kW)) =
+                  make_uint4(wl[4], wl[5], wl[6], wl[7]);
+            }
+          }
+          if (!last) {
+            ready(s);
+            continue;
+          }
+          if (more) {
+            put(s, v, v2);
+            ready(s);
+          }
+          if (h > 0) {
+#pragma unroll
+            for (int o = 0; o < 3; ++o)
+              if (o < a.d) ypart[((h - 1) * 128 + rw) * 3 + o] = y[o];
+          }
+          tc3_epi_sync();
+          if (h == 0 && rs.kidx >= 0) {
+            float* o = a.out + ((int64_t)rs.kidx * a.n + rs.p) * a.d;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              if (i >= a.d) break;
+              float v = (y[i] + ypart[rw * 3 + i]) + (ypart[(128 + rw) * 3 + i] + ypart[(256 + rw) * 3 + i]);
+              if (primal) v += __ldg(&a.bout[i]);
+              o[i] = v * a.norm[3 * a.d + i] + (primal ? a.norm[2 * a.d + i] : 0.f);
+            }
+          }
+          tc3_epi_sync();   // ypart is free for the next tile
+        }
+      }
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_free<256 * NS>(tail->tmem);
+}
+
 // Transposed FP32 copies of the square layers for the CUDA-core path:
 // WT[l][k][f] = W[l][f][k].
 __global__ void decoder_transpose(const float* W, int n_layers, float* WT) {
@@ -1080,6 +1596,39 @@ __global__ void decoder_pack_w0(const float* W0, int d, int r, uint8_t* img) {
   }
 }
 
+// Weight stream of decoder_tc3: per layer its low, middle and high BF16 images (w = hi + mid + lo
+// exactly, each rounded to nearest), as atoms of 128 output rows x 64 K in the 128-byte swizzled
+// K-major layout: the first layer (K = d + r <= 40, zero-padded) one atom per image, the square
+// layers two.
+__global__ void decoder_pack3(const float* W0, int K0, const float* wsq, int n_tc, uint8_t* out) {
+  const int64_t total = (int64_t)(1 + 2 * n_tc) * kW * 64;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int blk = (int)(e / (kW * 64)), rem = (int)(e % (kW * 64));
+    const int row = rem / 64, k = rem % 64;
+    float w;
+    int64_t at;   // low atom, and the distance to the next image's
+    int step;
+    if (blk == 0) {
+      w = k < K0 ? W0[row * K0 + k] : 0.f;
+      at = 0;
+      step = 1;
+    } else {
+      const int l = (blk - 1) / 2, kh = (blk - 1) & 1;
+      w = wsq[((int64_t)l * kW + row) * kW + kh * 64 + k];
+      at = 3 + 6 * l + kh;
+      step = 2;
+    }
+    const __nv_bfloat16 hi = __float2bfloat16_rn(w);
+    const float r1 = w - __bfloat162float(hi);
+    const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+    uint8_t* o = out + at * kAtomBytes + tc::sw128_offset(row, k, kW);
+    *reinterpret_cast<__nv_bfloat16*>(o) = lo;
+    *reinterpret_cast<__nv_bfloat16*>(o + step * kAtomBytes) = mid;
+    *reinterpret_cast<__nv_bfloat16*>(o + 2 * step * kAtomBytes) = hi;
+  }
+}
+
 }  // namespace mpmrom
 
 using namespace mpmrom;
@@ -1097,6 +1646,12 @@ size_t dec_smem_bytes(bool split) {
 size_t dec_primal_smem_bytes() {
   return 1024 + kMaxTC * kLayerBytes + kLayerBytes / 2 + 2 * kLayerBytes +
          (2 * 128 * 3 + kW + kMaxTC * kW + 3 * kW) * sizeof(float) + sizeof(PrimSmemTail);
+}
+
+template <int NS>
+size_t dec_tc3_smem_bytes() {
+  return 1024 + kRing * kAtomBytes + NS * kLayerBytes + (3 * 128 * 3 + kW + kMaxTC * kW + 3 * kW) * sizeof(float) +
+         sizeof(Tc3Tail);
 }
 
 size_t dec_f32_smem_bytes() {
@@ -1118,6 +1673,9 @@ mpm_status refresh_derived_impl(mpm_decoder* dec, cudaStream_t s) {
   MPM_CUDA_TRY(cudaGetLastError());
   decoder_transpose<<<16, 256, 0, s>>>(dec->wsq, dec->n_tc, dec->wsqT);
   MPM_CUDA_TRY(cudaGetLastError());
+  decoder_pack3<<<std::max(1, std::min(dec->n_sm * 4, (1 + 2 * dec->n_tc) * 32)), 256, 0, s>>>(
+      dec->params + dec->w_off[0], dec->d + dec->r, dec->wsq, dec->n_tc, dec->wstream);
+  MPM_CUDA_TRY(cudaGetLastError());
   if (dec->w0img) {
     decoder_pack_w0<<<16, 256, 0, s>>>(dec->params + dec->w_off[0], dec->d, dec->r, dec->w0img);
     MPM_CUDA_TRY(cudaGetLastError());
@@ -1137,7 +1695,7 @@ void decoder_shape(const mpm_decoder* dec, int* d, int* r) {
 // Internal launcher for on-device point sets (used by the reduced-order step).
 mpm_status decoder_launch_dev(const mpm_decoder* dec, const float* X, const int32_t* idx, const int32_t* n_dev,
                               int n_rep, int64_t capacity, const float* latents, const float* dirs,
-                              const int* kinds, int R, float* out, cudaStream_t s);
+                              const int* kinds, int R, float* out, cudaStream_t s, bool cuda_cores);
 }
 
 extern "C" {
@@ -1175,16 +1733,33 @@ mpm_status decoder_create(const decoder_desc* desc, mpm_decoder** out) {
   cudaDeviceGetAttribute(&dec->n_sm, cudaDevAttrMultiProcessorCount, dev);
   dec->smem = dec_smem_bytes(false);
   dec->smem_split = dec_smem_bytes(true);
-  cudaError_t e = cudaMalloc((void**)&dec->params, sizeof(float) * dec->n_params);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&dec->norm, sizeof(float) * 4 * dec->d);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&dec->status, sizeof(uint32_t));
-  if (e == cudaSuccess && dec->n_tc > 0) {
-    e = cudaMalloc((void**)&dec->wsq, sizeof(float) * dec->n_tc * kW * kW);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&dec->bsq, sizeof(float) * dec->n_tc * kW);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&dec->wimg, (size_t)dec->n_tc * kLayerBytes);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&dec->wimg_lo, (size_t)dec->n_tc * kLayerBytes);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&dec->wsqT, sizeof(float) * dec->n_tc * kW * kW);
-    if (e == cudaSuccess && kTcLat + dec->r <= 32) e = cudaMalloc((void**)&dec->w0img, (size_t)kLayerBytes / 2);
+  // one allocation for every buffer of the decoder (each cudaMalloc costs tens of microseconds)
+  size_t bytes = 0;
+  auto place = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 1023) / 1024 * 1024;
+    return at;
+  };
+  const size_t sq = sizeof(float) * dec->n_tc * kW * kW, img = (size_t)dec->n_tc * kLayerBytes;
+  const size_t o_params = place(sizeof(float) * dec->n_params), o_norm = place(sizeof(float) * 4 * dec->d);
+  const size_t o_status = place(sizeof(uint32_t));
+  const size_t o_wsq = place(sq), o_bsq = place(sizeof(float) * dec->n_tc * kW), o_wsqT = place(sq);
+  const size_t o_wimg = place(img), o_wimg_lo = place(img), o_w0img = place(kLayerBytes / 2);
+  const size_t o_wstream = place(dec->n_tc > 0 ? (size_t)(3 + 6 * dec->n_tc) * kAtomBytes : 0);
+  cudaError_t e = cudaMalloc((void**)&dec->pool, bytes);
+  if (e == cudaSuccess) {
+    dec->params = (float*)(dec->pool + o_params);
+    dec->norm = (float*)(dec->pool + o_norm);
+    dec->status = (uint32_t*)(dec->pool + o_status);
+    if (dec->n_tc > 0) {
+      dec->wsq = (float*)(dec->pool + o_wsq);
+      dec->bsq = (float*)(dec->pool + o_bsq);
+      dec->wsqT = (float*)(dec->pool + o_wsqT);
+      dec->wimg = dec->pool + o_wimg;
+      dec->wimg_lo = dec->pool + o_wimg_lo;
+      dec->wstream = dec->pool + o_wstream;
+      if (kTcLat + dec->r <= 32) dec->w0img = dec->pool + o_w0img;
+    }
   }
   if (e == cudaSuccess) e = cudaMemset(dec->params, 0, sizeof(float) * dec->n_params);
   if (e == cudaSuccess) e = cudaMemset(dec->status, 0, sizeof(uint32_t));
@@ -1195,6 +1770,10 @@ mpm_status decoder_create(const decoder_desc* desc, mpm_decoder** out) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(decoder_tc_primal, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)dec_primal_smem_bytes());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(decoder_tc3<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec_tc3_smem_bytes<1>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(decoder_tc3<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec_tc3_smem_bytes<2>());
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(decoder_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec_f32_smem_bytes());
   if (e == cudaSuccess)
@@ -1209,15 +1788,7 @@ mpm_status decoder_create(const decoder_desc* desc, mpm_decoder** out) {
 
 void decoder_destroy(mpm_decoder* dec) {
   if (!dec) return;
-  cudaFree(dec->params);
-  cudaFree(dec->norm);
-  cudaFree(dec->wsq);
-  cudaFree(dec->bsq);
-  cudaFree(dec->wimg);
-  cudaFree(dec->wimg_lo);
-  cudaFree(dec->wsqT);
-  cudaFree(dec->w0img);
-  cudaFree(dec->status);
+  cudaFree(dec->pool);
   delete dec;
 }
 
@@ -1256,7 +1827,7 @@ mpm_status decoder_get_params(const mpm_decoder* dec, float* params, float* norm
 static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const int32_t* lat_idx,
                                  const float* latents, const float* dirs, const int32_t* kinds, int R, int64_t n,
                                  float* out, const int32_t* idx, const int32_t* n_dev, int n_rep, cudaStream_t s,
-                                 const DecArgs* extra = nullptr);
+                                 const DecArgs* extra = nullptr, bool cuda_cores = false);
 
 mpm_status decoder_eval(const mpm_decoder* dec, const float* X, const int32_t* lat_idx, const float* latents,
                         const float* dirs, const int32_t* kinds, int R, int64_t n, float* out, void* stream) {
@@ -1270,7 +1841,7 @@ mpm_status decoder_eval(const mpm_decoder* dec, const float* X, const int32_t* l
 static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const int32_t* lat_idx,
                                  const float* latents, const float* dirs, const int32_t* kinds, int R, int64_t n,
                                  float* out, const int32_t* idx, const int32_t* n_dev, int n_rep, cudaStream_t s,
-                                 const DecArgs* extra) {
+                                 const DecArgs* extra, bool cuda_cores) {
   MPM_CHECK_ARG(R >= 1 && R <= kMaxR && R <= 128, "R must be in [1, 64]");
   MPM_CHECK_ARG(X && latents && out, "null argument");
   DecArgs a{};
@@ -1290,6 +1861,7 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
   a.wimg_lo = dec->wimg_lo;
   a.w0img = dec->w0img;
   a.wsq = dec->wsq;
+  a.wstream = dec->wstream;
   a.wsqT = dec->wsqT;
   a.X = X;
   a.lat = lat_idx;
@@ -1347,10 +1919,30 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
   // the tensor-core kernel's input layout holds r <= 36 latents (decoder_create allows d + r <= 40):
   // larger latents take the FP32 kernel
   const bool f32_path = (dec->fp32 == 1 || dec->r > 40 - kTcLat) && !a.dstore;
+  // FP32 calls run on the tensor cores (decoder_tc3) but for mixed rows (their partner rows are not in
+  // the row's warp), for callers that keep decoder_f32's rounding, and for a lone caller's small calls
+  // with secant rows (256 samples x 12 or 18 rows: 32 us against 40 us; without secants, 256 x 17
+  // rows, 31 us against 27 us the other way; 4096 x 4 rows 98 against 29 us)
+  bool secants = false;
+  for (int k = 0; k < R; ++k) secants |= kind_class(kinds[k]) == 2;
+  const bool tc3 = f32_path && !has_mixed && !cuda_cores &&
+                   !(secants && dec->concurrency == 1 && n * R <= 31 * (int64_t)dec->n_sm);
   if (dec->n_tc == 0) {
     int64_t rows = n * R;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((rows + 127) / 128, dec->n_sm * 8));
     decoder_simt<<<blocks, 128, 0, s>>>(a);
+  } else if (tc3) {
+    // rows in (point, kind) order, 32 (whole points) or 31 per lane group, four lane groups per
+    // tile; one tile per CTA while every tile has an SM of its own (of this caller's share), else two
+    a.tc3_U = 32 % R == 0 ? 32 : 31;
+    const int64_t tiles = (n * R + 4 * a.tc3_U - 1) / (4 * a.tc3_U);
+    const int64_t share = std::max(1, dec->n_sm / std::max(1, dec->concurrency));
+    if (tiles <= share) {
+      decoder_tc3<1><<<(int)tiles, tc3_threads<1>(), dec_tc3_smem_bytes<1>(), s>>>(a);
+    } else {
+      const int blocks = (int)std::min<int64_t>((tiles + 1) / 2, dec->n_sm);
+      decoder_tc3<2><<<blocks, tc3_threads<2>(), dec_tc3_smem_bytes<2>(), s>>>(a);
+    }
   } else if (f32_path) {
     MPM_CHECK_ARG(R <= kF32Rows, "the FP32 path takes at most 64 row kinds");
     int64_t tiles;
@@ -1411,9 +2003,10 @@ mpm_status decoder_launch_train(const mpm_decoder* dec, const float* X, const fl
 
 mpm_status decoder_launch_dev(const mpm_decoder* dec, const float* X, const int32_t* idx, const int32_t* n_dev,
                               int n_rep, int64_t capacity, const float* latents, const float* dirs,
-                              const int* kinds, int R, float* out, cudaStream_t s) {
+                              const int* kinds, int R, float* out, cudaStream_t s, bool cuda_cores) {
   if (capacity <= 0) return MPM_OK;
-  return decoder_launch(dec, X, nullptr, latents, dirs, kinds, R, capacity, out, idx, n_dev, n_rep, s);
+  return decoder_launch(dec, X, nullptr, latents, dirs, kinds, R, capacity, out, idx, n_dev, n_rep, s, nullptr,
+                        cuda_cores);
 }
 }  // namespace mpmrom
 

@@ -31,6 +31,8 @@ struct DecArgs {
   // padded layout): rows = output features, hi at K 0 .. 31 and lo at K 32 .. 63 of one
   // 128-byte swizzled row; null when the first layer runs on the CUDA cores
   const uint8_t* w0img;
+  // every layer's weights as three BF16 images (decoder_pack3) in the order decoder_tc3 reads them
+  const uint8_t* wstream;
   const float* wsq;   // (n_tc, W, W) FP32 square-layer weights, (out, in) row-major
   const float* wsqT;  // (n_tc, W, W) the same transposed, (in, out) row-major
   const float* X;
@@ -57,6 +59,8 @@ struct DecArgs {
   int lat_per_point;
   // FP32 path: useful rows per packed tile (0: point-aligned tiles of Pt points)
   int f32_U;
+  // decoder_tc3: rows per lane group (32: whole points; 31: packed, lane 0 a recomputed primal)
+  int tc3_U;
   // direction blocks per latent row in `dirs` (KIND_SECANT_DIR rows; 1 otherwise)
   int n_dirs;
   // training: per hidden layer l, stored feature-major [l][feature][row] (row =
@@ -124,7 +128,7 @@ struct RowInfo {
   int ja, jb;    // mixed rows: kind indices of the paired JVP and tangent rows
 };
 
-__device__ __forceinline__ int kind_class(int kind) {
+__host__ __device__ __forceinline__ int kind_class(int kind) {
   if (kind == KIND_PRIMAL) return 0;
   if (kind == KIND_SECANT || kind >= KIND_SECANT_DIR) return 2;
   return kind > KIND_MIXED ? 3 : 1;
@@ -343,6 +347,7 @@ struct mpm_decoder {
   int n_tc = 0;
   int64_t n_params = 0;
   std::vector<int64_t> w_off, b_off;  // per linear layer offsets into params
+  uint8_t* pool = nullptr;            // the one allocation that holds the buffers below
   float* params = nullptr;            // FP32 master copy
   float* norm = nullptr;
   float* wsq = nullptr;               // square-layer weights gathered contiguously (n_tc, W, W)
@@ -351,6 +356,7 @@ struct mpm_decoder {
   uint8_t* wimg = nullptr;            // BF16 swizzled images
   uint8_t* wimg_lo = nullptr;         // residual images bf16(w - bf16(w)) for the split-BF16 path
   uint8_t* w0img = nullptr;           // first-layer split image (16 KB) when kTcLat + r <= 32
+  uint8_t* wstream = nullptr;         // three-image weight stream of decoder_tc3
   uint32_t* status = nullptr;
   int n_sm = 0;
   size_t smem = 0;

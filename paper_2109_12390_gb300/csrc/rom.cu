@@ -56,7 +56,7 @@ struct mpm_decoder;
 namespace mpmrom {
 mpm_status decoder_launch_dev(const mpm_decoder* dec, const float* X, const int32_t* idx, const int32_t* n_dev,
                               int n_rep, int64_t capacity, const float* latents, const float* dirs,
-                              const int* kinds, int R, float* out, cudaStream_t s);
+                              const int* kinds, int R, float* out, cudaStream_t s, bool cuda_cores = false);
 void decoder_shape(const mpm_decoder* dec, int* d, int* r);
 }
 
@@ -1613,10 +1613,16 @@ mpm_status rom_launch_lagrangian(rom_ctx* c, const int* kq, int Rq, bool affine,
   const int d = c->d;
   const int M = c->cfg.material, T = c->cfg.transfer;
   mpm_status st = MPM_OK;
+  // with the reference gradient the strain is the small difference of two decoded gradients, and FP32
+  // rounding of either is about 1e-4 of it: the decodes of gradients keep the rounding of decoder_f32
+  // (on the tensor cores, at the same distance from 64 bits, latent velocities of the 4096-particle
+  // block moved by up to 4e-5; without the reference gradient the two differ by 4e-6)
+  const bool cuda_cores = c->cfg.f_reference != 0;
   if (c->merged) {
     // 1 + 3. one decode of every particle with the quadrature rows: positions (x_all is its
     // primal block) and F, v for whichever particles the neighbourhood selects
-    st = decoder_launch_dev(c->dec, c->X, nullptr, c->nP_all, 1, c->P, c->sv.xh32, c->sv.vh32, kq, Rq, c->outQ, s);
+    st = decoder_launch_dev(c->dec, c->X, nullptr, c->nP_all, 1, c->P, c->sv.xh32, c->sv.vh32, kq, Rq, c->outQ, s,
+                            cuda_cores);
     if (st != MPM_OK) return st;
   } else {
     // 1. decode all particles at xhat_n
@@ -1643,7 +1649,7 @@ mpm_status rom_launch_lagrangian(rom_ctx* c, const int* kq, int Rq, bool affine,
   if (!c->merged) {
     // 3. F and v at the quadrature points Q
     st = decoder_launch_dev(c->dec, c->X, c->qlist, c->counts + 1, 1, c->P, c->sv.xh32, c->sv.vh32, kq, Rq, c->outQ,
-                            s);
+                            s, cuda_cores);
     if (st != MPM_OK) return st;
   }
   // 4. local P2G onto I
@@ -2395,7 +2401,8 @@ mpm_status rom_set_reference(rom_ctx* c, const double* xhat_ref, void* stream) {
   std::vector<float> h32(h.begin(), h.end());
   MPM_CUDA_TRY(cudaMemcpyAsync(c->xref32, h32.data(), sizeof(float) * r, cudaMemcpyHostToDevice, s));
   int kr[4] = {0, 1, 2, 3};
-  mpm_status st = decoder_launch_dev(c->dec, c->X, nullptr, c->nP_all, 1, P, c->xref32, nullptr, kr, d + 1, c->outQ, s);
+  mpm_status st = decoder_launch_dev(c->dec, c->X, nullptr, c->nP_all, 1, P, c->xref32, nullptr, kr, d + 1, c->outQ, s,
+                                     true);   // as the step's gradients (rom_launch_lagrangian)
   if (st != MPM_OK) return st;
   const int b = std::max(1, std::min(ceil_div(P, 256), c->n_sm * 4));
   if (d == 2)

@@ -26,6 +26,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
                : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t phase) {
   uint32_t ok;
   asm volatile(
@@ -41,6 +44,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, uint32_
   for (uint32_t i = 0; i < max_tries; ++i)
     if (mbar_try_wait(bar, phase)) return true;
   return false;
+}
+
+// True in one lane of the (converged) warp, the same one on every call.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+  return ok != 0;
 }
 
 // ------------------------------------------------------ bulk async copy (TMA)
@@ -109,6 +119,57 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
       : "memory");
 }
 
+// Low and high word of smem_desc_sw128 (the high word does not depend on the address; advancing by
+// 16 K entries adds 2 to the low word).
+__device__ __forceinline__ uint32_t smem_desc_sw128_lo(uint32_t saddr) {
+  return ((saddr & 0x3FFFFu) >> 4) | ((16u >> 4) << 16);
+}
+constexpr uint32_t kDescSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+
+// Four K steps of 16 (one 64-wide atom) of D (+)= A B^T in one statement, so that the issuing thread
+// prepares its descriptors once per atom: A in tensor memory, or A in shared memory.
+__device__ __forceinline__ void mma4_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_lo, uint32_t idesc,
+                                             uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 b<4>;\n .reg .b32 l<4>, a<4>;\n"
+      " setp.ne.b32 p, %4, 0;\n setp.eq.b32 q, 0, 0;\n"
+      " add.u32 l1, %2, 2;\n add.u32 l2, %2, 4;\n add.u32 l3, %2, 6;\n"
+      " add.u32 a1, %1, 8;\n add.u32 a2, %1, 16;\n add.u32 a3, %1, 24;\n"
+      " mov.b64 b0, {%2, %5};\n mov.b64 b1, {l1, %5};\n mov.b64 b2, {l2, %5};\n mov.b64 b3, {l3, %5};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b0, %3, p;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, q;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, q;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, q;\n}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(kDescSw128Hi)
+      : "memory");
+}
+__device__ __forceinline__ void mma4_bf16_ss(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
+  asm volatile(
+      "{\n .reg .pred q;\n .reg .b64 a<4>, b<4>;\n .reg .b32 l<4>, m<4>;\n"
+      " setp.eq.b32 q, 0, 0;\n"
+      " add.u32 l1, %2, 2;\n add.u32 l2, %2, 4;\n add.u32 l3, %2, 6;\n"
+      " add.u32 m1, %1, 2;\n add.u32 m2, %1, 4;\n add.u32 m3, %1, 6;\n"
+      " mov.b64 b0, {%2, %4};\n mov.b64 b1, {l1, %4};\n mov.b64 b2, {l2, %4};\n mov.b64 b3, {l3, %4};\n"
+      " mov.b64 a0, {%1, %4};\n mov.b64 a1, {m1, %4};\n mov.b64 a2, {m2, %4};\n mov.b64 a3, {m3, %4};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a0, b0, %3, q;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, q;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, q;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, q;\n}\n" ::"r"(tmem_d),
+      "r"(a_lo), "r"(b_lo), "r"(idesc), "n"(kDescSw128Hi)
+      : "memory");
+}
+
+// D[tmem] (+)= A[tmem] * B[smem]^T: A row i sits in tensor-memory lane i, two consecutive BF16 K
+// entries per 32-bit column (8 columns per K step of 16).
+__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
 // Arrives on `bar` once all previously issued tcgen05 ops of this thread completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
@@ -131,6 +192,31 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+
+// 32 lanes x 16 columns, load and wait in one statement (the registers stay where the load put them).
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+      : "r"(taddr)
+      : "memory");
+}
+
+// 32 lanes x 8 (4) columns of 32-bit stored by a warp: thread i writes lane (base + i).  The
+// stores are visible to later tensor-core reads after tmem_wait_st and a fenced barrier.
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t r[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t r[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Byte offset of element (row, k) of a K-major BF16 tile with 128-byte
 // swizzle: K split into 64-element atoms (each `rows` x 128 B), 16-byte
