@@ -504,198 +504,6 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
 }
 
 // --------------------------------------------------------------------------
-// Tensor-core decoder for calls of primal rows only (one row kind), inputs of at most 32
-// entries in the padded layout, BF16 operands: two 128-row tiles in flight per CTA.  512
-// threads in two groups of eight warps; each group runs decoder_tc's tile loop (split-BF16 first
-// layer, square layers, fused output layer) on its own operand tile, tensor-memory columns, MMA
-// barrier and named barrier, so that one group's epilogue overlaps the other group's MMAs.  The
-// weights and the first layer's split image are resident once per CTA.  Same arithmetic, in the
-// same order, as decoder_tc<false>.
-// --------------------------------------------------------------------------
-constexpr int kPrimThreads = 512;
-
-struct __align__(8) PrimSmemTail {
-  uint64_t bar_w;
-  uint64_t bar_mma[2];
-  uint32_t tmem;
-  int abort[2];   // per group: set before a group barrier, read after it
-};
-
-__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory"); }
-
-__global__ void __launch_bounds__(kPrimThreads, 1) decoder_tc_primal(DecArgs a) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* wsm = smem;                                   // kMaxTC x 32 KB square layers
-  uint8_t* w0s = smem + kMaxTC * kLayerBytes;            // 16 KB first-layer split image
-  uint8_t* atiles = w0s + kLayerBytes / 2;               // 2 x 32 KB operand tiles, one per group
-  float* ypart = (float*)(atiles + 2 * kLayerBytes);     // [2 groups][128 rows][3]
-  float* sb0 = ypart + 2 * 128 * 3;                      // [128]
-  float* sbh = sb0 + kW;                                 // [kMaxTC][128]
-  float* sWout = sbh + kMaxTC * kW;                      // [3][128]
-  PrimSmemTail* tail = (PrimSmemTail*)(sWout + 3 * kW);
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int g = warp >> 3, tg = t & 255;                 // group, thread within the group
-  const int rw = (warp & 3) * 32 + lane;                 // tile row / tensor-memory lane
-  const int h = (warp >> 2) & 1;                         // column half
-  uint8_t* atile = atiles + g * kLayerBytes;
-  float* yp = ypart + g * 128 * 3;
-
-  if (t == 0) {
-    tc::mbar_init(&tail->bar_w, 1);
-    tc::mbar_init(&tail->bar_mma[0], 1);
-    tc::mbar_init(&tail->bar_mma[1], 1);
-    tail->abort[0] = 0;
-    tail->abort[1] = 0;
-    tc::fence_mbar_init();
-  }
-  if (warp == 0) tc::tmem_alloc<2 * kW>(&tail->tmem);
-  tc::tc_fence_before();
-  __syncthreads();
-  tc::tc_fence_after();
-  const uint32_t tmem = tail->tmem + (uint32_t)(g * kW);   // this group's 128 columns
-
-  for (int e = t; e < kW; e += kPrimThreads) sb0[e] = a.b0[e];
-  for (int e = t; e < a.n_tc * kW; e += kPrimThreads) sbh[e] = a.bh[e];
-  for (int e = t; e < a.d * kW; e += kPrimThreads) sWout[e] = a.Wout[e];
-  if (t == 0) {
-    tc::mbar_expect_tx(&tail->bar_w, (uint32_t)(a.n_tc * kLayerBytes + kLayerBytes / 2));
-    for (int l = 0; l < a.n_tc; ++l)
-      tc::bulk_g2s(wsm + l * kLayerBytes, a.wimg + (size_t)l * kLayerBytes, kLayerBytes, &tail->bar_w);
-    tc::bulk_g2s(w0s, a.w0img, kLayerBytes / 2, &tail->bar_w);
-  }
-  if (!tc::mbar_wait(&tail->bar_w, 0)) {
-    raise_status(a.status, STATUS_TIMEOUT);
-    tail->abort[0] = 1;
-    tail->abort[1] = 1;
-  }
-  __syncthreads();
-
-  constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW);
-  uint32_t mma_phase = 0;
-  const int64_t n_pts = dec_count(a);
-  const int64_t n_tiles = (n_pts + 127) / 128;
-  for (int64_t tile = 2 * (int64_t)blockIdx.x + g; tile < n_tiles && !tail->abort[g]; tile += 2 * (int64_t)gridDim.x) {
-    const int64_t first = tile * 128;
-    const RowInfo ri = row_info(a, rw, first, n_pts);
-    {
-      float in[40], dir[40];
-      if (ri.cls >= 0) row_inputs_tc(a, ri, in, dir);
-      // the first layer's operand row: half 0 stores the high parts at columns 0 .. 31, half 1
-      // the low parts at 32 .. 63; zero for rows past the end
-#pragma unroll
-      for (int c0 = 0; c0 < 32; c0 += 8) {
-        float p[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float v = ri.cls == 0 ? in[c0 + j] : 0.f;
-          const float hi = __bfloat162float(__float2bfloat16_rn(v));
-          p[j] = h == 0 ? hi : v - hi;
-        }
-        store_bf16x8(atile, rw, 32 * h + c0, p);
-      }
-    }
-    float y[3] = {0.f, 0.f, 0.f};
-    for (int l = -1; l < a.n_tc; ++l) {
-      tc::fence_async_smem();
-      tc::tc_fence_before();
-      group_sync(g);
-      if (tg == 0) {
-        tc::tc_fence_after();
-        const uint32_t a_base = tc::smem_addr(atile);
-        if (l < 0) {
-          const uint32_t b_base = tc::smem_addr(w0s);
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            const uint32_t hi = (uint32_t)(k * 32), lo = (uint32_t)(64 + k * 32);
-            tc::mma_bf16(tmem, tc::smem_desc_sw128(a_base + hi), tc::smem_desc_sw128(b_base + hi), idesc,
-                         k > 0 ? 1u : 0u);
-            tc::mma_bf16(tmem, tc::smem_desc_sw128(a_base + hi), tc::smem_desc_sw128(b_base + lo), idesc, 1u);
-            tc::mma_bf16(tmem, tc::smem_desc_sw128(a_base + lo), tc::smem_desc_sw128(b_base + hi), idesc, 1u);
-          }
-        } else {
-          const uint32_t b_base = tc::smem_addr(wsm + l * kLayerBytes);
-#pragma unroll
-          for (int k = 0; k < kW / 16; ++k) {
-            const uint32_t koff = (uint32_t)((k >> 2) * (kW * 128) + (k & 3) * 32);
-            tc::mma_bf16(tmem, tc::smem_desc_sw128(a_base + koff), tc::smem_desc_sw128(b_base + koff), idesc,
-                         k > 0 ? 1u : 0u);
-          }
-        }
-        tc::mma_commit(&tail->bar_mma[g]);
-      }
-      if (!tc::mbar_wait(&tail->bar_mma[g], mma_phase)) {
-        raise_status(a.status, STATUS_TIMEOUT);
-        tail->abort[g] = 1;
-      }
-      mma_phase ^= 1u;
-      tc::tc_fence_after();
-      group_sync(g);
-      if (tail->abort[g]) break;
-      const bool last = (l == a.n_tc - 1);
-      const float* bl = l < 0 ? sb0 : sbh + l * kW;
-      for (int i2 = 0; i2 < 2; ++i2) {
-        const int ch = 2 * h + i2;
-        float acc[32];
-        tc::tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch * 32, acc);
-        if (ri.cls == 0) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            const float4 b4 = *reinterpret_cast<const float4*>(bl + ch * 32 + i);
-            acc[i] += b4.x;
-            acc[i + 1] += b4.y;
-            acc[i + 2] += b4.z;
-            acc[i + 3] += b4.w;
-          }
-          if (a.act == 0) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) acc[i] = elu_bf16_input(acc[i]);
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-        }
-        if (last) {
-#pragma unroll
-          for (int o = 0; o < 3; ++o) {   // compile-time bound: y stays in registers
-            if (o >= a.d) break;
-            float sacc = 0.f;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) sacc = fmaf(sWout[o * kW + ch * 32 + i], acc[i], sacc);
-            y[o] += sacc;
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; j += 8) store_bf16x8(atile, rw, ch * 32 + j, acc + j);
-        }
-      }
-      tc::tc_fence_before();
-    }
-    if (tail->abort[g]) break;
-    // combine the two column halves of the output layer
-    if (h == 1) {
-#pragma unroll
-      for (int o = 0; o < 3; ++o)
-        if (o < a.d) yp[rw * 3 + o] = y[o];
-    }
-    group_sync(g);
-    if (h == 0 && ri.cls >= 0) {
-      float* o = a.out + ri.p * a.d;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        if (i >= a.d) break;
-        const float v = y[i] + yp[rw * 3 + i] + __ldg(&a.bout[i]);
-        o[i] = v * a.norm[3 * a.d + i] + a.norm[2 * a.d + i];
-      }
-    }
-    group_sync(g);
-  }
-  __syncthreads();
-  tc::tc_fence_after();
-  if (warp == 0) tc::tmem_free<2 * kW>(tail->tmem);
-}
-
-// --------------------------------------------------------------------------
 // FP32 decoder on the CUDA cores, for calls whose rows are too few to keep the
 // tensor cores busy and whose results need FP32 accuracy (the reduced step's
 // positions and gradients).  Same row kinds as decoder_tc; one persistent CTA
@@ -1039,14 +847,14 @@ __global__ void __launch_bounds__(kF32Threads, 1) decoder_f32(DecArgs a) {
 // accumulated in FP32 in that order (small terms first, so that the accumulator holds its final
 // magnitude for the eight K steps of Ah Wh only); the dropped products are below 2^-23 of each term
 // with signs of their own.  All layers but the output layer (N = d, FP32 on the CUDA cores) run
-// this way, the first one with K = d + r padded to a multiple of 16.
+// this way, the first one with its inputs padded (coordinates to 4, all to a multiple of 16).
 //
 // A tile is 128 rows: four lane groups of 32 rows, each owned by four warps (32 columns apiece).
 // Rows are taken in (point, kind) order, so that a derivative row finds its point's primal
 // pre-activation in another lane of its warp (one shuffle per feature; no exchange through shared
 // memory and no block barrier):
-//   tc3_U = 32   32 % R == 0: a lane group holds whole points;
-//   tc3_U = 31   any R: 31 consecutive rows, lane 0 recomputing the primal row of the first one's
+//   pipe_U = 32   32 % R == 0: a lane group holds whole points;
+//   pipe_U = 31   any R: 31 consecutive rows, lane 0 recomputing the primal row of the first one's
 //                point (not written out).
 // NS tile slots per CTA: the sixteen epilogue warps take the slots in turn, so that one slot's
 // epilogue overlaps the other's MMAs (NS = 1: calls of at most one tile per SM).  The A operand's
@@ -1055,17 +863,18 @@ __global__ void __launch_bounds__(kF32Threads, 1) decoder_f32(DecArgs a) {
 // (atoms of 128 rows x 64 K, 16 KB) through a ring of kRing slots with bulk copies, one warp per
 // tile slot issues its MMAs.  A ring slot is refilled once both tile slots' MMAs on it completed.
 // What bounds it: per tile and layer the tensor core takes 48 MMAs (about 65 cycles each), the sixteen
-// epilogue warps about 3.8k cycles (21 instructions per element, 2.2 of 4 issue slots), the two
-// overlapped.  262,144 points x 4 rows, r = 16: 0.71 ms (decoder_f32: 5.07 ms), distance from 64 bits
-// 4e-8 .. 7e-8 (6.5e-8); 256 points x 17 rows: 27 us (31 us).
+// epilogue warps about 3.2k cycles (18 instructions per element, 2.2 of 4 issue slots), the two
+// overlapped.  262,144 points x 4 rows, r = 16: 0.63 ms (decoder_f32: 5.07 ms), distance from 64 bits
+// 4e-8 .. 7e-8 (6.5e-8); 256 points x 17 rows: 24 us (31 us); 20,000 points x 12 rows with secants:
+// 0.34 ms (1.36 ms).
 // After a wait that ran out nothing waits on the copies or MMAs any more: the pass runs to its end
 // (in bounds, its results void) with the TIMEOUT status raised.
 // --------------------------------------------------------------------------
-constexpr int kTc3Epi = 512;              // epilogue threads
+constexpr int kEpiThreads = 512;              // epilogue threads
 constexpr int kAtomBytes = kW * 128;      // 128 rows x 64 BF16
 constexpr int kRing = 9;
 template <int NS>
-constexpr int tc3_threads() { return kTc3Epi + 32 + 32 * NS; }
+constexpr int tc3_threads() { return kEpiThreads + 32 + 32 * NS; }
 
 struct __align__(8) Tc3Tail {
   uint64_t full[kRing];
@@ -1077,7 +886,7 @@ struct __align__(8) Tc3Tail {
 };
 
 // Bounded wait; after a timeout anywhere in the CTA no further waits are made.
-__device__ __forceinline__ void tc3_wait(const DecArgs& a, int* abort, uint64_t* bar, uint32_t phase) {
+__device__ __forceinline__ void pipe_wait(const DecArgs& a, int* abort, uint64_t* bar, uint32_t phase) {
   if (*(volatile int*)abort) return;
   if (!tc::mbar_wait(bar, phase)) {
     raise_status(a.status, STATUS_TIMEOUT);
@@ -1088,14 +897,17 @@ __device__ __forceinline__ void tc3_wait(const DecArgs& a, int* abort, uint64_t*
 // Barriers 1 + s: the epilogue warps arrive when slot s's next operand is complete (and its
 // accumulator read), the slot's issuer warp waits.  Barriers 3 + s: the issuer arrives when the
 // accumulator is complete, the epilogue warps wait (blocked, where polling the MMA barrier would
-// take issue slots).  Barrier 5: the epilogue warps among themselves.
-__device__ __forceinline__ void tc3_arrive(int id) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kTc3Epi + 32) : "memory");
+// take issue slots).  Barrier 5: the column parts' output sums are in shared memory.
+__device__ __forceinline__ void pipe_arrive(int id) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kEpiThreads + 32) : "memory");
 }
-__device__ __forceinline__ void tc3_sync(int id) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kTc3Epi + 32) : "memory");
+__device__ __forceinline__ void pipe_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kEpiThreads + 32) : "memory");
 }
-__device__ __forceinline__ void tc3_epi_sync() { asm volatile("bar.sync 5, %0;" ::"n"(kTc3Epi) : "memory"); }
+__device__ __forceinline__ void pipe_combine(int part) {
+  if (part == 3) asm volatile("bar.sync 5, %0;" ::"n"(kEpiThreads) : "memory");
+  else asm volatile("bar.arrive 5, %0;" ::"n"(kEpiThreads) : "memory");
+}
 
 // 2^x on the special-function unit, results below the normal range flushed to zero
 __device__ __forceinline__ float ex2_ftz(float x) {
@@ -1122,6 +934,9 @@ __device__ __forceinline__ void fma2(float& a0, float& a1, float b0, float b1, f
       : "+f"(a0), "+f"(a1)
       : "f"(b0), "f"(b1), "f"(c));
 }
+// What the rows of a call need of their activations (a template parameter: one variant's code per
+// kernel keeps the epilogue loop small)
+enum { PIPE_PRIMAL = 0, PIPE_TANGENT = 1, PIPE_SECANT = 2, PIPE_IDENTITY = 3 };
 constexpr float kLog2e = 1.4426950408889634f;   // __expf(z) is 2^(z kLog2e)
 
 // hi, mid and lo words (two BF16 values each, first value in the low half) of an FP32 pair: each
@@ -1138,13 +953,200 @@ __device__ __forceinline__ void split3(float v0, float v1, uint32_t& hi, uint32_
   lo = __byte_perm(__float_as_uint(v0), __float_as_uint(v1), 0x7632);
 }
 
-// One thread's row of a tile slot.
-struct Tc3Row {
+// One thread's row of a tile slot (rows and points are counted in 32 bits: pipe_launch's callers take
+// another kernel for 2^31 rows or more).
+struct PipeRow {
   int cls, psrc, kidx;   // class, lane of the point's primal row, output block (-1: not written)
-  int64_t p;             // point
+  int p;                 // point
+};
+// Its raw first-layer inputs 8 c .. 8 c + 7 in the padded layout (coordinates at 0 .. 3, latents from
+// kTcLat): latents or directions, and coordinates of primal rows as stored; hot is the one-hot entry
+// of a tangent row (-1: none).
+struct PipeIn {
+  float v[8];
+  int hot;
+  bool primal;
 };
 
-template <int NS>
+// Row of a lane in the lane group whose first row is g0 (rows in (point, kind) order, U per group).
+template <int MODE>
+__device__ __forceinline__ PipeRow pipe_row(const DecArgs& a, int g0, int U, int n_rows, int lane, int& kind) {
+  PipeRow rs;
+  kind = -1;
+  rs.cls = -1;
+  rs.psrc = lane;
+  rs.kidx = -1;
+  if (MODE == PIPE_PRIMAL) {
+    rs.p = g0 + lane;
+    if (rs.p < n_rows) kind = rs.cls = rs.kidx = 0;
+    return rs;
+  }
+  const int p0 = (int)((uint32_t)g0 / (uint32_t)a.R);   // point of the group's first row
+  const int row = U == 32 ? g0 + lane : lane == 0 ? p0 * a.R : g0 + lane - 1;
+  const uint32_t off = (uint32_t)(row - p0 * a.R);      // 0 .. R + 30
+  const int dp = (int)(off / (uint32_t)a.R), k = (int)off - dp * a.R;
+  rs.p = p0 + dp;
+  if (row < n_rows) {
+    kind = a.kinds[k];
+    rs.cls = kind_class(kind);
+    rs.kidx = (U != 32 && lane == 0) ? -1 : k;
+    rs.psrc = U == 32 ? lane - k : max(lane - k, 0);    // before the group's first row: lane 0's copy
+  }
+  return rs;
+}
+
+// The row's inputs (loads only: pipe_finish does the arithmetic, so that the loads stay in flight).
+// vec4: latent and direction rows are 16-byte aligned and r is a multiple of 4.
+template <int MODE>
+__device__ __forceinline__ PipeRow pipe_load(const DecArgs& a, int g0, int U, int n_rows, int lane, int c, bool vec4,
+                                             PipeIn& in) {
+  int kind;
+  const PipeRow rs = pipe_row<MODE>(a, g0, U, n_rows, lane, kind);
+  const float *vec = nullptr, *xp = nullptr;   // latent part, coordinates
+  in.hot = -1;
+  in.primal = rs.cls == 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) in.v[j] = 0.f;
+  if (rs.cls >= 0) {
+    int64_t xrow = rs.p;
+    int li = 0;
+    if (a.n_dev && a.n_rep <= 1) {
+      if (a.idx) xrow = a.idx[rs.p];           // one latent row: point p is row idx[p]
+    } else if (!a.n_dev) {
+      li = a.lat ? a.lat[rs.p] : a.lat_per_point ? rs.p : 0;
+    } else {
+      RowInfo ri;
+      ri.p = rs.p;
+      row_source(a, ri, xrow, li);
+    }
+    if (rs.cls == 0) {
+      vec = a.latents + (int64_t)li * a.r;
+      xp = a.X + xrow * a.d;
+    } else if (rs.cls == 1 && kind != KIND_JVP) {
+      in.hot = kind - 1 < a.d ? kind - 1 : kind - 1 - a.d + kTcLat;
+    } else {
+      vec = a.dirs + dir_offset(a, kind, li);
+    }
+  }
+  const int i0 = 8 * c - kTcLat;               // latent index of the first input
+  if (c == 0 && xp) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (j < a.d) in.v[j] = xp[j];
+  }
+  if (vec) {
+    if (vec4) {
+      if (c > 0 && i0 < a.r) {
+        const float4 q = *reinterpret_cast<const float4*>(vec + i0);
+        in.v[0] = q.x;
+        in.v[1] = q.y;
+        in.v[2] = q.z;
+        in.v[3] = q.w;
+      }
+      if (i0 + 4 < a.r) {
+        const float4 q = *reinterpret_cast<const float4*>(vec + i0 + 4);
+        in.v[4] = q.x;
+        in.v[5] = q.y;
+        in.v[6] = q.z;
+        in.v[7] = q.w;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (i0 + j >= 0 && i0 + j < a.r) in.v[j] = vec[i0 + j];
+    }
+  }
+  return rs;
+}
+template <int MODE>
+__device__ __forceinline__ void pipe_finish(int d, const float* norm, int c, PipeIn& in) {
+  if (c == 0) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (j < d) in.v[j] = in.primal ? (in.v[j] - norm[j]) / norm[d + j] : in.hot == j ? 1.f / norm[d + j] : 0.f;
+  }
+  if (MODE != PIPE_PRIMAL) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (8 * c + j == in.hot && in.hot >= kTcLat) in.v[j] = 1.f;
+  }
+}
+__device__ __forceinline__ bool pipe_vec4(const DecArgs& a) {
+  return (a.r & 3) == 0 && (((uintptr_t)a.latents | (uintptr_t)a.dirs) & 15u) == 0;
+}
+
+// Activations of 16 columns of a row from their pre-activations (bias included on primal rows):
+//   primal   z, or e^z - 1 below zero           tangent  zd, or e^zp zd
+//   secant   dz, or e^zp expm1(dz) while both ends are negative and dz is small, else elu_secant
+// with zp the primal pre-activation of the row's point (lane psrc).  Below zero all three are
+// e^zp m + c: per-lane constants make one expression of the classes of a warp's rows.
+template <int MODE>
+__device__ __forceinline__ void pipe_activate(float (&z)[16], const PipeRow& rs) {
+  if (MODE == PIPE_IDENTITY) return;
+  if (MODE == PIPE_PRIMAL) {
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+      float x0 = z[i], x1 = z[i + 1];
+      mul2(x0, x1, kLog2e);
+      x0 = ex2_ftz(x0);
+      x1 = ex2_ftz(x1);
+      add2(x0, x1, -1.0f, -1.0f);
+      z[i] = z[i] > 0.f ? z[i] : x0;
+      z[i + 1] = z[i + 1] > 0.f ? z[i + 1] : x1;
+    }
+    return;
+  }
+  const bool primal = rs.cls == 0;
+  const float neg_c = primal ? -1.0f : 0.0f;
+  const uint32_t keep = primal ? 0u : 0xffffffffu, one = primal ? 0x3f800000u : 0u;
+  if (MODE == PIPE_TANGENT) {
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+      const float p0 = __shfl_sync(0xffffffffu, z[i], rs.psrc);
+      const float p1 = __shfl_sync(0xffffffffu, z[i + 1], rs.psrc);
+      float x0 = p0, x1 = p1;
+      mul2(x0, x1, kLog2e);
+      x0 = fmaf(ex2_ftz(x0), __uint_as_float((__float_as_uint(z[i]) & keep) | one), neg_c);
+      x1 = fmaf(ex2_ftz(x1), __uint_as_float((__float_as_uint(z[i + 1]) & keep) | one), neg_c);
+      z[i] = p0 > 0.f ? z[i] : x0;
+      z[i + 1] = p1 > 0.f ? z[i + 1] : x1;
+    }
+    return;
+  }
+  const bool sec = rs.cls == 2;
+  const float secf = sec ? 1.0f : 0.0f;
+#pragma unroll
+  for (int i0 = 0; i0 < 16; i0 += 8) {
+    float zp[8], out[8];
+    bool rare = false;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float dz = z[i0 + j];
+      zp[j] = __shfl_sync(0xffffffffu, dz, rs.psrc);
+      const float z1 = fmaf(dz, secf, zp[j]);
+      const bool pos = fminf(zp[j], z1) > 0.f;
+      const float poly =
+          dz *
+          fmaf(0.5f * dz,
+               fmaf(dz * (1.f / 3.f), fmaf(0.25f * dz, fmaf(0.2f * dz, fmaf(dz, 1.f / 6.f, 1.f), 1.f), 1.f), 1.f), 1.f);
+      const float m = sec ? poly : __uint_as_float((__float_as_uint(dz) & keep) | one);
+      rare |= sec && !pos && !(fmaxf(zp[j], z1) <= 0.f && fabsf(dz) < 0.03125f);
+      out[j] = pos ? dz : fmaf(ex2_ftz(zp[j] * kLog2e), m, neg_c);
+    }
+    // ends of opposite sign or a large increment: the general form, for the lanes that need it
+    if (__any_sync(0xffffffffu, rare)) {
+      if (rare) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) out[j] = elu_secant(zp[j], z[i0 + j]);
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) z[i0 + j] = out[j];
+  }
+}
+
+template <int NS, int MODE>
 __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte alignment by an offset, so that the pointers stay known as shared memory
@@ -1155,7 +1157,8 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
   float* sb0 = ypart + 3 * 128 * 3;                      // [128]
   float* sbh = sb0 + kW;                                 // [kMaxTC][128]
   float* sWout = sbh + kMaxTC * kW;                      // [3][128]
-  Tc3Tail* tail = (Tc3Tail*)(sWout + 3 * kW);
+  float* snorm = sWout + 3 * kW;                         // [8] X_min, X_range
+  Tc3Tail* tail = (Tc3Tail*)(snorm + 8);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 
   if (t == 0) {
@@ -1173,29 +1176,29 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
   for (int e = t; e < kW; e += tc3_threads<NS>()) sb0[e] = a.b0[e];
   for (int e = t; e < a.n_tc * kW; e += tc3_threads<NS>()) sbh[e] = a.bh[e];
   for (int e = t; e < 3 * kW; e += tc3_threads<NS>()) sWout[e] = e < a.d * kW ? a.Wout[e] : 0.f;
+  if (t < 2 * a.d) snorm[t] = a.norm[t];
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
 
-  const int64_t n_pts = dec_count(a);
-  const int64_t n_rows = n_pts * a.R;
-  const int U = a.tc3_U;
-  const int64_t n_tiles = (n_rows + 4 * U - 1) / (4 * U);
+  const int n_rows = (int)dec_count(a) * a.R;
+  const int U = a.pipe_U;
+  const int n_tiles = (int)(((int64_t)n_rows + 4 * U - 1) / (4 * U));
   // tiles per pass: one while every tile has a CTA of its own (slot 1 then has none)
-  const int NT = n_tiles <= gridDim.x ? 1 : NS;
-  const int64_t n_iter = (n_tiles + NT - 1) / NT;
-  const int K0 = a.d + a.r;
-  const int KS0 = (K0 + 15) / 16;                         // first-layer K steps
+  const int NT = n_tiles <= (int)gridDim.x ? 1 : NS;
+  const int n_iter = (n_tiles + NT - 1) / NT;
+  const int K0 = kTcLat + a.r;                            // first-layer inputs, padded layout
+  const int KS0 = (K0 + 15) / 16;                         // their K steps
   const int atoms = 3 + 6 * a.n_tc;
 
-  if (warp == kTc3Epi / 32) {
+  if (warp == kEpiThreads / 32) {
     // ---- weight stream
     if (lane == 0) {
       uint32_t i = 0;
-      for (int64_t it = blockIdx.x; it < n_iter; it += gridDim.x)
+      for (int it = blockIdx.x; it < n_iter; it += gridDim.x)
         for (int j = 0; j < atoms; ++j, ++i) {
           const uint32_t slot = i % kRing, use = i / kRing;
-          if (use > 0) tc3_wait(a, &tail->abort, &tail->empty[slot], (use - 1) & 1u);
+          if (use > 0) pipe_wait(a, &tail->abort, &tail->empty[slot], (use - 1) & 1u);
           tc::mbar_expect_tx(&tail->full[slot], (uint32_t)kAtomBytes);
           tc::bulk_g2s(ring + slot * kAtomBytes, a.wstream + (size_t)j * kAtomBytes, kAtomBytes, &tail->full[slot]);
         }
@@ -1205,9 +1208,9 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
           (void)tc::mbar_wait(&tail->full[k % kRing], (k / kRing) & 1u);
     }
     __syncwarp();
-  } else if (warp > kTc3Epi / 32) {
+  } else if (warp > kEpiThreads / 32) {
     // ---- MMA issuer of slot s.  The whole warp runs the loop; one elected lane issues.
-    const int s = warp - kTc3Epi / 32 - 1;
+    const int s = warp - kEpiThreads / 32 - 1;
     const bool leader = tc::elect_one();
     const uint32_t tD = tail->tmem + (uint32_t)(s * 256), tAh = tD + 128, tAm = tD + 192;
     const uint32_t lo_desc = tc::smem_desc_sw128_lo(tc::smem_addr(lotile + s * kLayerBytes));
@@ -1217,12 +1220,12 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
     // waits for the next atom of the stream, returns its ring slot
     auto take = [&]() {
       const uint32_t slot = atom % kRing;
-      tc3_wait(a, &tail->abort, &tail->full[slot], (atom / kRing) & 1u);
+      pipe_wait(a, &tail->abort, &tail->full[slot], (atom / kRing) & 1u);
       __syncwarp();
       ++atom;
       return slot;
     };
-    for (int64_t it = blockIdx.x; it < n_iter; it += gridDim.x) {
+    for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
       if (s >= NT || it * NT + s >= n_tiles) {
         // no tile: the slot only releases the pass's atoms
         for (int j = 0; j < atoms; ++j) {
@@ -1232,7 +1235,7 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
         continue;
       }
       for (int l = -1; l < a.n_tc; ++l) {
-        tc3_sync(1 + s);
+        pipe_sync(1 + s);
         tc::tc_fence_after();
         if (l < 0) {
           // first layer: one atom per image, KS0 K steps
@@ -1289,12 +1292,12 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
         }
         if (leader) tc::mma_commit(&tail->bar_mma[s]);
         __syncwarp();
-        tc3_wait(a, &tail->abort, &tail->bar_mma[s], mma_phase);
+        pipe_wait(a, &tail->abort, &tail->bar_mma[s], mma_phase);
         mma_phase ^= 1u;
         __syncwarp();
         tc::tc_fence_after();
         tc::tc_fence_before();
-        tc3_arrive(3 + s);
+        pipe_arrive(3 + s);
       }
     }
     // MMAs of a timed-out pass complete (bounded) before the tensor memory is freed
@@ -1305,81 +1308,9 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
   } else {
     // ---- epilogue warps: rows 32 (warp % 4) + lane, columns 32 h .. 32 h + 31
     const int h = warp >> 2;
+    const bool vec4 = pipe_vec4(a);
     const int rw = (warp & 3) * 32 + lane;                 // tile row / tensor-memory lane
     const uint32_t tbase = tail->tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const bool deriv = a.R > 1;
-    bool secants = false;
-    for (int k = 1; k < a.R; ++k) secants |= kind_class(a.kinds[k]) == 2;
-
-    // The row of this thread in a tile, and its first-layer operand: inputs of primal rows,
-    // directions of the others (a one-hot entry, or a latent direction), 8 inputs per column part.
-    // load() reads the row's inputs (ahead of the last layer's accumulator wait, so that their
-    // latency is hidden), put() writes the operand once the slot is free.
-    auto load = [&](int64_t tile, float v[8], float v2[8]) {
-      const int64_t g0 = (tile * 4 + (warp & 3)) * U;
-      Tc3Row rs;
-      int kind = -1;
-      {
-        // point of the lane group's first row
-        const int64_t p0 = g0 < (int64_t)1 << 31 ? (int64_t)((uint32_t)g0 / (uint32_t)a.R) : g0 / a.R;
-        const int64_t row = U == 32 ? g0 + lane : lane == 0 ? p0 * a.R : g0 + lane - 1;
-        const int off = (int)(row - p0 * a.R);             // 0 .. R + 30
-        const int dp = off / a.R, k = off - dp * a.R;
-        rs.p = p0 + dp;
-        rs.cls = -1;
-        rs.psrc = lane;
-        rs.kidx = -1;
-        if (row < n_rows) {
-          kind = a.kinds[k];
-          rs.cls = kind_class(kind);
-          rs.kidx = (U != 32 && lane == 0) ? -1 : k;
-          rs.psrc = U == 32 ? lane - k : max(lane - k, 0);   // before the group's first row: lane 0's copy
-        }
-      }
-      const int d = a.d;
-      const float *vec = nullptr, *xp = nullptr;           // latent part, coordinates
-      int hot = -1;
-      if (rs.cls >= 0) {
-        RowInfo ri;
-        ri.p = rs.p;
-        int64_t xrow;
-        int li;
-        row_source(a, ri, xrow, li);
-        if (rs.cls == 0) {
-          vec = a.latents + (int64_t)li * a.r;
-          xp = a.X + xrow * d;
-        } else if (rs.cls == 1 && kind != KIND_JVP) {
-          hot = kind - 1;
-        } else {
-          vec = a.dirs + dir_offset(a, kind, li);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int i = 8 * h + j;
-        v[j] = (vec != nullptr && i >= d && i < K0) ? vec[i - d] : 0.f;
-        if (i == hot) v[j] = 1.f;
-      }
-      if (h == 0) {
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          if (j < d) {
-            const float range = a.norm[d + j];
-            if (xp != nullptr) v[j] = (xp[j] - a.norm[j]) / range;
-            if (j == hot) v[j] = 1.f / range;
-          }
-        }
-      }
-      if (K0 > 32) {                                       // inputs 32 .. 39 (d + r <= 40), column part 0
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int i = 32 + j;
-          v2[j] = (vec != nullptr && i < K0) ? vec[i - d] : 0.f;
-          if (i == hot) v2[j] = 1.f;
-        }
-      }
-      return rs;
-    };
     auto put8 = [&](int s, int c, const float v[8]) {      // inputs 8 c .. 8 c + 7 of the slot's operand row
       uint32_t wh[4], wm[4], wl[4];
 #pragma unroll
@@ -1390,11 +1321,16 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
       *reinterpret_cast<uint4*>(lotile + s * kLayerBytes + tc::sw128_offset(rw, 8 * c, kW)) =
           make_uint4(wl[0], wl[1], wl[2], wl[3]);
     };
-    auto put = [&](int s, const float v[8], const float v2[8]) {
-      if (h < 2 * KS0) put8(s, h, v);
+    // first-layer operand of a slot: inputs 0 .. 31 by the four column parts, 32 .. 47 (K0 > 32) by
+    // the first two, which load the last 8 here
+    auto put = [&](int s, int tile, PipeIn& in) {
+      pipe_finish<MODE>(a.d, snorm, h, in);
+      if (h < 2 * KS0) put8(s, h, in.v);
       if (K0 > 32 && h < 2) {
-        const float zero[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        put8(s, 4 + h, h == 0 ? v2 : zero);
+        PipeIn hi;
+        (void)pipe_load<MODE>(a, (tile * 4 + (warp & 3)) * U, U, n_rows, lane, 4 + h, vec4, hi);
+        pipe_finish<MODE>(a.d, snorm, 4 + h, hi);
+        put8(s, 4 + h, hi.v);
       }
     };
     // the slot's operand is complete and its accumulator read: its issuer may go on
@@ -1402,42 +1338,43 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
       tc::tmem_wait_st();
       tc::fence_async_smem();
       tc::tc_fence_before();
-      tc3_arrive(1 + s);
+      pipe_arrive(1 + s);
     };
 
-    Tc3Row rows[NS];
+    PipeRow rows[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-      const int64_t tile = (int64_t)blockIdx.x * NT + s;
-      if (blockIdx.x < n_iter && s < NT && tile < n_tiles) {
-        float v[8], v2[8];
-        rows[s] = load(tile, v, v2);
-        put(s, v, v2);
+      const int tile = blockIdx.x * NT + s;
+      if ((int)blockIdx.x < n_iter && s < NT && tile < n_tiles) {
+        PipeIn in;
+        rows[s] = pipe_load<MODE>(a, (tile * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
+        put(s, tile, in);
         ready(s);
       }
     }
-    for (int64_t it = blockIdx.x; it < n_iter; it += gridDim.x) {
+    for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
       for (int l = -1; l < a.n_tc; ++l) {
         const bool last = l == a.n_tc - 1;
         const float* bl = l < 0 ? sb0 : sbh + l * kW;
-#pragma unroll
+#pragma unroll 1
         for (int s = 0; s < NS; ++s) {
           if (s >= NT || it * NT + s >= n_tiles) break;
-          const Tc3Row rs = rows[s];
+          const PipeRow rs = s == 0 ? rows[0] : rows[NS - 1];
           const bool primal = rs.cls == 0;
-          // per-lane constants that make one expression of both row classes: below zero a primal row
-          // is e^z 1 - 1, a tangent row e^z zd + 0; the factor is (zd & keep) | one
-          const float neg_c = primal ? -1.0f : 0.0f, one_p = primal ? 1.0f : 0.0f;
-          const uint32_t keep = primal ? 0u : 0xffffffffu, one = __float_as_uint(one_p);
+          const float one_p = primal ? 1.0f : 0.0f;
           const uint32_t ts = tbase + s * 256;
           uint8_t* lo_t = lotile + s * kLayerBytes;
           float y[3] = {0.f, 0.f, 0.f};
           // the slot's next tile: its inputs load while the last accumulator completes
-          float v[8], v2[8];
-          const int64_t next = it + gridDim.x;
-          const bool more = last && next < n_iter && next * NT + s < n_tiles;
-          if (more) rows[s] = load(next * NT + s, v, v2);
-          tc3_sync(3 + s);
+          PipeIn in;
+          const int next = (it + (int)gridDim.x) * NT + s;
+          const bool more = last && it + (int)gridDim.x < n_iter && next < n_tiles;
+          if (more) {
+            const PipeRow nr = pipe_load<MODE>(a, (next * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
+            if (s == 0) rows[0] = nr;
+            else rows[NS - 1] = nr;
+          }
+          pipe_sync(3 + s);
           tc::tc_fence_after();
 #pragma unroll 1
           for (int c0 = 32 * h; c0 < 32 * h + 32; c0 += 16) {
@@ -1450,41 +1387,7 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
               fma2(z[i], z[i + 1], b4.x, b4.y, one_p);
               fma2(z[i + 2], z[i + 3], b4.z, b4.w, one_p);
             }
-            if (a.act == 0) {
-              if (!deriv) {
-#pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                  float x0 = z[i], x1 = z[i + 1];
-                  mul2(x0, x1, kLog2e);
-                  x0 = ex2_ftz(x0);
-                  x1 = ex2_ftz(x1);
-                  add2(x0, x1, -1.0f, -1.0f);
-                  z[i] = z[i] > 0.f ? z[i] : x0;
-                  z[i + 1] = z[i + 1] > 0.f ? z[i + 1] : x1;
-                }
-              } else if (!secants) {
-                // primal rows: z, or e^z - 1 below zero; tangent rows: zd, or e^z zd
-#pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                  const float p0 = __shfl_sync(0xffffffffu, z[i], rs.psrc);
-                  const float p1 = __shfl_sync(0xffffffffu, z[i + 1], rs.psrc);
-                  float x0 = p0, x1 = p1;
-                  mul2(x0, x1, kLog2e);
-                  x0 = fmaf(ex2_ftz(x0), __uint_as_float((__float_as_uint(z[i]) & keep) | one), neg_c);
-                  x1 = fmaf(ex2_ftz(x1), __uint_as_float((__float_as_uint(z[i + 1]) & keep) | one), neg_c);
-                  z[i] = p0 > 0.f ? z[i] : x0;
-                  z[i + 1] = p1 > 0.f ? z[i + 1] : x1;
-                }
-              } else {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                  const float zp = __shfl_sync(0xffffffffu, z[i], rs.psrc);
-                  const float neg = fmaf(ex2_ftz(zp * kLog2e), primal ? 1.0f : z[i], neg_c);
-                  const float pt = zp > 0.f ? z[i] : neg;
-                  z[i] = rs.cls == 2 ? elu_secant(zp, z[i]) : pt;
-                }
-              }
-            }
+            pipe_activate<MODE>(z, rs);
             if (last) {
               // output layer fused into the last epilogue (FP32), partial over this part's columns
 #pragma unroll
@@ -1517,26 +1420,275 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
             continue;
           }
           if (more) {
-            put(s, v, v2);
+            put(s, next, in);
             ready(s);
           }
-          if (h > 0) {
+          if (h < 3) {
 #pragma unroll
             for (int o = 0; o < 3; ++o)
-              if (o < a.d) ypart[((h - 1) * 128 + rw) * 3 + o] = y[o];
+              if (o < a.d) ypart[(h * 128 + rw) * 3 + o] = y[o];
           }
-          tc3_epi_sync();
-          if (h == 0 && rs.kidx >= 0) {
+          // part 3 (part 0 has the coordinates' divisions in put) waits for the others; they go on
+          // (ypart is rewritten after the next accumulator barrier, which part 3 reaches only when it
+          // has read it)
+          pipe_combine(h);
+          if (h == 3 && rs.kidx >= 0) {
             float* o = a.out + ((int64_t)rs.kidx * a.n + rs.p) * a.d;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
               if (i >= a.d) break;
-              float v = (y[i] + ypart[rw * 3 + i]) + (ypart[(128 + rw) * 3 + i] + ypart[(256 + rw) * 3 + i]);
+              float v = (ypart[rw * 3 + i] + ypart[(128 + rw) * 3 + i]) + (ypart[(256 + rw) * 3 + i] + y[i]);
               if (primal) v += __ldg(&a.bout[i]);
               o[i] = v * a.norm[3 * a.d + i] + (primal ? a.norm[2 * a.d + i] : 0.f);
             }
           }
-          tc3_epi_sync();   // ypart is free for the next tile
+        }
+      }
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_free<256 * NS>(tail->tmem);
+}
+
+// --------------------------------------------------------------------------
+// BF16 decoder for calls without mixed rows (primal, tangent, JVP and secant rows; inputs of at
+// most 32 entries in the padded layout), built like decoder_tc3: rows in (point, kind) order, the
+// primal pre-activation of a derivative row fetched by a shuffle, sixteen epilogue warps taking the
+// NS tile slots in turn, one MMA issuer warp per slot.  All weights are resident (four 32 KB layers
+// and the first layer's split image), and the A operand sits in tensor memory alone: 64 columns of
+// BF16 activations, or for the first layer 16 + 16 of the inputs' high and low parts.  The
+// arithmetic and its order are decoder_tc<false>'s, so the results are the same bits.
+//
+// What bounds it: the epilogue, 1.7k cycles per tile and layer (the special-function unit's 16
+// exponentials a clock take 1.0k of them), and about 3k per tile for its inputs and outputs; the
+// tensor core is busy 20 % of the time.  1,048,576 primal rows: 0.297 ms (0.493 ms as two groups of
+// eight warps with a tile each, whose epilogues ran at the latency of two warps per scheduler);
+// 100,003 points x 4 rows 0.173 ms (0.446 ms in decoder_tc, which exchanges the rows'
+// pre-activations through shared memory); 5,001 points x 9 rows 35 us (87 us).
+// --------------------------------------------------------------------------
+template <int NS>
+constexpr int bf16_threads() { return kEpiThreads + 32 * NS; }
+
+struct __align__(8) Bf16Tail {
+  uint64_t bar_w;
+  uint64_t bar_mma[2];
+  uint64_t drain;
+  uint32_t tmem;
+  int abort;      // a wait ran out (as in decoder_tc3)
+};
+
+template <int NS, int MODE>
+__global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (tc::smem_addr(smem_raw) & 1023u)) & 1023u);
+  uint8_t* wsm = smem;                                   // kMaxTC x 32 KB square layers
+  uint8_t* w0s = smem + kMaxTC * kLayerBytes;            // 16 KB first-layer split image
+  float* ypart = (float*)(w0s + kLayerBytes / 2);        // [3][128][3]
+  float* sb0 = ypart + 3 * 128 * 3;                      // [128]
+  float* sbh = sb0 + kW;                                 // [kMaxTC][128]
+  float* sWout = sbh + kMaxTC * kW;                      // [3][128]
+  float* snorm = sWout + 3 * kW;                         // [8] X_min, X_range
+  Bf16Tail* tail = (Bf16Tail*)(snorm + 8);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+
+  if (t == 0) {
+    tc::mbar_init(&tail->bar_w, 1);
+    tc::mbar_init(&tail->bar_mma[0], 1);
+    tc::mbar_init(&tail->bar_mma[1], 1);
+    tc::mbar_init(&tail->drain, NS);
+    tail->abort = 0;
+    tc::fence_mbar_init();
+    tc::mbar_expect_tx(&tail->bar_w, (uint32_t)(a.n_tc * kLayerBytes + kLayerBytes / 2));
+    tc::bulk_g2s(w0s, a.w0img, kLayerBytes / 2, &tail->bar_w);
+    for (int l = 0; l < a.n_tc; ++l)
+      tc::bulk_g2s(wsm + l * kLayerBytes, a.wimg + (size_t)l * kLayerBytes, kLayerBytes, &tail->bar_w);
+  }
+  if (warp == 0) tc::tmem_alloc<256 * NS>(&tail->tmem);
+  for (int e = t; e < kW; e += bf16_threads<NS>()) sb0[e] = a.b0[e];
+  for (int e = t; e < a.n_tc * kW; e += bf16_threads<NS>()) sbh[e] = a.bh[e];
+  for (int e = t; e < 3 * kW; e += bf16_threads<NS>()) sWout[e] = e < a.d * kW ? a.Wout[e] : 0.f;
+  if (t < 2 * a.d) snorm[t] = a.norm[t];
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+
+  const int n_rows = (int)dec_count(a) * a.R;
+  const int U = a.pipe_U;
+  const int n_tiles = (int)(((int64_t)n_rows + 4 * U - 1) / (4 * U));
+  const int NT = n_tiles <= (int)gridDim.x ? 1 : NS;          // tiles per pass, as in decoder_tc3
+  const int n_iter = (n_tiles + NT - 1) / NT;
+
+  if (warp >= kEpiThreads / 32) {
+    // ---- MMA issuer of slot s
+    const int s = warp - kEpiThreads / 32;
+    const bool leader = tc::elect_one();
+    const uint32_t tD = tail->tmem + (uint32_t)(s * 256), tA = tD + 128, tI = tD + 192;   // tI: inputs hi, lo
+    const uint32_t w_desc = tc::smem_desc_sw128_lo(tc::smem_addr(wsm));
+    const uint32_t w0_desc = tc::smem_desc_sw128_lo(tc::smem_addr(w0s));
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW);
+    uint32_t mma_phase = 0;
+    pipe_wait(a, &tail->abort, &tail->bar_w, 0);
+    __syncwarp();
+    for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
+      if (s >= NT || it * NT + s >= n_tiles) continue;
+      for (int l = -1; l < a.n_tc; ++l) {
+        pipe_sync(1 + s);
+        tc::tc_fence_after();
+        if (leader) {
+          if (l < 0) {
+            auto desc = [](uint32_t lo) { return ((uint64_t)tc::kDescSw128Hi << 32) | lo; };
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {   // hi at byte 0 of an image row, lo at byte 64
+              tc::mma_bf16_ts(tD, tI + 8 * k, desc(w0_desc + 2 * k), idesc, k > 0 ? 1u : 0u);
+              tc::mma_bf16_ts(tD, tI + 8 * k, desc(w0_desc + 4 + 2 * k), idesc, 1u);
+              tc::mma_bf16_ts(tD, tI + 16 + 8 * k, desc(w0_desc + 2 * k), idesc, 1u);
+            }
+          } else {
+            const uint32_t bd = w_desc + (uint32_t)l * (kLayerBytes >> 4);
+            tc::mma4_bf16_ts(tD, tA, bd, idesc, 0u);
+            tc::mma4_bf16_ts(tD, tA + 32, bd + (kAtomBytes >> 4), idesc, 1u);
+          }
+          tc::mma_commit(&tail->bar_mma[s]);
+        }
+        __syncwarp();
+        pipe_wait(a, &tail->abort, &tail->bar_mma[s], mma_phase);
+        mma_phase ^= 1u;
+        __syncwarp();
+        tc::tc_fence_after();
+        tc::tc_fence_before();
+        pipe_arrive(3 + s);
+      }
+    }
+    // MMAs of a timed-out pass complete (bounded) before the tensor memory is freed; the weights
+    // have landed (waited for above, or here after a timeout)
+    if (leader) tc::mma_commit(&tail->drain);
+    __syncwarp();
+    (void)tc::mbar_wait(&tail->drain, 0);
+    if (*(volatile int*)&tail->abort) (void)tc::mbar_wait(&tail->bar_w, 0);
+    __syncwarp();
+  } else {
+    // ---- epilogue warps: rows 32 (warp % 4) + lane, columns 32 h .. 32 h + 31
+    const int h = warp >> 2;
+    const bool vec4 = pipe_vec4(a);
+    const int rw = (warp & 3) * 32 + lane;
+    const uint32_t tbase = tail->tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    auto pack2 = [](float v0, float v1) {
+      const __nv_bfloat162 b = __floats2bfloat162_rn(v0, v1);
+      return *reinterpret_cast<const uint32_t*>(&b);
+    };
+    // first-layer operand (inputs in the padded layout: coordinates at 0 .. 3, latents from
+    // kTcLat): bf16(v) and bf16(v - bf16(v))
+    auto put = [&](int s, PipeIn& in) {
+      pipe_finish<MODE>(a.d, snorm, h, in);
+      const float* v = in.v;
+      uint32_t wh[4], wl[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        wh[j] = pack2(v[2 * j], v[2 * j + 1]);
+        wl[j] = pack2(v[2 * j] - __uint_as_float(wh[j] << 16), v[2 * j + 1] - __uint_as_float(wh[j] & 0xffff0000u));
+      }
+      __syncwarp();
+      tc::tmem_st4(tbase + s * 256 + 192 + 4 * h, wh);
+      tc::tmem_st4(tbase + s * 256 + 208 + 4 * h, wl);
+    };
+    auto ready = [&](int s) {
+      tc::tmem_wait_st();
+      tc::tc_fence_before();
+      pipe_arrive(1 + s);
+    };
+
+    PipeRow rows[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int tile = blockIdx.x * NT + s;
+      if ((int)blockIdx.x < n_iter && s < NT && tile < n_tiles) {
+        PipeIn in;
+        rows[s] = pipe_load<MODE>(a, (tile * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
+        put(s, in);
+        ready(s);
+      }
+    }
+    for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
+      for (int l = -1; l < a.n_tc; ++l) {
+        const bool last = l == a.n_tc - 1;
+        const float* bl = l < 0 ? sb0 : sbh + l * kW;
+#pragma unroll 1
+        for (int s = 0; s < NS; ++s) {
+          if (s >= NT || it * NT + s >= n_tiles) break;
+          const PipeRow rs = s == 0 ? rows[0] : rows[NS - 1];
+          const bool primal = rs.cls == 0;
+          const float one_p = primal ? 1.0f : 0.0f;
+          const uint32_t ts = tbase + s * 256;
+          float y[3] = {0.f, 0.f, 0.f};
+          // the slot's next tile: its inputs load while the last accumulator completes
+          PipeIn in;
+          const int next = (it + (int)gridDim.x) * NT + s;
+          const bool more = last && it + (int)gridDim.x < n_iter && next < n_tiles;
+          if (more) {
+            const PipeRow nr = pipe_load<MODE>(a, (next * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
+            if (s == 0) rows[0] = nr;
+            else rows[NS - 1] = nr;
+          }
+          pipe_sync(3 + s);
+          tc::tc_fence_after();
+#pragma unroll 1
+          for (int c0 = 32 * h; c0 < 32 * h + 32; c0 += 16) {
+            float z[16];
+            tc::tmem_ld16(ts + c0, z);
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) {   // the bias of primal rows (a factor 0 on the others)
+              const float4 b4 = *reinterpret_cast<const float4*>(bl + c0 + i);
+              fma2(z[i], z[i + 1], b4.x, b4.y, one_p);
+              fma2(z[i + 2], z[i + 3], b4.z, b4.w, one_p);
+            }
+            pipe_activate<MODE>(z, rs);
+            if (last) {
+              // output layer fused into the last epilogue (FP32): one chain over the part's 32 columns
+#pragma unroll
+              for (int o = 0; o < 3; ++o) {
+                if (o >= a.d) break;
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                  const float4 w4 = *reinterpret_cast<const float4*>(sWout + o * kW + c0 + i);
+                  y[o] = fmaf(w4.x, z[i], y[o]);
+                  y[o] = fmaf(w4.y, z[i + 1], y[o]);
+                  y[o] = fmaf(w4.z, z[i + 2], y[o]);
+                  y[o] = fmaf(w4.w, z[i + 3], y[o]);
+                }
+              }
+            } else {
+              uint32_t w[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) w[j] = pack2(z[2 * j], z[2 * j + 1]);
+              tc::tmem_st8(ts + 128 + c0 / 2, w);
+            }
+          }
+          if (!last) {
+            ready(s);
+            continue;
+          }
+          if (more) {
+            put(s, in);
+            ready(s);
+          }
+          if (h < 3) {
+#pragma unroll
+            for (int o = 0; o < 3; ++o)
+              if (o < a.d) ypart[(h * 128 + rw) * 3 + o] = y[o];
+          }
+          pipe_combine(h);   // as in decoder_tc3
+          if (h == 3 && rs.kidx >= 0) {
+            float* o = a.out + ((int64_t)rs.kidx * a.n + rs.p) * a.d;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              if (i >= a.d) break;
+              float vo = (ypart[rw * 3 + i] + ypart[(128 + rw) * 3 + i]) + (ypart[(256 + rw) * 3 + i] + y[i]);
+              vo += primal ? __ldg(&a.bout[i]) : 0.f;
+              o[i] = vo * a.norm[3 * a.d + i] + (primal ? a.norm[2 * a.d + i] : 0.f);
+            }
+          }
         }
       }
     }
@@ -1598,9 +1750,9 @@ __global__ void decoder_pack_w0(const float* W0, int d, int r, uint8_t* img) {
 
 // Weight stream of decoder_tc3: per layer its low, middle and high BF16 images (w = hi + mid + lo
 // exactly, each rounded to nearest), as atoms of 128 output rows x 64 K in the 128-byte swizzled
-// K-major layout: the first layer (K = d + r <= 40, zero-padded) one atom per image, the square
-// layers two.
-__global__ void decoder_pack3(const float* W0, int K0, const float* wsq, int n_tc, uint8_t* out) {
+// K-major layout: the first layer (padded inputs, at most 42) one atom per image, the square layers
+// two.
+__global__ void decoder_pack3(const float* W0, int d, int r, const float* wsq, int n_tc, uint8_t* out) {
   const int64_t total = (int64_t)(1 + 2 * n_tc) * kW * 64;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int blk = (int)(e / (kW * 64)), rem = (int)(e % (kW * 64));
@@ -1609,7 +1761,8 @@ __global__ void decoder_pack3(const float* W0, int K0, const float* wsq, int n_t
     int64_t at;   // low atom, and the distance to the next image's
     int step;
     if (blk == 0) {
-      w = k < K0 ? W0[row * K0 + k] : 0.f;
+      const int i = k < kTcLat ? (k < d ? k : -1) : (k - kTcLat < r ? d + k - kTcLat : -1);
+      w = i >= 0 ? W0[row * (d + r) + i] : 0.f;
       at = 0;
       step = 1;
     } else {
@@ -1643,15 +1796,53 @@ size_t dec_smem_bytes(bool split) {
          sizeof(DecSmemTail);
 }
 
-size_t dec_primal_smem_bytes() {
-  return 1024 + kMaxTC * kLayerBytes + kLayerBytes / 2 + 2 * kLayerBytes +
-         (2 * 128 * 3 + kW + kMaxTC * kW + 3 * kW) * sizeof(float) + sizeof(PrimSmemTail);
+template <int NS>
+size_t dec_bf16_smem_bytes() {
+  return 1024 + kMaxTC * kLayerBytes + kLayerBytes / 2 + (3 * 128 * 3 + kW + kMaxTC * kW + 3 * kW + 8) * sizeof(float) +
+         sizeof(Bf16Tail);
 }
 
 template <int NS>
 size_t dec_tc3_smem_bytes() {
-  return 1024 + kRing * kAtomBytes + NS * kLayerBytes + (3 * 128 * 3 + kW + kMaxTC * kW + 3 * kW) * sizeof(float) +
+  return 1024 + kRing * kAtomBytes + NS * kLayerBytes + (3 * 128 * 3 + kW + kMaxTC * kW + 3 * kW + 8) * sizeof(float) +
          sizeof(Tc3Tail);
+}
+
+template <int NS, int MODE>
+cudaError_t pipe_limit() {
+  const cudaError_t e = cudaFuncSetAttribute(decoder_bf16<NS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)dec_bf16_smem_bytes<NS>());
+  return e != cudaSuccess ? e
+                          : cudaFuncSetAttribute(decoder_tc3<NS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)dec_tc3_smem_bytes<NS>());
+}
+cudaError_t pipe_limits() {
+  for (cudaError_t (*f)() : {pipe_limit<1, 0>, pipe_limit<1, 1>, pipe_limit<1, 2>, pipe_limit<1, 3>, pipe_limit<2, 0>,
+                             pipe_limit<2, 1>, pipe_limit<2, 2>, pipe_limit<2, 3>})
+    if (const cudaError_t e = f(); e != cudaSuccess) return e;
+  return cudaSuccess;
+}
+
+// decoder_tc3 (fp32) or decoder_bf16 over `tiles` tiles of 128 rows with NS tile slots per CTA.
+template <int NS, int MODE>
+void pipe_launch(const DecArgs& a, bool fp32, int blocks, cudaStream_t s) {
+  if (fp32)
+    decoder_tc3<NS, MODE><<<blocks, tc3_threads<NS>(), dec_tc3_smem_bytes<NS>(), s>>>(a);
+  else
+    decoder_bf16<NS, MODE><<<blocks, bf16_threads<NS>(), dec_bf16_smem_bytes<NS>(), s>>>(a);
+}
+// Rows in (point, kind) order, 32 (whole points) or 31 per lane group, four lane groups per tile; one
+// tile per CTA while every tile has an SM of its own (of this caller's share), else two.
+void pipe_launch(DecArgs& a, bool fp32, int64_t n_rows, int n_sm, int share, bool secants, cudaStream_t s) {
+  a.pipe_U = 32 % a.R == 0 ? 32 : 31;
+  const int64_t tiles = (n_rows + 4 * a.pipe_U - 1) / (4 * a.pipe_U);
+  const int mode = a.act != 0 ? PIPE_IDENTITY : a.R == 1 ? PIPE_PRIMAL : secants ? PIPE_SECANT : PIPE_TANGENT;
+  const bool one = tiles <= share;
+  const int blocks = (int)(one ? tiles : std::min<int64_t>((tiles + 1) / 2, n_sm));
+  void (*f[2][4])(const DecArgs&, bool, int, cudaStream_t) = {
+      {pipe_launch<1, 0>, pipe_launch<1, 1>, pipe_launch<1, 2>, pipe_launch<1, 3>},
+      {pipe_launch<2, 0>, pipe_launch<2, 1>, pipe_launch<2, 2>, pipe_launch<2, 3>}};
+  f[one ? 0 : 1][mode](a, fp32, blocks, s);
 }
 
 size_t dec_f32_smem_bytes() {
@@ -1674,7 +1865,7 @@ mpm_status refresh_derived_impl(mpm_decoder* dec, cudaStream_t s) {
   decoder_transpose<<<16, 256, 0, s>>>(dec->wsq, dec->n_tc, dec->wsqT);
   MPM_CUDA_TRY(cudaGetLastError());
   decoder_pack3<<<std::max(1, std::min(dec->n_sm * 4, (1 + 2 * dec->n_tc) * 32)), 256, 0, s>>>(
-      dec->params + dec->w_off[0], dec->d + dec->r, dec->wsq, dec->n_tc, dec->wstream);
+      dec->params + dec->w_off[0], dec->d, dec->r, dec->wsq, dec->n_tc, dec->wstream);
   MPM_CUDA_TRY(cudaGetLastError());
   if (dec->w0img) {
     decoder_pack_w0<<<16, 256, 0, s>>>(dec->params + dec->w_off[0], dec->d, dec->r, dec->w0img);
@@ -1767,13 +1958,7 @@ mpm_status decoder_create(const decoder_desc* desc, mpm_decoder** out) {
     e = cudaFuncSetAttribute(decoder_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec->smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(decoder_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec->smem_split);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(decoder_tc_primal, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)dec_primal_smem_bytes());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(decoder_tc3<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec_tc3_smem_bytes<1>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(decoder_tc3<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec_tc3_smem_bytes<2>());
+  if (e == cudaSuccess) e = pipe_limits();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(decoder_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec_f32_smem_bytes());
   if (e == cudaSuccess)
@@ -1922,27 +2107,18 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
   // FP32 calls run on the tensor cores (decoder_tc3) but for mixed rows (their partner rows are not in
   // the row's warp), for callers that keep decoder_f32's rounding, and for a lone caller's small calls
   // with secant rows (256 samples x 12 or 18 rows: 32 us against 40 us; without secants, 256 x 17
-  // rows, 31 us against 27 us the other way; 4096 x 4 rows 98 against 29 us)
+  // rows, 31 us against 24 us the other way; 4096 x 4 rows 98 against 25 us)
   bool secants = false;
   for (int k = 0; k < R; ++k) secants |= kind_class(kinds[k]) == 2;
-  const bool tc3 = f32_path && !has_mixed && !cuda_cores &&
+  const bool pipe = !has_mixed && n * R < ((int64_t)1 << 31) - 4096;   // row numbers and their padding fit 32 bits
+  const bool tc3 = f32_path && pipe && !cuda_cores &&
                    !(secants && dec->concurrency == 1 && n * R <= 31 * (int64_t)dec->n_sm);
   if (dec->n_tc == 0) {
     int64_t rows = n * R;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((rows + 127) / 128, dec->n_sm * 8));
     decoder_simt<<<blocks, 128, 0, s>>>(a);
   } else if (tc3) {
-    // rows in (point, kind) order, 32 (whole points) or 31 per lane group, four lane groups per
-    // tile; one tile per CTA while every tile has an SM of its own (of this caller's share), else two
-    a.tc3_U = 32 % R == 0 ? 32 : 31;
-    const int64_t tiles = (n * R + 4 * a.tc3_U - 1) / (4 * a.tc3_U);
-    const int64_t share = std::max(1, dec->n_sm / std::max(1, dec->concurrency));
-    if (tiles <= share) {
-      decoder_tc3<1><<<(int)tiles, tc3_threads<1>(), dec_tc3_smem_bytes<1>(), s>>>(a);
-    } else {
-      const int blocks = (int)std::min<int64_t>((tiles + 1) / 2, dec->n_sm);
-      decoder_tc3<2><<<blocks, tc3_threads<2>(), dec_tc3_smem_bytes<2>(), s>>>(a);
-    }
+    pipe_launch(a, true, n * R, dec->n_sm, std::max(1, dec->n_sm / std::max(1, dec->concurrency)), secants, s);
   } else if (f32_path) {
     MPM_CHECK_ARG(R <= kF32Rows, "the FP32 path takes at most 64 row kinds");
     int64_t tiles;
@@ -1967,12 +2143,9 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
       decoder_f32<32><<<blocks, kF32Threads, dec_f32_smem_bytes(), s>>>(a);
     else
       decoder_f32<64><<<blocks, kF32Threads, dec_f32_smem_bytes(), s>>>(a);
-  } else if (dec->fp32 == 0 && R == 1 && a.kinds[0] == KIND_PRIMAL && !a.dstore && !a.astore && dec->w0img &&
-             kTcLat + dec->r <= 32) {
-    // primal rows only: two tiles in flight per CTA
-    const int64_t tiles = (n + 127) / 128;
-    int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((tiles + 1) / 2, dec->n_sm));
-    decoder_tc_primal<<<blocks, kPrimThreads, dec_primal_smem_bytes(), s>>>(a);
+  } else if (dec->fp32 == 0 && pipe && !a.dstore && dec->w0img) {
+    // BF16 rows without partners beyond the primal, first layer on the tensor cores (r <= 28)
+    pipe_launch(a, false, n * R, dec->n_sm, dec->n_sm, secants, s);
   } else {
     const int64_t tiles = (n + a.Pt - 1) / a.Pt;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, dec->n_sm));

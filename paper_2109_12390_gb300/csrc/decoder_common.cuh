@@ -59,8 +59,8 @@ struct DecArgs {
   int lat_per_point;
   // FP32 path: useful rows per packed tile (0: point-aligned tiles of Pt points)
   int f32_U;
-  // decoder_tc3: rows per lane group (32: whole points; 31: packed, lane 0 a recomputed primal)
-  int tc3_U;
+  // decoder_tc3, decoder_bf16: rows per lane group (32: whole points; 31: packed, lane 0 a recomputed primal)
+  int pipe_U;
   // direction blocks per latent row in `dirs` (KIND_SECANT_DIR rows; 1 otherwise)
   int n_dirs;
   // training: per hidden layer l, stored feature-major [l][feature][row] (row =
