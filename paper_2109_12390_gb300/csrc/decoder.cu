@@ -40,6 +40,7 @@
 #include "tc.cuh"
 
 #include "decoder_common.cuh"
+#include "pipe.cuh"
 
 namespace mpmrom {
 
@@ -870,8 +871,6 @@ __global__ void __launch_bounds__(kF32Threads, 1) decoder_f32(DecArgs a) {
 // After a wait that ran out nothing waits on the copies or MMAs any more: the pass runs to its end
 // (in bounds, its results void) with the TIMEOUT status raised.
 // --------------------------------------------------------------------------
-constexpr int kEpiThreads = 512;              // epilogue threads
-constexpr int kAtomBytes = kW * 128;      // 128 rows x 64 BF16
 constexpr int kRing = 9;
 template <int NS>
 constexpr int tc3_threads() { return kEpiThreads + 32 + 32 * NS; }
@@ -885,60 +884,6 @@ struct __align__(8) Tc3Tail {
   int abort;      // a wait ran out
 };
 
-// Bounded wait; after a timeout anywhere in the CTA no further waits are made.
-__device__ __forceinline__ void pipe_wait(const DecArgs& a, int* abort, uint64_t* bar, uint32_t phase) {
-  if (*(volatile int*)abort) return;
-  if (!tc::mbar_wait(bar, phase)) {
-    raise_status(a.status, STATUS_TIMEOUT);
-    atomicExch(abort, 1);
-  }
-}
-
-// Barriers 1 + s: the epilogue warps arrive when slot s's next operand is complete (and its
-// accumulator read), the slot's issuer warp waits.  Barriers 3 + s: the issuer arrives when the
-// accumulator is complete, the epilogue warps wait (blocked, where polling the MMA barrier would
-// take issue slots).  Barrier 5: the column parts' output sums are in shared memory.
-__device__ __forceinline__ void pipe_arrive(int id) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kEpiThreads + 32) : "memory");
-}
-__device__ __forceinline__ void pipe_sync(int id) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kEpiThreads + 32) : "memory");
-}
-__device__ __forceinline__ void pipe_combine(int part) {
-  if (part == 3) asm volatile("bar.sync 5, %0;" ::"n"(kEpiThreads) : "memory");
-  else asm volatile("bar.arrive 5, %0;" ::"n"(kEpiThreads) : "memory");
-}
-
-// 2^x on the special-function unit, results below the normal range flushed to zero
-__device__ __forceinline__ float ex2_ftz(float x) {
-  float e;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x));
-  return e;
-}
-// Pairs of FP32 operations in one instruction (each rounded as the scalar operation)
-__device__ __forceinline__ void add2(float& a0, float& a1, float b0, float b1) {
-  asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n add.rn.f32x2 a, a, b;\n"
-      " mov.b64 {%0, %1}, a;\n}\n"
-      : "+f"(a0), "+f"(a1)
-      : "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ void mul2(float& a0, float& a1, float b) {
-  asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %2};\n mul.rn.f32x2 a, a, b;\n"
-      " mov.b64 {%0, %1}, a;\n}\n"
-      : "+f"(a0), "+f"(a1)
-      : "f"(b));
-}
-__device__ __forceinline__ void fma2(float& a0, float& a1, float b0, float b1, float c) {   // a += b c
-  asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n mov.b64 c, {%4, %4};\n"
-      " fma.rn.f32x2 a, b, c, a;\n mov.b64 {%0, %1}, a;\n}\n"
-      : "+f"(a0), "+f"(a1)
-      : "f"(b0), "f"(b1), "f"(c));
-}
-// What the rows of a call need of their activations (a template parameter: one variant's code per
-// kernel keeps the epilogue loop small)
-enum { PIPE_PRIMAL = 0, PIPE_TANGENT = 1, PIPE_SECANT = 2, PIPE_IDENTITY = 3 };
-constexpr float kLog2e = 1.4426950408889634f;   // __expf(z) is 2^(z kLog2e)
-
 // hi, mid and lo words (two BF16 values each, first value in the low half) of an FP32 pair: each
 // image the truncation of what the previous ones leave, so the three hold the 24 bits exactly
 __device__ __forceinline__ void split3(float v0, float v1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
@@ -951,128 +896,6 @@ __device__ __forceinline__ void split3(float v0, float v1, uint32_t& hi, uint32_
   mid = __byte_perm(u0, u1, 0x7632);
   add2(v0, v1, __uint_as_float((u0 & top) ^ neg), __uint_as_float((u1 & top) ^ neg));
   lo = __byte_perm(__float_as_uint(v0), __float_as_uint(v1), 0x7632);
-}
-
-// One thread's row of a tile slot (rows and points are counted in 32 bits: pipe_launch's callers take
-// another kernel for 2^31 rows or more).
-struct PipeRow {
-  int cls, psrc, kidx;   // class, lane of the point's primal row, output block (-1: not written)
-  int p;                 // point
-};
-// Its raw first-layer inputs 8 c .. 8 c + 7 in the padded layout (coordinates at 0 .. 3, latents from
-// kTcLat): latents or directions, and coordinates of primal rows as stored; hot is the one-hot entry
-// of a tangent row (-1: none).
-struct PipeIn {
-  float v[8];
-  int hot;
-  bool primal;
-};
-
-// Row of a lane in the lane group whose first row is g0 (rows in (point, kind) order, U per group).
-template <int MODE>
-__device__ __forceinline__ PipeRow pipe_row(const DecArgs& a, int g0, int U, int n_rows, int lane, int& kind) {
-  PipeRow rs;
-  kind = -1;
-  rs.cls = -1;
-  rs.psrc = lane;
-  rs.kidx = -1;
-  if (MODE == PIPE_PRIMAL) {
-    rs.p = g0 + lane;
-    if (rs.p < n_rows) kind = rs.cls = rs.kidx = 0;
-    return rs;
-  }
-  const int p0 = (int)((uint32_t)g0 / (uint32_t)a.R);   // point of the group's first row
-  const int row = U == 32 ? g0 + lane : lane == 0 ? p0 * a.R : g0 + lane - 1;
-  const uint32_t off = (uint32_t)(row - p0 * a.R);      // 0 .. R + 30
-  const int dp = (int)(off / (uint32_t)a.R), k = (int)off - dp * a.R;
-  rs.p = p0 + dp;
-  if (row < n_rows) {
-    kind = a.kinds[k];
-    rs.cls = kind_class(kind);
-    rs.kidx = (U != 32 && lane == 0) ? -1 : k;
-    rs.psrc = U == 32 ? lane - k : max(lane - k, 0);    // before the group's first row: lane 0's copy
-  }
-  return rs;
-}
-
-// The row's inputs (loads only: pipe_finish does the arithmetic, so that the loads stay in flight).
-// vec4: latent and direction rows are 16-byte aligned and r is a multiple of 4.
-template <int MODE>
-__device__ __forceinline__ PipeRow pipe_load(const DecArgs& a, int g0, int U, int n_rows, int lane, int c, bool vec4,
-                                             PipeIn& in) {
-  int kind;
-  const PipeRow rs = pipe_row<MODE>(a, g0, U, n_rows, lane, kind);
-  const float *vec = nullptr, *xp = nullptr;   // latent part, coordinates
-  in.hot = -1;
-  in.primal = rs.cls == 0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) in.v[j] = 0.f;
-  if (rs.cls >= 0) {
-    int64_t xrow = rs.p;
-    int li = 0;
-    if (a.n_dev && a.n_rep <= 1) {
-      if (a.idx) xrow = a.idx[rs.p];           // one latent row: point p is row idx[p]
-    } else if (!a.n_dev) {
-      li = a.lat ? a.lat[rs.p] : a.lat_per_point ? rs.p : 0;
-    } else {
-      RowInfo ri;
-      ri.p = rs.p;
-      row_source(a, ri, xrow, li);
-    }
-    if (rs.cls == 0) {
-      vec = a.latents + (int64_t)li * a.r;
-      xp = a.X + xrow * a.d;
-    } else if (rs.cls == 1 && kind != KIND_JVP) {
-      in.hot = kind - 1 < a.d ? kind - 1 : kind - 1 - a.d + kTcLat;
-    } else {
-      vec = a.dirs + dir_offset(a, kind, li);
-    }
-  }
-  const int i0 = 8 * c - kTcLat;               // latent index of the first input
-  if (c == 0 && xp) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-      if (j < a.d) in.v[j] = xp[j];
-  }
-  if (vec) {
-    if (vec4) {
-      if (c > 0 && i0 < a.r) {
-        const float4 q = *reinterpret_cast<const float4*>(vec + i0);
-        in.v[0] = q.x;
-        in.v[1] = q.y;
-        in.v[2] = q.z;
-        in.v[3] = q.w;
-      }
-      if (i0 + 4 < a.r) {
-        const float4 q = *reinterpret_cast<const float4*>(vec + i0 + 4);
-        in.v[4] = q.x;
-        in.v[5] = q.y;
-        in.v[6] = q.z;
-        in.v[7] = q.w;
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (i0 + j >= 0 && i0 + j < a.r) in.v[j] = vec[i0 + j];
-    }
-  }
-  return rs;
-}
-template <int MODE>
-__device__ __forceinline__ void pipe_finish(int d, const float* norm, int c, PipeIn& in) {
-  if (c == 0) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-      if (j < d) in.v[j] = in.primal ? (in.v[j] - norm[j]) / norm[d + j] : in.hot == j ? 1.f / norm[d + j] : 0.f;
-  }
-  if (MODE != PIPE_PRIMAL) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (8 * c + j == in.hot && in.hot >= kTcLat) in.v[j] = 1.f;
-  }
-}
-__device__ __forceinline__ bool pipe_vec4(const DecArgs& a) {
-  return (a.r & 3) == 0 && (((uintptr_t)a.latents | (uintptr_t)a.dirs) & 15u) == 0;
 }
 
 // Activations of 16 columns of a row from their pre-activations (bias included on primal rows):
@@ -1198,7 +1021,7 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
       for (int it = blockIdx.x; it < n_iter; it += gridDim.x)
         for (int j = 0; j < atoms; ++j, ++i) {
           const uint32_t slot = i % kRing, use = i / kRing;
-          if (use > 0) pipe_wait(a, &tail->abort, &tail->empty[slot], (use - 1) & 1u);
+          if (use > 0) pipe_wait(a.status, &tail->abort, &tail->empty[slot], (use - 1) & 1u);
           tc::mbar_expect_tx(&tail->full[slot], (uint32_t)kAtomBytes);
           tc::bulk_g2s(ring + slot * kAtomBytes, a.wstream + (size_t)j * kAtomBytes, kAtomBytes, &tail->full[slot]);
         }
@@ -1220,7 +1043,7 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
     // waits for the next atom of the stream, returns its ring slot
     auto take = [&]() {
       const uint32_t slot = atom % kRing;
-      pipe_wait(a, &tail->abort, &tail->full[slot], (atom / kRing) & 1u);
+      pipe_wait(a.status, &tail->abort, &tail->full[slot], (atom / kRing) & 1u);
       __syncwarp();
       ++atom;
       return slot;
@@ -1278,7 +1101,7 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
           for (int kh = 0; kh < 2; ++kh) {               // high: the small products of both atoms first
             rh[kh] = take();
             if (leader) {
-              tc::mma4_bf16_ss(tD, lo_desc + kh * kAtomDesc, ring_desc + rh[kh] * kAtomDesc, idesc);
+              tc::mma4_bf16_ss(tD, lo_desc + kh * kAtomDesc, ring_desc + rh[kh] * kAtomDesc, idesc, 1u);
               tc::mma4_bf16_ts(tD, tAm + kh * 32, ring_desc + rh[kh] * kAtomDesc, idesc, 1u);
             }
           }
@@ -1292,7 +1115,7 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
         }
         if (leader) tc::mma_commit(&tail->bar_mma[s]);
         __syncwarp();
-        pipe_wait(a, &tail->abort, &tail->bar_mma[s], mma_phase);
+        pipe_wait(a.status, &tail->abort, &tail->bar_mma[s], mma_phase);
         mma_phase ^= 1u;
         __syncwarp();
         tc::tc_fence_after();
@@ -1461,6 +1284,13 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
 // BF16 activations, or for the first layer 16 + 16 of the inputs' high and low parts.  The
 // arithmetic and its order are decoder_tc<false>'s, so the results are the same bits.
 //
+// TRAIN: whole points only (pipe_U = R floor(32 / R) rows per lane group, the other lanes idle); every
+// layer's operand is also stored as the tile image the MMA reads (128 rows x 128 BF16 in the 128-byte
+// swizzle, 32 KB): the epilogue writes it to shared memory, from where the MMA reads it and one bulk
+// copy stores it (16-byte stores of each thread's row touch 32 lines per instruction: 280 us instead
+// of 150 us for 65,536 points x 4 rows); and the primal rows' slope records per point, 16-byte
+// chunks permuted per point (stage_chunk).
+//
 // What bounds it: the epilogue, 1.7k cycles per tile and layer (the special-function unit's 16
 // exponentials a clock take 1.0k of them), and about 3k per tile for its inputs and outputs; the
 // tensor core is busy 20 % of the time.  1,048,576 primal rows: 0.297 ms (0.493 ms as two groups of
@@ -1479,13 +1309,14 @@ struct __align__(8) Bf16Tail {
   int abort;      // a wait ran out (as in decoder_tc3)
 };
 
-template <int NS, int MODE>
+template <int NS, int MODE, bool TRAIN>
 __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (tc::smem_addr(smem_raw) & 1023u)) & 1023u);
   uint8_t* wsm = smem;                                   // kMaxTC x 32 KB square layers
   uint8_t* w0s = smem + kMaxTC * kLayerBytes;            // 16 KB first-layer split image
-  float* ypart = (float*)(w0s + kLayerBytes / 2);        // [3][128][3]
+  uint8_t* images = w0s + kLayerBytes / 2;               // TRAIN: NS x 32 KB operand images
+  float* ypart = (float*)(images + (TRAIN ? NS * kLayerBytes : 0));   // [3][128][3]
   float* sb0 = ypart + 3 * 128 * 3;                      // [128]
   float* sbh = sb0 + kW;                                 // [kMaxTC][128]
   float* sWout = sbh + kMaxTC * kW;                      // [3][128]
@@ -1529,8 +1360,15 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
     const uint32_t w0_desc = tc::smem_desc_sw128_lo(tc::smem_addr(w0s));
     constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW);
     uint32_t mma_phase = 0;
-    pipe_wait(a, &tail->abort, &tail->bar_w, 0);
+    pipe_wait(a.status, &tail->abort, &tail->bar_w, 0);
     __syncwarp();
+    uint8_t* image = images + s * kLayerBytes;
+    const uint32_t image_desc = tc::smem_desc_sw128_lo(tc::smem_addr(image));
+    // TRAIN: the image of activation layer `layer` leaves for the store
+    auto store_image = [&](int layer, int tile) {
+      tc::bulk_s2g(a.astore + ((int64_t)layer * a.rows_total + (int64_t)tile * 128) * kW, image, kLayerBytes);
+    };
+    int prev = -1;   // this slot's previous tile, whose last image is not stored yet
     for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
       if (s >= NT || it * NT + s >= n_tiles) continue;
       for (int l = -1; l < a.n_tc; ++l) {
@@ -1547,19 +1385,36 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
             }
           } else {
             const uint32_t bd = w_desc + (uint32_t)l * (kLayerBytes >> 4);
-            tc::mma4_bf16_ts(tD, tA, bd, idesc, 0u);
-            tc::mma4_bf16_ts(tD, tA + 32, bd + (kAtomBytes >> 4), idesc, 1u);
+            if (TRAIN) {
+              tc::mma4_bf16_ss(tD, image_desc, bd, idesc, 0u);
+              tc::mma4_bf16_ss(tD, image_desc + (kAtomBytes >> 4), bd + (kAtomBytes >> 4), idesc, 1u);
+            } else {
+              tc::mma4_bf16_ts(tD, tA, bd, idesc, 0u);
+              tc::mma4_bf16_ts(tD, tA + 32, bd + (kAtomBytes >> 4), idesc, 1u);
+            }
           }
           tc::mma_commit(&tail->bar_mma[s]);
+          if (TRAIN && l >= 0) store_image(l, it * NT + s);
+          if (TRAIN && l < 0 && prev >= 0) store_image(a.n_tc, prev);
         }
         __syncwarp();
-        pipe_wait(a, &tail->abort, &tail->bar_mma[s], mma_phase);
+        pipe_wait(a.status, &tail->abort, &tail->bar_mma[s], mma_phase);
         mma_phase ^= 1u;
+        if (TRAIN && leader) tc::bulk_wait_read();   // the image may be rewritten
         __syncwarp();
         tc::tc_fence_after();
         tc::tc_fence_before();
         pipe_arrive(3 + s);
       }
+      prev = it * NT + s;
+    }
+    if (TRAIN && prev >= 0) {
+      pipe_sync(1 + s);
+      if (leader) {
+        store_image(a.n_tc, prev);
+        tc::bulk_wait_all();
+      }
+      __syncwarp();
     }
     // MMAs of a timed-out pass complete (bounded) before the tensor memory is freed; the weights
     // have landed (waited for above, or here after a timeout)
@@ -1595,6 +1450,7 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
     };
     auto ready = [&](int s) {
       tc::tmem_wait_st();
+      if (TRAIN) tc::fence_async_smem();
       tc::tc_fence_before();
       pipe_arrive(1 + s);
     };
@@ -1605,7 +1461,7 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
       const int tile = blockIdx.x * NT + s;
       if ((int)blockIdx.x < n_iter && s < NT && tile < n_tiles) {
         PipeIn in;
-        rows[s] = pipe_load<MODE>(a, (tile * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
+        rows[s] = pipe_load<MODE, TRAIN>(a, (tile * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
         put(s, in);
         ready(s);
       }
@@ -1620,6 +1476,7 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
           const PipeRow rs = s == 0 ? rows[0] : rows[NS - 1];
           const bool primal = rs.cls == 0;
           const float one_p = primal ? 1.0f : 0.0f;
+          const bool first_lane = TRAIN && lane < U && lane % a.R == 0;   // a point's (valid or padding) primal row
           const uint32_t ts = tbase + s * 256;
           float y[3] = {0.f, 0.f, 0.f};
           // the slot's next tile: its inputs load while the last accumulator completes
@@ -1627,7 +1484,7 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
           const int next = (it + (int)gridDim.x) * NT + s;
           const bool more = last && it + (int)gridDim.x < n_iter && next < n_tiles;
           if (more) {
-            const PipeRow nr = pipe_load<MODE>(a, (next * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
+            const PipeRow nr = pipe_load<MODE, TRAIN>(a, (next * 4 + (warp & 3)) * U, U, n_rows, lane, h, vec4, in);
             if (s == 0) rows[0] = nr;
             else rows[NS - 1] = nr;
           }
@@ -1643,7 +1500,33 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
               fma2(z[i], z[i + 1], b4.x, b4.y, one_p);
               fma2(z[i + 2], z[i + 3], b4.z, b4.w, one_p);
             }
-            pipe_activate<MODE>(z, rs);
+            if (TRAIN) {
+              // the primal rows' slope records (act_slope_record), and both activations from them
+              uint32_t rec[8];
+#pragma unroll
+              for (int i = 0; i < 16; i += 2) {
+                const float p0 = __shfl_sync(0xffffffffu, z[i], rs.psrc);
+                const float p1 = __shfl_sync(0xffffffffu, z[i + 1], rs.psrc);
+                float s0 = p0, s1 = p1;
+                mul2(s0, s1, kLog2e);
+                s0 = MODE != PIPE_IDENTITY && p0 < 0.f ? ex2_ftz(s0) : -1.f;
+                s1 = MODE != PIPE_IDENTITY && p1 < 0.f ? ex2_ftz(s1) : -1.f;
+                rec[i / 2] = pack2(s0, s1);
+                z[i] = s0 < 0.f ? z[i] : primal ? s0 - 1.0f : s0 * z[i];
+                z[i + 1] = s1 < 0.f ? z[i + 1] : primal ? s1 - 1.0f : s1 * z[i + 1];
+              }
+              if (first_lane) {
+                // the point's row of 256 bytes, its chunks permuted by its place in the tile
+                uint8_t* o = reinterpret_cast<uint8_t*>(a.dstore + ((int64_t)(l + 1) * a.points_total + rs.p) * kW);
+                const int pt = (warp & 3) * (U / a.R) + lane / a.R;
+                *reinterpret_cast<uint4*>(o + stage_chunk(pt, c0 / 8) - pt * 256) =
+                    make_uint4(rec[0], rec[1], rec[2], rec[3]);
+                *reinterpret_cast<uint4*>(o + stage_chunk(pt, c0 / 8 + 1) - pt * 256) =
+                    make_uint4(rec[4], rec[5], rec[6], rec[7]);
+              }
+            } else {
+              pipe_activate<MODE>(z, rs);
+            }
             if (last) {
               // output layer fused into the last epilogue (FP32): one chain over the part's 32 columns
 #pragma unroll
@@ -1658,21 +1541,26 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
                   y[o] = fmaf(w4.w, z[i + 3], y[o]);
                 }
               }
-            } else {
+            }
+            if (!last || TRAIN) {
               uint32_t w[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) w[j] = pack2(z[2 * j], z[2 * j + 1]);
-              tc::tmem_st8(ts + 128 + c0 / 2, w);
+              if (TRAIN) {
+                uint8_t* image = images + s * kLayerBytes;
+                *reinterpret_cast<uint4*>(image + tc::sw128_offset(rw, c0, kW)) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(image + tc::sw128_offset(rw, c0 + 8, kW)) = make_uint4(w[4], w[5], w[6], w[7]);
+              } else {
+                tc::tmem_st8(ts + 128 + c0 / 2, w);
+              }
             }
           }
           if (!last) {
             ready(s);
             continue;
           }
-          if (more) {
-            put(s, in);
-            ready(s);
-          }
+          if (more) put(s, in);
+          if (more || TRAIN) ready(s);   // TRAIN: the last image, stored by the issuer
           if (h < 3) {
 #pragma unroll
             for (int o = 0; o < 3; ++o)
@@ -1797,8 +1685,8 @@ size_t dec_smem_bytes(bool split) {
 }
 
 template <int NS>
-size_t dec_bf16_smem_bytes() {
-  return 1024 + kMaxTC * kLayerBytes + kLayerBytes / 2 + (3 * 128 * 3 + kW + kMaxTC * kW + 3 * kW + 8) * sizeof(float) +
+size_t dec_bf16_smem_bytes(bool train = false) {
+  return 1024 + kMaxTC * kLayerBytes + kLayerBytes / 2 + (train ? NS * kLayerBytes : 0) + (3 * 128 * 3 + kW + kMaxTC * kW + 3 * kW + 8) * sizeof(float) +
          sizeof(Bf16Tail);
 }
 
@@ -1810,15 +1698,25 @@ size_t dec_tc3_smem_bytes() {
 
 template <int NS, int MODE>
 cudaError_t pipe_limit() {
-  const cudaError_t e = cudaFuncSetAttribute(decoder_bf16<NS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(decoder_bf16<NS, MODE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)dec_bf16_smem_bytes<NS>());
   return e != cudaSuccess ? e
                           : cudaFuncSetAttribute(decoder_tc3<NS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)dec_tc3_smem_bytes<NS>());
 }
+template <int NS>
+cudaError_t pipe_limit_train() {
+  const cudaError_t e = cudaFuncSetAttribute(decoder_bf16<NS, PIPE_TANGENT, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)dec_bf16_smem_bytes<NS>(true));
+  return e != cudaSuccess ? e
+                          : cudaFuncSetAttribute(decoder_bf16<NS, PIPE_IDENTITY, true>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)dec_bf16_smem_bytes<NS>(true));
+}
 cudaError_t pipe_limits() {
   for (cudaError_t (*f)() : {pipe_limit<1, 0>, pipe_limit<1, 1>, pipe_limit<1, 2>, pipe_limit<1, 3>, pipe_limit<2, 0>,
-                             pipe_limit<2, 1>, pipe_limit<2, 2>, pipe_limit<2, 3>})
+                             pipe_limit<2, 1>, pipe_limit<2, 2>, pipe_limit<2, 3>, pipe_limit_train<1>, pipe_limit_train<2>})
     if (const cudaError_t e = f(); e != cudaSuccess) return e;
   return cudaSuccess;
 }
@@ -1829,7 +1727,7 @@ void pipe_launch(const DecArgs& a, bool fp32, int blocks, cudaStream_t s) {
   if (fp32)
     decoder_tc3<NS, MODE><<<blocks, tc3_threads<NS>(), dec_tc3_smem_bytes<NS>(), s>>>(a);
   else
-    decoder_bf16<NS, MODE><<<blocks, bf16_threads<NS>(), dec_bf16_smem_bytes<NS>(), s>>>(a);
+    decoder_bf16<NS, MODE, false><<<blocks, bf16_threads<NS>(), dec_bf16_smem_bytes<NS>(), s>>>(a);
 }
 // Rows in (point, kind) order, 32 (whole points) or 31 per lane group, four lane groups per tile; one
 // tile per CTA while every tile has an SM of its own (of this caller's share), else two.
@@ -2093,6 +1991,7 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
     a.dstore = extra->dstore;
     a.astore = extra->astore;
     a.rows_total = extra->rows_total;
+    a.points_total = extra->points_total;
     MPM_CHECK_ARG(!a.dstore || dec->n_tc > 0, "training stores need square hidden layers");
     MPM_CHECK_ARG(!a.dstore || !has_mixed, "training stores take no mixed rows");
     MPM_CHECK_ARG(!a.dstore || R > 1, "training stores need the tangent rows (R > 1)");
@@ -2146,6 +2045,20 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
   } else if (dec->fp32 == 0 && pipe && !a.dstore && dec->w0img) {
     // BF16 rows without partners beyond the primal, first layer on the tensor cores (r <= 28)
     pipe_launch(a, false, n * R, dec->n_sm, dec->n_sm, secants, s);
+  } else if (a.dstore && a.points_total > 0) {
+    // training on decoder_bf16: whole points per lane group
+    a.pipe_U = 32 / R * R;
+    const int tiles = (int)(a.rows_total / 128);
+    const bool one = tiles <= dec->n_sm;
+    const int blocks = one ? tiles : std::min((tiles + 1) / 2, dec->n_sm);
+    if (one && a.act == 0)
+      decoder_bf16<1, PIPE_TANGENT, true><<<blocks, bf16_threads<1>(), dec_bf16_smem_bytes<1>(true), s>>>(a);
+    else if (one)
+      decoder_bf16<1, PIPE_IDENTITY, true><<<blocks, bf16_threads<1>(), dec_bf16_smem_bytes<1>(true), s>>>(a);
+    else if (a.act == 0)
+      decoder_bf16<2, PIPE_TANGENT, true><<<blocks, bf16_threads<2>(), dec_bf16_smem_bytes<2>(true), s>>>(a);
+    else
+      decoder_bf16<2, PIPE_IDENTITY, true><<<blocks, bf16_threads<2>(), dec_bf16_smem_bytes<2>(true), s>>>(a);
   } else {
     const int64_t tiles = (n + a.Pt - 1) / a.Pt;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, dec->n_sm));
@@ -2161,12 +2074,19 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
 }  // extern "C"
 
 namespace mpmrom {
+// Whether the training forward runs on decoder_bf16 (row-major stores; else decoder_tc's
+// feature-major ones).
+bool decoder_train_pipe(const mpm_decoder* dec, int64_t rows_total) {
+  return dec->n_tc > 0 && dec->w0img != nullptr && rows_total < ((int64_t)1 << 31) - 4096;
+}
+
 // Training forward: one latent and one JVP direction per point; stores the
 // per-layer activations of every tile row and the primal rows' activation slopes.
 mpm_status decoder_launch_train(const mpm_decoder* dec, const float* X, const float* latents, const float* dirs,
                                 const int* kinds, int R, int64_t n, float* out, __nv_bfloat16* dstore,
-                                __nv_bfloat16* astore, int64_t rows_total, cudaStream_t s) {
+                                __nv_bfloat16* astore, int64_t rows_total, int64_t points_total, cudaStream_t s) {
   DecArgs extra{};
+  extra.points_total = points_total;
   extra.lat_per_point = 1;
   extra.dstore = dstore;
   extra.astore = astore;

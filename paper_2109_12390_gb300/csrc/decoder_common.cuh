@@ -70,6 +70,10 @@ struct DecArgs {
   __nv_bfloat16* dstore;
   __nv_bfloat16* astore;
   int64_t rows_total;
+  // decoder_bf16's training stores: astore [l][tile] images of 128 rows (32 KB, sw128_offset), dstore
+  // [l][point] rows of 256 bytes (stage_chunk), points_total points with the tiles' padding; 0 with
+  // decoder_tc
+  int64_t points_total;
 };
 
 __device__ __forceinline__ float elu(float z) { return z > 0.f ? z : expm1f(z); }
@@ -307,6 +311,10 @@ __device__ __forceinline__ void store_bf16x8(uint8_t* tile, int row, int col, co
   *reinterpret_cast<uint4*>(tile + tc::sw128_offset(row, col, kW)) = u;
 }
 
+
+// Byte offset of 16-byte chunk c of row `row` among rows of 256 bytes, the chunks permuted per row (a
+// warp's 16-byte accesses to one chunk of neighbouring rows fall in distinct banks).
+__device__ __forceinline__ int stage_chunk(int row, int c) { return row * 256 + ((c ^ (row & 7)) << 4); }
 
 __device__ __forceinline__ uint32_t u4_word(const uint4& v, int i) {
   return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;

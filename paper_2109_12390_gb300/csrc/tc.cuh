@@ -64,6 +64,17 @@ __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gmem_src, u
       : "memory");
 }
 
+// shared -> global, in the issuing thread's bulk group; _read waits until the groups have read their
+// shared memory, _all until they are complete.  Alignment and size as above.
+__device__ __forceinline__ void bulk_s2g(void* gmem_dst, const void* smem_src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gmem_dst), "r"(smem_addr(smem_src)),
+               "r"(bytes)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 // ------------------------------------------------------------ proxy fences
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -97,6 +108,14 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
   d |= (uint64_t)1 << 46;                            // version
   d |= (uint64_t)2 << 61;                            // SWIZZLE_128B
   return d;
+}
+
+// Transposed (outer index contiguous) operand, 128-byte swizzle: rows of K, each 64 BF16 of the outer
+// index (128 bytes, its 16-byte chunks XOR-ed with row % 8); 8-row groups 1024 bytes apart (SBO), the
+// next 64 of the outer index `lead` bytes on (LBO).
+__device__ __forceinline__ uint64_t smem_desc_sw128_mn(uint32_t saddr, uint32_t lead) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lead >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
 // Instruction descriptor of tcgen05.mma kind::f16: D = F32, A = B = BF16,
@@ -143,19 +162,20 @@ __device__ __forceinline__ void mma4_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, u
       "r"(tmem_a), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(kDescSw128Hi)
       : "memory");
 }
-__device__ __forceinline__ void mma4_bf16_ss(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
+__device__ __forceinline__ void mma4_bf16_ss(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                             uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred q;\n .reg .b64 a<4>, b<4>;\n .reg .b32 l<4>, m<4>;\n"
-      " setp.eq.b32 q, 0, 0;\n"
+      "{\n .reg .pred p, q;\n .reg .b64 a<4>, b<4>;\n .reg .b32 l<4>, m<4>;\n"
+      " setp.ne.b32 p, %5, 0;\n setp.eq.b32 q, 0, 0;\n"
       " add.u32 l1, %2, 2;\n add.u32 l2, %2, 4;\n add.u32 l3, %2, 6;\n"
       " add.u32 m1, %1, 2;\n add.u32 m2, %1, 4;\n add.u32 m3, %1, 6;\n"
       " mov.b64 b0, {%2, %4};\n mov.b64 b1, {l1, %4};\n mov.b64 b2, {l2, %4};\n mov.b64 b3, {l3, %4};\n"
       " mov.b64 a0, {%1, %4};\n mov.b64 a1, {m1, %4};\n mov.b64 a2, {m2, %4};\n mov.b64 a3, {m3, %4};\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], a0, b0, %3, q;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a0, b0, %3, p;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, q;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, q;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, q;\n}\n" ::"r"(tmem_d),
-      "r"(a_lo), "r"(b_lo), "r"(idesc), "n"(kDescSw128Hi)
+      "r"(a_lo), "r"(b_lo), "r"(idesc), "n"(kDescSw128Hi), "r"(accumulate)
       : "memory");
 }
 

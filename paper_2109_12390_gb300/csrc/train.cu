@@ -36,11 +36,13 @@
 
 #include "decoder_common.cuh"
 #include "encoder.cuh"
+#include "pipe.cuh"
 
 namespace mpmrom {
 mpm_status decoder_launch_train(const mpm_decoder* dec, const float* X, const float* latents, const float* dirs,
                                 const int* kinds, int R, int64_t n, float* out, __nv_bfloat16* dstore,
-                                __nv_bfloat16* astore, int64_t rows_total, cudaStream_t s);
+                                __nv_bfloat16* astore, int64_t rows_total, int64_t points_total, cudaStream_t s);
+bool decoder_train_pipe(const mpm_decoder* dec, int64_t rows_total);
 
 __device__ __forceinline__ uint64_t tr_splitmix(uint64_t state, uint64_t k) {
   uint64_t z = state + 0x9E3779B97F4A7C15ull * (k + 1ull);
@@ -122,7 +124,7 @@ __global__ void train_sample(Store st, Batch b, const float* latents, float dt_s
 struct BwdArgs {
   float n_norm;   // points of the whole minibatch (over all data-parallel shards)
   int d, r, n_hidden, n_tc, act, R, Pt;
-  int64_t n, rows_total;
+  int64_t n, rows_total, points_total;
   const float* W0;      // (W, d + r)
   const float* Wout;    // (d, W)
   const float* norm;
@@ -431,9 +433,363 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_tc(BwdArgs a) {
   if (warp == 0) tc::tmem_free<kW>(tmem);
 }
 
+// --------------------------------------------------------------------------
+// Backward over decoder_bf16's stores (train_bwd_pipe): the reverse sweep of train_bwd_tc with the same
+// arithmetic per row, on the alternating-tile pipeline.  A lane group of 32 rows holds whole points (R
+// consecutive lanes each), so a point's curvature terms reach its primal row by shuffles, in the order
+// of its tangent rows.  Per (tile slot, layer) the slot's 32 KB activation image and its points' slope
+// records arrive by bulk copies; a thread takes 32 columns of its row: adjoint from tensor memory (or,
+// for the last hidden layer, Wout^T ybar), and writes the new adjoint over the activation it read.
+// The image then is the MMA's operand and is stored by one bulk copy for the weight-gradient GEMM.
+// Bias gradients: the primal rows' adjoints pass through a small per-warp buffer and are summed per
+// column; output-layer gradients likewise per column and warp; both kept on chip over all tiles of
+// the CTA.
+// --------------------------------------------------------------------------
+constexpr int kBwdPipeThreads = kEpiThreads + 64;
+
+struct __align__(8) BwdPipeTail {
+  uint64_t bar_w;
+  uint64_t full[2];
+  uint64_t bar_mma[2];
+  uint64_t drain;
+  uint32_t tmem;
+  int abort;
+};
+
+size_t bwd_pipe_smem_bytes() {
+  return 1024 + kMaxTC * kLayerBytes + 2 * kLayerBytes + 2 * 32 * 256 +
+         (16 * 8 * 8 + 16 * (kMaxTC + 1) * 32 + 3 * kW) * sizeof(float) + sizeof(BwdPipeTail);
+}
+
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+__global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (tc::smem_addr(smem_raw) & 1023u)) & 1023u);
+  uint8_t* wt = smem;                                    // kMaxTC x 32 KB transposed square weights
+  uint8_t* images = wt + kMaxTC * kLayerBytes;           // [2 slots] activation, then adjoint images
+  uint8_t* slopes = images + 2 * kLayerBytes;            // [2 slots][32 points][256 B] slope records
+  float* scratch = (float*)(slopes + 2 * 32 * 256);      // [16 warps][8 primal rows][8 columns]
+  float* sbias = scratch + 16 * 8 * 8;                   // [16 warps][hidden layers][32 columns]
+  float* sWout = sbias + 16 * (kMaxTC + 1) * 32;         // [3][128]
+  BwdPipeTail* tail = (BwdPipeTail*)(sWout + 3 * kW);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int d = a.d, R = a.R;
+  const int ppg = 32 / R, U = ppg * R;                   // points and rows per lane group
+
+  if (t == 0) {
+    tc::mbar_init(&tail->bar_w, 1);
+    tc::mbar_init(&tail->full[0], 1);
+    tc::mbar_init(&tail->full[1], 1);
+    tc::mbar_init(&tail->bar_mma[0], 1);
+    tc::mbar_init(&tail->bar_mma[1], 1);
+    tc::mbar_init(&tail->drain, 2);
+    tail->abort = 0;
+    tc::fence_mbar_init();
+    tc::mbar_expect_tx(&tail->bar_w, (uint32_t)(a.n_tc * kLayerBytes));
+    for (int l = a.n_tc - 1; l >= 0; --l)
+      tc::bulk_g2s(wt + l * kLayerBytes, a.wtimg + (size_t)l * kLayerBytes, kLayerBytes, &tail->bar_w);
+  }
+  if (warp == 0) tc::tmem_alloc<512>(&tail->tmem);
+  for (int e = t; e < 16 * (kMaxTC + 1) * 32; e += kBwdPipeThreads) sbias[e] = 0.f;
+  for (int e = t; e < 3 * kW; e += kBwdPipeThreads) sWout[e] = e < d * kW ? a.Wout[e] : 0.f;
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+
+  const int n_tiles = (int)(a.rows_total / 128);
+  const int NT = n_tiles <= (int)gridDim.x ? 1 : 2;      // tiles per pass
+  const int n_iter = (n_tiles + NT - 1) / NT;
+
+  if (warp >= kEpiThreads / 32) {
+    // ---- slot s's copies and MMAs (adjoint of the layer below: z_bar W, B operand the W^T image)
+    const int s = warp - kEpiThreads / 32;
+    const bool leader = tc::elect_one();
+    const uint32_t tD = tail->tmem + (uint32_t)(s * 256);
+    uint8_t* image = images + s * kLayerBytes;
+    uint8_t* slope = slopes + s * 32 * 256;
+    const uint32_t a_desc = tc::smem_desc_sw128_lo(tc::smem_addr(image));
+    const uint32_t w_desc = tc::smem_desc_sw128_lo(tc::smem_addr(wt));
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW);
+    const uint32_t slope_bytes = (uint32_t)(4 * ppg * 256);
+    uint32_t mma_phase = 0, full_phase = 0;
+    // activations and slopes of layer l of a tile into the slot
+    auto fetch = [&](int tile, int l) {
+      tc::mbar_expect_tx(&tail->full[s], (uint32_t)kLayerBytes + slope_bytes);
+      tc::bulk_g2s(image, a.astore + ((int64_t)l * a.rows_total + (int64_t)tile * 128) * kW, kLayerBytes,
+                   &tail->full[s]);
+      tc::bulk_g2s(slope, a.dstore + ((int64_t)l * a.points_total + (int64_t)tile * 4 * ppg) * kW, slope_bytes,
+                   &tail->full[s]);
+    };
+    pipe_wait(a.status, &tail->abort, &tail->bar_w, 0);
+    __syncwarp();
+    bool first = true;
+    for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
+      const int tile = it * NT + s;
+      if (s >= NT || tile >= n_tiles) continue;
+      if (first && leader) fetch(tile, a.n_hidden - 1);
+      first = false;
+      for (int l = a.n_hidden - 1; l >= 0; --l) {
+        __syncwarp();
+        pipe_wait(a.status, &tail->abort, &tail->full[s], full_phase);
+        full_phase ^= 1u;
+        __syncwarp();
+        tc::tc_fence_after();
+        tc::tc_fence_before();
+        pipe_arrive(3 + s);                              // data and (below the last layer) adjoints are there
+        pipe_sync(1 + s);                                // the epilogue has replaced them by the new adjoints
+        tc::tc_fence_after();
+        if (l >= 1) {
+          if (leader) {
+            const uint32_t bd = w_desc + (uint32_t)(l - 1) * (kLayerBytes >> 4);
+            tc::mma4_bf16_ss(tD, a_desc, bd, idesc, 0u);
+            tc::mma4_bf16_ss(tD, a_desc + (kAtomBytes >> 4), bd + (kAtomBytes >> 4), idesc, 1u);
+            tc::mma_commit(&tail->bar_mma[s]);
+            tc::bulk_s2g(a.zbstore + ((int64_t)(l - 1) * a.rows_total + (int64_t)tile * 128) * kW, image, kLayerBytes);
+          }
+          __syncwarp();
+          pipe_wait(a.status, &tail->abort, &tail->bar_mma[s], mma_phase);
+          mma_phase ^= 1u;
+          if (leader) {
+            tc::bulk_wait_read();
+            fetch(tile, l - 1);
+          }
+        } else if (leader) {
+          const int next = (it + (int)gridDim.x) * NT + s;
+          if (it + (int)gridDim.x < n_iter && next < n_tiles) fetch(next, a.n_hidden - 1);
+        }
+      }
+    }
+    // nothing is in flight when the memory is freed: the stores, and after a timeout (bounded) the
+    // MMAs, the weights and the last fetch
+    if (leader) {
+      tc::bulk_wait_all();
+      tc::mma_commit(&tail->drain);
+    }
+    __syncwarp();
+    (void)tc::mbar_wait(&tail->drain, 0);
+    if (*(volatile int*)&tail->abort) {
+      (void)tc::mbar_wait(&tail->bar_w, 0);
+      if (!first) (void)tc::mbar_wait(&tail->full[s], full_phase ^ 1u);
+    }
+    __syncwarp();
+  } else {
+    const int h = warp >> 2, lg = warp & 3;
+    const int rw = lg * 32 + lane;                       // tile row / tensor-memory lane
+    const uint32_t tbase = tail->tmem + ((uint32_t)(lg * 32) << 16);
+    const int q = min(lane / R, ppg - 1), k = lane - (lane / R) * R;   // point within the group, row kind
+    const bool prim = lane < U && k == 0;
+    float* wscratch = scratch + warp * 64;
+    float* wbias = sbias + warp * (kMaxTC + 1) * 32;
+    double my_loss = 0.0;
+    float gwo[3] = {0.f, 0.f, 0.f}, gbo[3] = {0.f, 0.f, 0.f};
+    float yb[2][3];                                      // output adjoints of the two slots' rows
+    const float wk = k == 0 ? 1.f : k <= d ? a.lamF : a.lamv;
+
+    // output and target of the thread's row (loads only)
+    auto residual_load = [&](int tile, float (&o)[3], float (&g)[3], float& m) {
+      const int p = (tile * 4 + lg) * ppg + q;
+      const bool live = lane < U && p < a.n;
+      m = live ? 1.f : 0.f;
+      if (live && k > d) m = a.b.mask[p];
+      const float* src = a.fwd + ((int64_t)k * a.n + p) * d;
+      const float* tgt = k == 0 ? a.b.tx + (int64_t)p * d : k <= d ? a.b.tF + (int64_t)p * d * d + (k - 1) : a.b.tv + (int64_t)p * d;
+      const int step = (k >= 1 && k <= d) ? d : 1;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        o[i] = live && i < d ? src[i] : 0.f;
+        g[i] = live && i < d ? tgt[i * step] : 0.f;
+      }
+    };
+    // output adjoints and, once per row, the loss
+    auto residual = [&](const float (&o)[3], const float (&g)[3], float m, float (&y)[3]) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const float e = k > d ? m * (o[i] - g[i]) : o[i] - g[i];
+        if (h == 0 && i < d) my_loss += (double)wk * e * e;
+        y[i] = i < d ? 2.f * wk * e * a.norm[3 * d + i] / a.n_norm : 0.f;
+      }
+    };
+
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int tile = blockIdx.x * NT + s;
+      if ((int)blockIdx.x < n_iter && s < NT && tile < n_tiles) {
+        float o[3], g[3], m;
+        residual_load(tile, o, g, m);
+        residual(o, g, m, yb[s]);
+      }
+    }
+    for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
+      for (int l = a.n_hidden - 1; l >= 0; --l) {
+        const bool top = l == a.n_hidden - 1;
+#pragma unroll 1
+        for (int s = 0; s < 2; ++s) {
+          const int tile = it * NT + s;
+          if (s >= NT || tile >= n_tiles) break;
+          const uint32_t ts = tbase + s * 256;
+          uint8_t* image = images + s * kLayerBytes;
+          const uint8_t* slope = slopes + s * 32 * 256;
+          const int64_t grow = (int64_t)tile * 128 + rw;
+          const float y0 = s == 0 ? yb[0][0] : yb[1][0], y1 = s == 0 ? yb[0][1] : yb[1][1];
+          const float y2 = s == 0 ? yb[0][2] : yb[1][2];
+          // the slot's next tile: its outputs and targets load while this step waits
+          float ro[3], rg[3], rm;
+          const int next = (it + (int)gridDim.x) * NT + s;
+          const bool more = l == 0 && it + (int)gridDim.x < n_iter && next < n_tiles;
+          if (more) residual_load(next, ro, rg, rm);
+          pipe_sync(3 + s);
+          tc::tc_fence_after();
+          if (top) {
+            // output layer: dWout[i][c] += sum over the warp's rows of ybar_i a[c], column c = lane
+#pragma unroll 8
+            for (int r2 = 0; r2 < 32; ++r2) {
+              const float av = __uint_as_float(
+                  (uint32_t)*reinterpret_cast<const uint16_t*>(image + tc::sw128_offset(lg * 32 + r2, 32 * h + lane, kW)) << 16);
+              gwo[0] = fmaf(__shfl_sync(0xffffffffu, y0, r2), av, gwo[0]);
+              gwo[1] = fmaf(__shfl_sync(0xffffffffu, y1, r2), av, gwo[1]);
+              if (d == 3) gwo[2] = fmaf(__shfl_sync(0xffffffffu, y2, r2), av, gwo[2]);
+            }
+            if (prim && h == 0) {
+              gbo[0] += y0;
+              gbo[1] += y1;
+              gbo[2] += y2;
+            }
+            __syncwarp();   // every lane has read the warp's rows before they are replaced
+          }
+#pragma unroll 1
+          for (int c0 = 32 * h; c0 < 32 * h + 32; c0 += 16) {
+            float z[16];
+            if (top) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                float sacc = fmaf(sWout[c0 + i], y0, 0.f);
+                sacc = fmaf(sWout[kW + c0 + i], y1, sacc);
+                if (d == 3) sacc = fmaf(sWout[2 * kW + c0 + i], y2, sacc);
+                z[i] = sacc;
+              }
+            } else {
+              tc::tmem_ld16(ts + c0, z);
+            }
+            // slope s: act'(z) = s, or 1 where s < 0; the curvature term of a tangent row is its own
+            // activation where s >= 0; the primal row adds its point's terms in the rows' order
+            uint4* own0 = reinterpret_cast<uint4*>(image + tc::sw128_offset(rw, c0, kW));
+            uint4* own1 = reinterpret_cast<uint4*>(image + tc::sw128_offset(rw, c0 + 8, kW));
+            uint32_t sw[8], aw[8];
+            {
+              const uint4 v0 = *reinterpret_cast<const uint4*>(slope + stage_chunk(lg * ppg + q, c0 / 8));
+              const uint4 v1 = *reinterpret_cast<const uint4*>(slope + stage_chunk(lg * ppg + q, c0 / 8 + 1));
+              const uint4 u0 = *own0, u1 = *own1;
+              sw[0] = v0.x, sw[1] = v0.y, sw[2] = v0.z, sw[3] = v0.w, sw[4] = v1.x, sw[5] = v1.y, sw[6] = v1.z, sw[7] = v1.w;
+              aw[0] = u0.x, aw[1] = u0.y, aw[2] = u0.z, aw[3] = u0.w, aw[4] = u1.x, aw[5] = u1.y, aw[6] = u1.z, aw[7] = u1.w;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float sp = (i & 1) ? bf16_hi(sw[i / 2]) : bf16_lo(sw[i / 2]);
+              const float at = (i & 1) ? bf16_hi(aw[i / 2]) : bf16_lo(aw[i / 2]);
+              const float term = (sp >= 0.f ? at : 0.f) * z[i];
+              float zb = (sp < 0.f ? 1.f : sp) * z[i];
+#pragma unroll
+              for (int kk = 1; kk < kBwdMaxR; ++kk) {
+                if (kk < R) {
+                  const float o = __shfl_down_sync(0xffffffffu, term, kk);
+                  if (prim) zb += o;
+                }
+              }
+              z[i] = zb;
+            }
+            // bias gradients: the primal rows' adjoints summed per column (column lane % 8, the rows
+            // in four parts)
+#pragma unroll
+            for (int c = 0; c < 16; c += 8) {
+              __syncwarp();
+              if (prim) {
+                float4* o = reinterpret_cast<float4*>(wscratch + q * 8);
+                o[0] = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
+                o[1] = make_float4(z[c + 4], z[c + 5], z[c + 6], z[c + 7]);
+              }
+              __syncwarp();
+              float v = 0.f;
+              for (int pr = lane >> 3; pr < ppg; pr += 4) v += wscratch[pr * 8 + (lane & 7)];
+              v += __shfl_xor_sync(0xffffffffu, v, 8);
+              v += __shfl_xor_sync(0xffffffffu, v, 16);
+              if (lane < 8) wbias[l * 32 + (c0 & 31) + c + lane] += v;
+            }
+            if (l >= 1) {
+              uint32_t w[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const __nv_bfloat162 b2 = __floats2bfloat162_rn(z[2 * j], z[2 * j + 1]);
+                w[j] = *reinterpret_cast<const uint32_t*>(&b2);
+              }
+              *own0 = make_uint4(w[0], w[1], w[2], w[3]);
+              *own1 = make_uint4(w[4], w[5], w[6], w[7]);
+            } else {
+              // first-layer adjoints (FP32, row-major): four neighbouring lanes exchange their 16 columns
+              // so that each store of the warp writes 64 contiguous bytes of eight rows
+              const int j = lane & 3;
+#pragma unroll
+              for (int r4 = 0; r4 < 4; ++r4) {           // row of lane (lane & ~3) + r4: its columns 4 j ..
+                float4 v;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                  const float e0 = __shfl_sync(0xffffffffu, z[c], (lane & ~3) + r4);
+                  const float e1 = __shfl_sync(0xffffffffu, z[4 + c], (lane & ~3) + r4);
+                  const float e2 = __shfl_sync(0xffffffffu, z[8 + c], (lane & ~3) + r4);
+                  const float e3 = __shfl_sync(0xffffffffu, z[12 + c], (lane & ~3) + r4);
+                  const float e = j == 0 ? e0 : j == 1 ? e1 : j == 2 ? e2 : e3;
+                  if (c == 0) v.x = e;
+                  else if (c == 1) v.y = e;
+                  else if (c == 2) v.z = e;
+                  else v.w = e;
+                }
+                *reinterpret_cast<float4*>(a.zb0 + (grow - j + r4) * kW + c0 + 4 * j) = v;
+              }
+            }
+          }
+          tc::fence_async_smem();
+          tc::tc_fence_before();
+          pipe_arrive(1 + s);
+          if (more) {
+            float y[3];
+            residual(ro, rg, rm, y);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              if (s == 0) yb[0][i] = y[i];
+              else yb[1][i] = y[i];
+            }
+          }
+        }
+      }
+    }
+    // gradients of the output layer (column 32 h + lane) and of the biases
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (i >= d) break;
+      atomicAdd(&a.gparams[a.gWout_off + i * kW + 32 * h + lane], gwo[i]);
+      float v = gbo[i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0 && h == 0) atomicAdd(&a.gparams[a.gbout_off + i], v);
+    }
+    __syncwarp();
+    for (int l = 0; l < a.n_hidden; ++l) atomicAdd(&a.gparams[a.gb_off[l] + 32 * h + lane], wbias[l * 32 + lane]);
+    if (h == 0) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_down_sync(0xffffffffu, my_loss, o);
+      if (lane == 0) atomicAdd(a.loss, my_loss);
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_free<512>(tail->tmem);
+}
+
 // ------------------------------------------- weight gradients (split-K GEMM)
 // dW_l[out][in] = sum_rows Zbar[out][row] A[in][row]; Zbar = zbstore[l], A = astore[l]
-// (the activations entering square layer l + 1).  Grid (n_tc, splits), 128 threads.
+// (the activations entering square layer l + 1).  Grid (n_tc, splits), 128 threads. 
 __global__ void __launch_bounds__(128, 1) train_dw_gemm(const __nv_bfloat16* zbstore, const __nv_bfloat16* astore,
                                                         int64_t rows_total, int64_t k_per_split, float* gparams,
                                                         const int64_t* w_off, uint32_t* status) {
@@ -511,6 +867,95 @@ __global__ void __launch_bounds__(128, 1) train_dw_gemm(const __nv_bfloat16* zbs
   if (warp == 0) tc::tmem_free<kW>(tmem);
 }
 
+// The same over the tile images of train_bwd_pipe and decoder_bf16: 64 rows of an image are two 8 KB
+// halves of 64 features, rows of 128 bytes in the 128-byte swizzle, which is the transposed (feature
+// contiguous) operand form of the MMA, K steps of 16 rows 2 KB apart.  Blocks of 64 rows of both
+// operands (32 KB) stream through kDwStages shared-memory stages by bulk copies: thread 0 copies,
+// thread 32 issues the MMAs.  Grid (n_tc, splits), two CTAs per SM.
+constexpr int kDwStages = 3;
+constexpr int kDwStageBytes = 4 * 8192;
+size_t dw_image_smem_bytes() { return 1024 + (size_t)kDwStages * kDwStageBytes; }
+__global__ void __launch_bounds__(128, 2) train_dw_gemm_image(const __nv_bfloat16* zbstore, const __nv_bfloat16* astore,
+                                                              int64_t rows_total, int64_t k_per_split, float* gparams,
+                                                              const int64_t* w_off, uint32_t* status) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* stages = smem_raw + ((1024u - (tc::smem_addr(smem_raw) & 1023u)) & 1023u);
+  __shared__ uint64_t full[kDwStages], empty[kDwStages], done;
+  __shared__ uint32_t tslot;
+  __shared__ int abort_flag;
+  const int t = threadIdx.x, warp = t >> 5;
+  const int l = blockIdx.x;
+  const uint8_t* Z = (const uint8_t*)(zbstore + (int64_t)l * kW * rows_total);
+  const uint8_t* A = (const uint8_t*)(astore + (int64_t)l * kW * rows_total);
+  const int64_t k0 = (int64_t)blockIdx.y * k_per_split;
+  const int64_t k1 = min(rows_total, k0 + k_per_split);
+  const int n_blk = (int)((k1 - k0) / 64);                 // rows_total and k_per_split are multiples of 64
+  if (t == 0) {
+    for (int i = 0; i < kDwStages; ++i) {
+      tc::mbar_init(&full[i], 1);
+      tc::mbar_init(&empty[i], 1);
+    }
+    tc::mbar_init(&done, 1);
+    abort_flag = 0;
+    tc::fence_mbar_init();
+  }
+  if (warp == 0) tc::tmem_alloc<kW>(&tslot);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = tslot;
+  if (t == 0) {
+    for (int b = 0; b < n_blk; ++b) {
+      const int st = b % kDwStages;
+      if (b >= kDwStages) pipe_wait(status, &abort_flag, &empty[st], (uint32_t)((b / kDwStages - 1) & 1));
+      const int64_t row = k0 + 64 * (int64_t)b;
+      const int64_t at = (row >> 7) * kLayerBytes + (row & 64) * 128;   // half of 64 features: 16 KB apart
+      uint8_t* dst = stages + st * kDwStageBytes;
+      tc::mbar_expect_tx(&full[st], (uint32_t)kDwStageBytes);
+      tc::bulk_g2s(dst, Z + at, 8192, &full[st]);
+      tc::bulk_g2s(dst + 8192, Z + at + kLayerBytes / 2, 8192, &full[st]);
+      tc::bulk_g2s(dst + 16384, A + at, 8192, &full[st]);
+      tc::bulk_g2s(dst + 24576, A + at + kLayerBytes / 2, 8192, &full[st]);
+    }
+    if (*(volatile int*)&abort_flag)   // after a timeout the last copies land before the CTA exits
+      for (int b = max(0, n_blk - kDwStages); b < n_blk; ++b)
+        (void)tc::mbar_wait(&full[b % kDwStages], (uint32_t)((b / kDwStages) & 1));
+  }
+  if (t == 32) {
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW) | (1u << 15) | (1u << 16);   // both operands transposed
+    for (int b = 0; b < n_blk; ++b) {
+      const int st = b % kDwStages;
+      pipe_wait(status, &abort_flag, &full[st], (uint32_t)((b / kDwStages) & 1));
+      const uint32_t a_base = tc::smem_addr(stages + st * kDwStageBytes), b_base = a_base + 16384;
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        tc::mma_bf16(tmem, tc::smem_desc_sw128_mn(a_base + kk * 2048, 8192),
+                     tc::smem_desc_sw128_mn(b_base + kk * 2048, 8192), idesc, (b > 0 || kk > 0) ? 1u : 0u);
+      tc::mma_commit(&empty[st]);
+    }
+    tc::mma_commit(&done);
+  }
+  __syncwarp();
+  bool ok = tc::mbar_wait(&done, 0);
+  if (!ok) raise_status(status, STATUS_TIMEOUT);
+  ok = __all_sync(0xffffffffu, ok && !*(volatile int*)&abort_flag);
+  tc::tc_fence_after();
+  if (n_blk > 0 && ok) {
+    float* g = gparams + w_off[l + 1];
+    for (int ch = 0; ch < kW / 32; ++ch) {
+      float v[32];
+      tc::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + ch * 32, v);
+      float4* g4 = reinterpret_cast<float4*>(g + t * kW + ch * 32);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) atomicAdd(g4 + i, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_free<kW>(tmem);
+}
+
 // First-layer weight gradient dW0[f][j] = sum_rows zbar0[f][row] in[row][j] and the latent
 // adjoints of the primal rows (d loss / d xhat) and of the JVP rows (d loss / d u),
 // sum_f zbar0[f][row] W0[f][d + j], from one pass over zbar0.  in[row] is the layer-0 input of
@@ -523,7 +968,9 @@ __global__ void __launch_bounds__(128, 1) train_dw_gemm(const __nv_bfloat16* zbs
 constexpr int kMaxIn = 40;
 constexpr int kDw0Stride = 132;       // floats per staged feature row (128 rows + pad; float4 aligned)
 constexpr int kDw0MaxPt = 64;         // points per tile (R >= 2)
-template <int D>
+// ROWMAJOR: zbar0 is stored row-major in decoder_bf16's row order (whole points of R = D + 2 consecutive
+// rows, floor(32 / R) points per 32 rows) and staged [row][feature].
+template <int D, bool ROWMAJOR>
 __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t rows_total, Batch b, int r, int Pt,
                                                      const float* norm, const float* W0, float* gW0, float* g_lat_pt,
                                                      float* g_u_pt) {
@@ -552,7 +999,11 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
     const int64_t row0 = tile * 128;
     __syncthreads();   // the previous tile's staged values are consumed
     // zbar0 rows of the tile: warp w stages features w, w + 8, ..., one float4 per lane
-    for (int ff = warp; ff < kW; ff += 8) {
+    for (int rr = warp; ROWMAJOR && rr < 128; rr += 8) {
+      const float4 v = *reinterpret_cast<const float4*>(zb0 + (row0 + rr) * kW + 4 * lane);
+      *reinterpret_cast<float4*>(sz + rr * kDw0Stride + 4 * lane) = v;
+    }
+    for (int ff = warp; !ROWMAJOR && ff < kW; ff += 8) {
       const float4 v = *reinterpret_cast<const float4*>(zb0 + (int64_t)ff * rows_total + row0 + 4 * lane);
       *reinterpret_cast<float4*>(sz + ff * kDw0Stride + 4 * lane) = v;
     }
@@ -575,7 +1026,12 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
     // four points at a time with float4 reads of the staged adjoints where the rows allow it (a
     // quarter warp's 16-byte reads then fall in distinct banks; the scalar reads of lanes 132
     // floats apart conflict 4 ways)
-    const bool vec4 = (Pt & 3) == 0 && (q_lo & 3) == 0 && (q_hi & 3) == 0;
+    const bool vec4 = !ROWMAJOR && (Pt & 3) == 0 && (q_lo & 3) == 0 && (q_hi & 3) == 0;
+    // a point's adjoint of feature f in row kind k
+    constexpr int R = D + 2, ppg = 32 / R;
+    auto zrow = [&](int q, int k) {
+      return ROWMAJOR ? sz[((q / ppg) * 32 + (q % ppg) * R + k) * kDw0Stride + f] : zf[k * Pt + q];
+    };
     for (int q4 = q_lo; vec4 && q4 < q_hi; q4 += 4) {
       const float4 zp4 = *reinterpret_cast<const float4*>(zf + q4);
       float4 zt4[D];
@@ -617,7 +1073,7 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
       }
     }
     for (int q = q_lo; !vec4 && q < q_hi; ++q) {
-      const float zp = zf[q];                        // primal row
+      const float zp = zrow(q, 0);                   // primal row
       const float* in = sin0 + q * kMaxIn;
 #pragma unroll
       for (int j = 0; j < kMaxIn; j += 4) {
@@ -631,8 +1087,8 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
       }
 #pragma unroll
       for (int a2 = 0; a2 < D; ++a2)                 // X-tangent rows: one input each
-        acc[a2] = fmaf(zf[(1 + a2) * Pt + q], inv_range[a2], acc[a2]);
-      const float zj = zf[(D + 1) * Pt + q];         // JVP row: [0, u] (u zero-padded to 32)
+        acc[a2] = fmaf(zrow(q, 1 + a2), inv_range[a2], acc[a2]);
+      const float zj = zrow(q, D + 1);               // JVP row: [0, u] (u zero-padded to 32)
       const float* uq = su + q * 32;
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
@@ -651,11 +1107,11 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
       const int g = o % n_groups, rr = o / n_groups;
       const int q = rr % Pt, jvp = rr / Pt;
       const int64_t pnt = tile * Pt + q;
-      const int row = (jvp ? d + 1 : 0) * Pt + q;
+      const int row = ROWMAJOR ? (q / ppg) * 32 + (q % ppg) * R + (jvp ? d + 1 : 0) : (jvp ? d + 1 : 0) * Pt + q;
       float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
 #pragma unroll 8
       for (int ff = 0; ff < kW; ++ff) {
-        const float z = sz[ff * kDw0Stride + row];
+        const float z = ROWMAJOR ? sz[row * kDw0Stride + ff] : sz[ff * kDw0Stride + row];
         const float4 w = *reinterpret_cast<const float4*>(sWl + ff * 36 + 4 * g);
         v0 = fmaf(z, w.x, v0);
         v1 = fmaf(z, w.y, v1);
@@ -790,6 +1246,8 @@ struct trainer_ctx {
   double* loss = nullptr;
   uint32_t* status = nullptr;
   size_t bwd_smem = 0;
+  bool pipe = false;            // decoder_bf16's tile images, train_bwd_pipe, train_dw_gemm_image
+  int64_t points_total = 0;     // points of all tiles, padding included (tile images)
   // encoder (Section 4.1) in place of the latent table
   bool enc = false;
   EncDesc E{};
@@ -929,7 +1387,7 @@ mpm_status train_launch_step(trainer_ctx* c, cudaStream_t s, int update) {
   for (int a = 0; a < d; ++a) kinds[1 + a] = 1 + a;
   kinds[1 + d] = 1000;
   mpm_status st = decoder_launch_train(dec, c->b.X, c->b.xh, c->b.u, kinds, c->R, c->B, c->fwd, c->dstore, c->astore,
-                                       c->rows_total, s);
+                                       c->rows_total, c->points_total, s);
   if (st != MPM_OK) return st;
   BwdArgs a{};
   a.d = d;
@@ -942,6 +1400,7 @@ mpm_status train_launch_step(trainer_ctx* c, cudaStream_t s, int update) {
   a.n = c->B;
   a.n_norm = c->n_norm;
   a.rows_total = c->rows_total;
+  a.points_total = c->points_total;
   const int L = (int)dec->w_off.size();
   a.W0 = dec->params + dec->w_off[0];
   a.Wout = dec->params + dec->w_off[L - 1];
@@ -966,26 +1425,30 @@ mpm_status train_launch_step(trainer_ctx* c, cudaStream_t s, int update) {
   a.loss = c->loss;
   a.status = c->status;
   const int bw = (int)std::max<int64_t>(1, std::min<int64_t>(c->n_tiles, c->n_sm));
-  train_bwd_tc<<<bw, kBwdThreads, c->bwd_smem, s>>>(a);
+  if (c->pipe)
+    train_bwd_pipe<<<bw, kBwdPipeThreads, c->bwd_smem, s>>>(a);
+  else
+    train_bwd_tc<<<bw, kBwdThreads, c->bwd_smem, s>>>(a);
   MPM_CUDA_TRY(cudaGetLastError());
   if (dec->n_tc > 0) {
-    // four CTAs per SM (32 KB of shared memory and 128 TMEM columns each), so that four K blocks'
-    // loads are in flight per SM; the splits' partial sums meet in vector reductions
-    const int splits = std::max(1, 4 * c->n_sm / dec->n_tc);
+    // several CTAs per SM (four with 32 KB of shared memory each, two with the streamed images), so that
+    // loads of as many K blocks are in flight per SM; the splits' partial sums meet in vector reductions
+    const int splits = std::max(1, (c->pipe ? 2 : 4) * c->n_sm / dec->n_tc);
     int64_t kps = (c->rows_total + splits - 1) / splits;
     kps = (kps + 63) / 64 * 64;
     dim3 g(dec->n_tc, (unsigned)((c->rows_total + kps - 1) / kps));
-    train_dw_gemm<<<g, 128, 0, s>>>(c->zbstore, c->astore, c->rows_total, kps, c->gparams, c->d_w_off, c->status);
+    if (c->pipe)
+      train_dw_gemm_image<<<g, 128, dw_image_smem_bytes(), s>>>(c->zbstore, c->astore, c->rows_total, kps, c->gparams,
+                                                                c->d_w_off, c->status);
+    else
+      train_dw_gemm<<<g, 128, 0, s>>>(c->zbstore, c->astore, c->rows_total, kps, c->gparams, c->d_w_off, c->status);
     MPM_CUDA_TRY(cudaGetLastError());
   }
-  if (d == 2)
-    train_dw0_lat<2><<<c->n_sm * 2, 256, dw0_smem_bytes(), s>>>(c->zb0, c->rows_total, c->b, r, c->Pt, dec->norm,
-                                                               dec->params + dec->w_off[0], c->gparams + dec->w_off[0],
-                                                               c->g_lat_pt, c->g_u_pt);
-  else
-    train_dw0_lat<3><<<c->n_sm * 2, 256, dw0_smem_bytes(), s>>>(c->zb0, c->rows_total, c->b, r, c->Pt, dec->norm,
-                                                               dec->params + dec->w_off[0], c->gparams + dec->w_off[0],
-                                                               c->g_lat_pt, c->g_u_pt);
+  auto* dw0 = d == 2 ? (c->pipe ? train_dw0_lat<2, true> : train_dw0_lat<2, false>)
+                     : (c->pipe ? train_dw0_lat<3, true> : train_dw0_lat<3, false>);
+  dw0<<<c->n_sm * 2, 256, dw0_smem_bytes(), s>>>(c->zb0, c->rows_total, c->b, r, c->Pt, dec->norm,
+                                                 dec->params + dec->w_off[0], c->gparams + dec->w_off[0], c->g_lat_pt,
+                                                 c->g_u_pt);
   MPM_CUDA_TRY(cudaGetLastError());
   train_lat_scatter<<<blocks, 256, 0, s>>>(c->b, r, c->g_lat_pt, c->g_u_pt, c->cfg.dt_snap, c->g_lat);
   MPM_CUDA_TRY(cudaGetLastError());
@@ -1117,12 +1580,17 @@ mpm_status trainer_create(mpm_decoder* dec, const train_config* cfg, const snaps
   c->d = dec->d;
   c->r = dec->r;
   c->R = c->d + 2;
-  c->Pt = 128 / c->R;
+  // whole points of R rows per 32 rows (decoder_bf16's order), or per 128 rows where that kernel
+  // does not take the decoder (r > 28)
+  c->Pt = 4 * (32 / c->R);
+  c->pipe = decoder_train_pipe(dec, ((int64_t)cfg->batch + c->Pt - 1) / c->Pt * 128);
+  if (!c->pipe) c->Pt = 128 / c->R;
   c->B = cfg->batch;
   c->i_offset = (int64_t)cfg->shard_index * cfg->batch;
   c->n_norm = (float)((double)cfg->batch * std::max(1, cfg->shard_count));
   c->n_tiles = (c->B + c->Pt - 1) / c->Pt;
   c->rows_total = c->n_tiles * 128;
+  c->points_total = c->pipe ? c->n_tiles * c->Pt : 0;
   c->n_snap = sd->n_snap;
   int devn = 0;
   cudaGetDevice(&devn);
@@ -1234,7 +1702,8 @@ mpm_status trainer_create(mpm_decoder* dec, const train_config* cfg, const snaps
   // activation stores
   const size_t rows = (size_t)c->rows_total;
   if ((st = talloc(&c->fwd, (size_t)c->R * B * d)) != MPM_OK) return st;
-  if ((st = talloc(&c->dstore, (size_t)dec->n_hidden * kW * rows)) != MPM_OK) return st;
+  if ((st = talloc(&c->dstore, (size_t)dec->n_hidden * kW * (c->pipe ? (size_t)c->points_total : rows))) != MPM_OK)
+    return st;
   if ((st = talloc(&c->astore, (size_t)dec->n_hidden * kW * rows)) != MPM_OK) return st;
   if ((st = talloc(&c->zbstore, (size_t)dec->n_tc * kW * rows)) != MPM_OK) return st;
   if ((st = talloc(&c->zb0, (size_t)kW * rows)) != MPM_OK) return st;
@@ -1260,8 +1729,14 @@ mpm_status trainer_create(mpm_decoder* dec, const train_config* cfg, const snaps
   c->bwd_smem = 1024 + kMaxTC * kLayerBytes + kLayerBytes + (size_t)2 * kExchRows * kChunkStride * 4 +
                 2 * 64 * 128 * 2 + 128 * 3 * 4 + kW * 4 + sizeof(DecSmemTail);
   MPM_CUDA_TRY(cudaFuncSetAttribute(train_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->bwd_smem));
-  MPM_CUDA_TRY(cudaFuncSetAttribute(train_dw0_lat<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw0_smem_bytes()));
-  MPM_CUDA_TRY(cudaFuncSetAttribute(train_dw0_lat<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw0_smem_bytes()));
+  if (c->pipe) {
+    c->bwd_smem = bwd_pipe_smem_bytes();
+    MPM_CUDA_TRY(cudaFuncSetAttribute(train_bwd_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->bwd_smem));
+    MPM_CUDA_TRY(cudaFuncSetAttribute(train_dw_gemm_image, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)dw_image_smem_bytes()));
+  }
+  for (auto* f : {train_dw0_lat<2, true>, train_dw0_lat<2, false>, train_dw0_lat<3, true>, train_dw0_lat<3, false>})
+    MPM_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw0_smem_bytes()));
   train_pack_transposed<<<std::max(1, dec->n_tc * 64), 256>>>(dec->params, c->d_w_off, dec->n_tc, c->wtimg);
   MPM_CUDA_TRY(cudaGetLastError());
   MPM_CUDA_TRY(cudaDeviceSynchronize());
