@@ -1455,6 +1455,8 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
       pipe_arrive(1 + s);
     };
 
+    const int pt = TRAIN ? (warp & 3) * (U / a.R) + lane / a.R : 0;   // the row's point within the tile
+    const bool pt_lane = TRAIN && lane < U && lane % a.R == 0;        // a point's (valid or padding) primal row
     PipeRow rows[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
@@ -1476,7 +1478,6 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
           const PipeRow rs = s == 0 ? rows[0] : rows[NS - 1];
           const bool primal = rs.cls == 0;
           const float one_p = primal ? 1.0f : 0.0f;
-          const bool first_lane = TRAIN && lane < U && lane % a.R == 0;   // a point's (valid or padding) primal row
           const uint32_t ts = tbase + s * 256;
           float y[3] = {0.f, 0.f, 0.f};
           // the slot's next tile: its inputs load while the last accumulator completes
@@ -1503,22 +1504,26 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
             if (TRAIN) {
               // the primal rows' slope records (act_slope_record), and both activations from them
               uint32_t rec[8];
+              const float neg_c = primal ? -1.0f : 0.0f;
+              const uint32_t keep = primal ? 0u : 0xffffffffu, one = primal ? 0x3f800000u : 0u;
 #pragma unroll
               for (int i = 0; i < 16; i += 2) {
                 const float p0 = __shfl_sync(0xffffffffu, z[i], rs.psrc);
                 const float p1 = __shfl_sync(0xffffffffu, z[i + 1], rs.psrc);
                 float s0 = p0, s1 = p1;
                 mul2(s0, s1, kLog2e);
-                s0 = MODE != PIPE_IDENTITY && p0 < 0.f ? ex2_ftz(s0) : -1.f;
-                s1 = MODE != PIPE_IDENTITY && p1 < 0.f ? ex2_ftz(s1) : -1.f;
-                rec[i / 2] = pack2(s0, s1);
-                z[i] = s0 < 0.f ? z[i] : primal ? s0 - 1.0f : s0 * z[i];
-                z[i + 1] = s1 < 0.f ? z[i + 1] : primal ? s1 - 1.0f : s1 * z[i + 1];
+                s0 = ex2_ftz(s0);
+                s1 = ex2_ftz(s1);
+                const bool lin0 = MODE == PIPE_IDENTITY || !(p0 < 0.f), lin1 = MODE == PIPE_IDENTITY || !(p1 < 0.f);
+                rec[i / 2] = pack2(lin0 ? -1.f : s0, lin1 ? -1.f : s1);
+                s0 = fmaf(s0, __uint_as_float((__float_as_uint(z[i]) & keep) | one), neg_c);
+                s1 = fmaf(s1, __uint_as_float((__float_as_uint(z[i + 1]) & keep) | one), neg_c);
+                z[i] = lin0 ? z[i] : s0;
+                z[i + 1] = lin1 ? z[i + 1] : s1;
               }
-              if (first_lane) {
+              if (pt_lane) {
                 // the point's row of 256 bytes, its chunks permuted by its place in the tile
                 uint8_t* o = reinterpret_cast<uint8_t*>(a.dstore + ((int64_t)(l + 1) * a.points_total + rs.p) * kW);
-                const int pt = (warp & 3) * (U / a.R) + lane / a.R;
                 *reinterpret_cast<uint4*>(o + stage_chunk(pt, c0 / 8) - pt * 256) =
                     make_uint4(rec[0], rec[1], rec[2], rec[3]);
                 *reinterpret_cast<uint4*>(o + stage_chunk(pt, c0 / 8 + 1) - pt * 256) =

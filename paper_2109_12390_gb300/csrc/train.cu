@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_tc(BwdArgs a) {
 // Backward over decoder_bf16's stores (train_bwd_pipe): the reverse sweep of train_bwd_tc with the same
 // arithmetic per row, on the alternating-tile pipeline.  A lane group of 32 rows holds whole points (R
 // consecutive lanes each), so a point's curvature terms reach its primal row by shuffles, in the order
-// of its tangent rows.  Per (tile slot, layer) the slot's 32 KB activation image and its points' slope
+// of its tangent rows (pairwise).  Per (tile slot, layer) the slot's 32 KB activation image and its points' slope
 // records arrive by bulk copies; a thread takes 32 columns of its row: adjoint from tensor memory (or,
 // for the last hidden layer, Wout^T ybar), and writes the new adjoint over the activation it read.
 // The image then is the MMA's operand and is stored by one bulk copy for the weight-gradient GEMM.
@@ -464,6 +464,7 @@ size_t bwd_pipe_smem_bytes() {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
+template <int D>
 __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (tc::smem_addr(smem_raw) & 1023u)) & 1023u);
@@ -475,8 +476,8 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
   float* sWout = sbias + 16 * (kMaxTC + 1) * 32;         // [3][128]
   BwdPipeTail* tail = (BwdPipeTail*)(sWout + 3 * kW);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int d = a.d, R = a.R;
-  const int ppg = 32 / R, U = ppg * R;                   // points and rows per lane group
+  constexpr int d = D, R = D + 2;
+  constexpr int ppg = 32 / R, U = ppg * R;               // points and rows per lane group
 
   if (t == 0) {
     tc::mbar_init(&tail->bar_w, 1);
@@ -673,7 +674,7 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
               tc::tmem_ld16(ts + c0, z);
             }
             // slope s: act'(z) = s, or 1 where s < 0; the curvature term of a tangent row is its own
-            // activation where s >= 0; the primal row adds its point's terms in the rows' order
+            // activation where s >= 0; the primal row adds its point's terms
             uint4* own0 = reinterpret_cast<uint4*>(image + tc::sw128_offset(rw, c0, kW));
             uint4* own1 = reinterpret_cast<uint4*>(image + tc::sw128_offset(rw, c0 + 8, kW));
             uint32_t sw[8], aw[8];
@@ -688,16 +689,13 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
             for (int i = 0; i < 16; ++i) {
               const float sp = (i & 1) ? bf16_hi(sw[i / 2]) : bf16_lo(sw[i / 2]);
               const float at = (i & 1) ? bf16_hi(aw[i / 2]) : bf16_lo(aw[i / 2]);
-              const float term = (sp >= 0.f ? at : 0.f) * z[i];
-              float zb = (sp < 0.f ? 1.f : sp) * z[i];
-#pragma unroll
-              for (int kk = 1; kk < kBwdMaxR; ++kk) {
-                if (kk < R) {
-                  const float o = __shfl_down_sync(0xffffffffu, term, kk);
-                  if (prim) zb += o;
-                }
-              }
-              z[i] = zb;
+              const float zb = (sp < 0.f ? 1.f : sp) * z[i];
+              const float term = prim ? zb : (sp >= 0.f ? at : 0.f) * z[i];
+              // (primal + first tangent) + (second + third), and with R = 5 the fourth
+              float sum = term + __shfl_down_sync(0xffffffffu, term, 1);
+              sum += __shfl_down_sync(0xffffffffu, sum, 2);
+              if (R == 5) sum += __shfl_down_sync(0xffffffffu, term, 4);
+              z[i] = prim ? sum : zb;
             }
             // bias gradients: the primal rows' adjoints summed per column (column lane % 8, the rows
             // in four parts)
@@ -711,7 +709,9 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
               }
               __syncwarp();
               float v = 0.f;
-              for (int pr = lane >> 3; pr < ppg; pr += 4) v += wscratch[pr * 8 + (lane & 7)];
+#pragma unroll
+              for (int pr = 0; pr < ppg; pr += 4)
+                if (pr + 4 <= ppg || pr + (lane >> 3) < ppg) v += wscratch[(pr + (lane >> 3)) * 8 + (lane & 7)];
               v += __shfl_xor_sync(0xffffffffu, v, 8);
               v += __shfl_xor_sync(0xffffffffu, v, 16);
               if (lane < 8) wbias[l * 32 + (c0 & 31) + c + lane] += v;
@@ -729,21 +729,25 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
               // first-layer adjoints (FP32, row-major): four neighbouring lanes exchange their 16 columns
               // so that each store of the warp writes 64 contiguous bytes of eight rows
               const int j = lane & 3;
+              float4 got[4];                             // after round x: columns 4 j .. of row j ^ x
 #pragma unroll
-              for (int r4 = 0; r4 < 4; ++r4) {           // row of lane (lane & ~3) + r4: its columns 4 j ..
-                float4 v;
+              for (int x = 0; x < 4; ++x) {
+                float g4[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                  const float e0 = __shfl_sync(0xffffffffu, z[c], (lane & ~3) + r4);
-                  const float e1 = __shfl_sync(0xffffffffu, z[4 + c], (lane & ~3) + r4);
-                  const float e2 = __shfl_sync(0xffffffffu, z[8 + c], (lane & ~3) + r4);
-                  const float e3 = __shfl_sync(0xffffffffu, z[12 + c], (lane & ~3) + r4);
-                  const float e = j == 0 ? e0 : j == 1 ? e1 : j == 2 ? e2 : e3;
-                  if (c == 0) v.x = e;
-                  else if (c == 1) v.y = e;
-                  else if (c == 2) v.z = e;
-                  else v.w = e;
+                  const int p = j ^ x;
+                  const float v = p == 0 ? z[c] : p == 1 ? z[4 + c] : p == 2 ? z[8 + c] : z[12 + c];
+                  g4[c] = x == 0 ? v : __shfl_xor_sync(0xffffffffu, v, x);
                 }
+                got[x] = make_float4(g4[0], g4[1], g4[2], g4[3]);
+              }
+#pragma unroll
+              for (int r4 = 0; r4 < 4; ++r4) {
+                const int x = j ^ r4;
+                float4 v = got[0];
+                if (x == 1) v = got[1];
+                if (x == 2) v = got[2];
+                if (x == 3) v = got[3];
                 *reinterpret_cast<float4*>(a.zb0 + (grow - j + r4) * kW + c0 + 4 * j) = v;
               }
             }
@@ -1426,7 +1430,7 @@ mpm_status train_launch_step(trainer_ctx* c, cudaStream_t s, int update) {
   a.status = c->status;
   const int bw = (int)std::max<int64_t>(1, std::min<int64_t>(c->n_tiles, c->n_sm));
   if (c->pipe)
-    train_bwd_pipe<<<bw, kBwdPipeThreads, c->bwd_smem, s>>>(a);
+    (d == 2 ? train_bwd_pipe<2> : train_bwd_pipe<3>)<<<bw, kBwdPipeThreads, c->bwd_smem, s>>>(a);
   else
     train_bwd_tc<<<bw, kBwdThreads, c->bwd_smem, s>>>(a);
   MPM_CUDA_TRY(cudaGetLastError());
@@ -1731,7 +1735,8 @@ mpm_status trainer_create(mpm_decoder* dec, const train_config* cfg, const snaps
   MPM_CUDA_TRY(cudaFuncSetAttribute(train_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->bwd_smem));
   if (c->pipe) {
     c->bwd_smem = bwd_pipe_smem_bytes();
-    MPM_CUDA_TRY(cudaFuncSetAttribute(train_bwd_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->bwd_smem));
+    for (auto* f : {train_bwd_pipe<2>, train_bwd_pipe<3>})
+      MPM_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->bwd_smem));
     MPM_CUDA_TRY(cudaFuncSetAttribute(train_dw_gemm_image, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)dw_image_smem_bytes()));
   }
