@@ -15,7 +15,7 @@
 //              state; grid[1-g] is zero except for blocks flagged in touched.
 //
 // One step = three kernels, captured in a CUDA graph by the caller if wanted:
-//   mpm_g2p2g      per work item (<= 256 particles of one grid block): load
+//   mpm_g2p2g      per work item (<= 512 particles of one grid block): load
 //                  the block's node tile of grid[g], apply the grid update of
 //                  Algorithm 1 (v = p/m + dt g, walls) while loading, gather to
 //                  the particles (grid-to-particle + advection), write the new
@@ -43,15 +43,24 @@
 
 namespace mpmrom {
 
-constexpr int kChunk = 256;           // threads per CTA of the fused kernel
-constexpr int kSlots = 2;             // particles per thread
-constexpr int kItem = kSlots * kChunk; // particles per work item at most
+// The fused kernel takes up to kItem particles per work item, kItem / CH per thread, in CTAs of CH
+// threads.  3D: grid blocks of 4^3 cells at 8 particles per cell, 512 = 256 x 2.  2D: blocks of 8^2
+// cells at 4 per cell hold about 256 particles; large contexts take them in CTAs of 128 threads, so
+// that twice as many items are in flight per SM (an item's phases are separated by barriers and
+// dependent loads): 1.03 M particles in 16 bodies 854 -> 744 us for 10 steps with the state's load and
+// read.  Small ones (less than one such block per SM) keep 256 threads, whose items have the lower
+// latency: 4096 particles 10.9 against 12.0 us per step.
+constexpr int kItem = 512;
+constexpr int kItemMin = 128;         // smallest bound of a work item (small contexts)
 
 // Dynamic shared memory of the fused kernel: per slot its P2G record (2 D + D^2 floats), its
 // position in cell order, its cell and its rank within the cell.
 template <int D>
 constexpr int fused_dyn_smem() { return kItem * ((2 * D + D * D) * 4 + 3 * 2); }
 static_assert(fused_dyn_smem<3>() <= 48 * 1024, "the fused kernel launches without raising its shared-memory limit");
+
+// Bits per axis of a work item's block coordinates.
+template <int D> constexpr int kCoordBits = D == 2 ? 15 : 10;
 
 template <int D> struct Blk;
 template <> struct Blk<2> { static constexpr int B = 8; };
@@ -257,8 +266,8 @@ __device__ __forceinline__ void count_key_aggregated(int key, int32_t* counts) {
 // The fused step kernel.  FIRST = true runs only the particle-to-grid half
 // (the transfer of a freshly loaded state).
 // --------------------------------------------------------------------------
-template <int D, int MATERIAL, int TRANSFER, bool FIRST, int POLAR>
-__global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView src, StateView dst,
+template <int D, int MATERIAL, int TRANSFER, bool FIRST, int POLAR, int CH>
+__global__ void __launch_bounds__(CH, 768 / CH) mpm_g2p2g(DevParams p, StateView src, StateView dst,
                                                         const int32_t* __restrict__ perm,
                                                         const int4* __restrict__ work, const int32_t* n_work,
                                                         const float4* __restrict__ grid_cur, float4* grid_nxt,
@@ -290,21 +299,16 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_tmask = 0u;
   for (int w = blockIdx.x; w < nw; w += gridDim.x) {
-    const int4 item = work[w];  // {key, start, count, -}
-    const int key = item.x;
-    const int inst = key / p.nblk;
-    int bk = key - inst * p.nblk;
+    const int4 item = work[w];  // {instance, start, count, block coordinates}
+    const int inst = item.x;
     int b0[D];
 #pragma unroll
-    for (int a = D - 1; a >= 0; --a) {
-      b0[a] = (bk % p.nb) * B;
-      bk /= p.nb;
-    }
+    for (int a = 0; a < D; ++a) b0[a] = ((item.w >> (kCoordBits<D> * a)) & ((1 << kCoordBits<D>) - 1)) * B;
     const float2 ml = p.mu_lam[inst];
     int tile_lo[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) tile_lo[a] = b0[a] - 1;
-    // kSlots particles per thread: slots threadIdx.x + sl kChunk of the item.  The first slot's
+    // kItem / CH particles per thread: slots threadIdx.x + sl CH of the item.  The first slot's
     // gather (binned order -> state) is issued before the node tile, so that its two dependent HBM
     // latencies overlap the tile's; the other slots' lines are fetched into L2.
     int s_src = 0, pid = 0;
@@ -318,9 +322,9 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
       pid = src.id[s_src];
     }
 #pragma unroll
-    for (int sl = 1; sl < kSlots; ++sl) {
-      if (threadIdx.x + sl * kChunk < item.z)
-        prefetch_state<D>(src, perm[item.y + threadIdx.x + sl * kChunk], P);
+    for (int sl = 1; sl < kItem / CH; ++sl) {
+      if (threadIdx.x + sl * CH < item.z)
+        prefetch_state<D>(src, perm[item.y + threadIdx.x + sl * CH], P);
     }
     // grid-to-particle tile with the grid update of Algorithm 1 applied on load
     if (!FIRST) {
@@ -344,8 +348,8 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
 
     if (threadIdx.x == 0) s_tmask = 0u;   // every thread read the previous item's mask before the barrier
 #pragma unroll 1
-    for (int sl = 0; sl < kSlots; ++sl) {
-    const int slot = threadIdx.x + sl * kChunk;
+    for (int sl = 0; sl < kItem / CH; ++sl) {
+    const int slot = threadIdx.x + sl * CH;
     const int j = item.y + slot;
     const bool active = slot < item.z;
     if (sl > 0 && active) {
@@ -361,7 +365,8 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
     float rec[PD];
     if (active) {
       const int s = s_src;
-      float v[D], C[DD];
+      float v[D], C[DD], R0[DD];
+      bool kept = false;
       if (FIRST) {
 #pragma unroll
         for (int a = 0; a < D; ++a) v[a] = src.base[(size_t)(D + a) * P + s];
@@ -481,7 +486,7 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
           }
 #pragma unroll
         for (int i = 0; i < DD; ++i) F[i] = Fn[i];
-        if (MATERIAL == MPM_FIXED_COROTATED_PLASTIC) plastic_return<D>(F, p.sv_lo, p.sv_hi);
+        if (MATERIAL == MPM_FIXED_COROTATED_PLASTIC) kept = plastic_return<D>(F, p.sv_lo, p.sv_hi, R0);
         if (p.kin_group) {
           // kinematic (Dirichlet) particle: prescribed velocity, no affine velocity; F follows the grid
           const int kg = p.kin_group[pid];
@@ -525,7 +530,11 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
       }
       // particle-to-grid record of the (new) state
       float tau[DD];
-      kirchhoff<D, MATERIAL, POLAR>(F, ml.x, ml.y, tau);
+      // where the return mapping left F, the rotation is the one it found
+      if (MATERIAL == MPM_FIXED_COROTATED_PLASTIC)
+        kirchhoff<D, MATERIAL, POLAR>(F, ml.x, ml.y, tau, kPolarSettled, R0, kept);
+      else
+        kirchhoff<D, MATERIAL, POLAR>(F, ml.x, ml.y, tau, kPolarConverged);
       int nb[D];
       bool out_of_grid = false, in_cells = true;
       float fx[D];
@@ -625,8 +634,8 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
     __syncthreads();
     // counting sort of the slots by cell
 #pragma unroll
-    for (int sl = 0; sl < kSlots; ++sl) {
-      const int slot = threadIdx.x + sl * kChunk;
+    for (int sl = 0; sl < kItem / CH; ++sl) {
+      const int slot = threadIdx.x + sl * CH;
       if (slot < item.z) {
         const int lc = s_lc[slot];
         if (lc >= 0) s_idx[s_off[lc] + s_rank[slot]] = (short)slot;
@@ -682,14 +691,15 @@ __global__ void __launch_bounds__(kChunk, 3) mpm_g2p2g(DevParams p, StateView sr
             const float w01 = (D == 3) ? w0 * wmid[o1] : w0;
             float c1[D];
 #pragma unroll
-            for (int a = 0; a < D; ++a) c1[a] = (D == 3) ? fmaf(A[a * D + 1], (float)o1 * p.dx, c0[a]) : c0[a];
+            for (int a = 0; a < D; ++a) c1[a] = (D == 3 && o1 > 0) ? fmaf(A[a * D + 1], (float)o1 * p.dx, c0[a]) : c0[a];
 #pragma unroll
             for (int kk = 0; kk < 3; ++kk) {
               const float wt = w01 * wlast[kk];
               am[o1][kk] = fmaf(wt, p.mass, am[o1][kk]);
 #pragma unroll
               for (int a = 0; a < D; ++a)
-                ap[o1][kk][a] = fmaf(wt, fmaf(A[a * D + D - 1], (float)kk * p.dx, c1[a]), ap[o1][kk][a]);
+                ap[o1][kk][a] =
+                    fmaf(wt, kk > 0 ? fmaf(A[a * D + D - 1], (float)kk * p.dx, c1[a]) : c1[a], ap[o1][kk][a]);
             }
           }
         } else {
@@ -767,16 +777,35 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// The nw work items of key k (c particles from `off` in the binned order, split evenly) into
+// work[woff ..]: {instance, start, count, block coordinates}.
+__device__ __forceinline__ void append_items(int k, int off, int c, int nw, int woff, int4* work, int max_work, int nb,
+                                             int nblk, int dim) {
+  if (nw == 0) return;
+  const int inst = k / nblk;
+  int bk = k - inst * nblk, packed = 0;
+  const int bits = dim == 2 ? kCoordBits<2> : kCoordBits<3>;
+  for (int a = dim - 1; a >= 0; --a) {
+    packed |= (bk % nb) << (bits * a);
+    bk /= nb;
+  }
+  for (int q = 0; q < nw; ++q) {
+    const int lo = (int)((long long)q * c / nw), hi = (int)((long long)(q + 1) * c / nw);
+    if (woff + q < max_work) work[woff + q] = make_int4(inst, off + lo, hi - lo, packed);
+  }
+}
+
 __global__ void __launch_bounds__(kScanTile) mpm_scan(int n_keys, int P, int32_t* counts, int32_t* offsets,
-                                                       int32_t* cursor, int4* work, int32_t* n_work, int max_work,
-                                                       unsigned long long* tile_state, uint32_t* status) {
+                                                       int32_t* cursor, int4* work, int32_t* n_work, int max_work, int item_cap,
+                                                       int nb, int nblk, int dim, unsigned long long* tile_state,
+                                                       uint32_t* status) {
   __shared__ int s_a[32], s_b[32];
   __shared__ long long s_prefix[2];
   pdl_enter();
   const int tile = blockIdx.x;
   const int k = tile * kScanTile + threadIdx.x;
   const int c = k < n_keys ? counts[k] : 0;
-  const int nw = (c + kItem - 1) / kItem;
+  const int nw = (c + item_cap - 1) / item_cap;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int a = c, b = nw;
 #pragma unroll
@@ -847,15 +876,10 @@ __global__ void __launch_bounds__(kScanTile) mpm_scan(int n_keys, int P, int32_t
   }
   __syncthreads();
   const int off = (int)s_prefix[0] + a - c + (warp > 0 ? s_a[warp - 1] : 0);
-  int woff = (int)s_prefix[1] + b - nw + (warp > 0 ? s_b[warp - 1] : 0);
+  const int woff = (int)s_prefix[1] + b - nw + (warp > 0 ? s_b[warp - 1] : 0);
   if (k < n_keys) {
     offsets[k] = off;
-    for (int q = 0; q < nw; ++q) {
-      // nw items of near-equal size (at most kItem particles each)
-      const int lo = (int)((long long)q * c / nw), hi = (int)((long long)(q + 1) * c / nw);
-      if (woff < max_work) work[woff] = make_int4(k, off + lo, hi - lo, 0);
-      ++woff;
-    }
+    append_items(k, off, c, nw, woff, work, max_work, nb, nblk, dim);
     counts[k] = 0;
     cursor[k] = 0;
   }
@@ -1070,6 +1094,8 @@ struct mpm_ctx {
   std::vector<float> E, nu;
   std::vector<int64_t> offs;
   int n_sm = 0, fused_grid = 0, max_work = 0;
+  int item_cap = kItem;         // particles per work item at most
+  bool narrow = false;          // 2D: CTAs of 128 threads
   // device
   float* state[2] = {nullptr, nullptr};
   int32_t* id[2] = {nullptr, nullptr};
@@ -1123,14 +1149,14 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, int block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kern, (KArgs)args...);
 }
 
-template <int D, int MAT, int TR, bool FIRST, int POLAR>
+template <int D, int MAT, int TR, bool FIRST, int POLAR, int CH>
 mpm_status launch_fused_t(mpm_ctx* c, cudaStream_t s) {
   StateView src{c->state[c->cur], c->id[c->cur]};
   StateView dst{c->state[1 - c->cur], c->id[1 - c->cur]};
   float4* gcur = c->grid[c->g];
   float4* gnxt = FIRST ? c->grid[c->g] : c->grid[1 - c->g];
   uint8_t* tn = FIRST ? c->touched[c->g] : c->touched[1 - c->g];
-  MPM_CUDA_TRY(launch_pdl(mpm_g2p2g<D, MAT, TR, FIRST, POLAR>, c->fused_grid, kChunk, fused_dyn_smem<D>(), s, c->dp,
+  MPM_CUDA_TRY(launch_pdl(mpm_g2p2g<D, MAT, TR, FIRST, POLAR, CH>, c->fused_grid, CH, fused_dyn_smem<D>(), s, c->dp,
                           src, dst,
                           (const int32_t*)c->perm, (const int4*)c->work, (const int32_t*)c->n_work,
                           (const float4*)gcur, gnxt, tn, c->key, c->counts, c->status));
@@ -1142,13 +1168,16 @@ mpm_status launch_fused(mpm_ctx* c, cudaStream_t s) {
   const int D = c->D, M = c->material, T = c->transfer;
   // the polar variant matters for the 3D fixed-corotated material only
 #define CASE(d, m, t)                                                                       \
-  if (D == d && M == m && T == t) return launch_fused_t<d, m, t, FIRST, POLAR_EFT>(c, s);
+  if (D == d && M == m && T == t)                                                           \
+    return c->narrow ? launch_fused_t<d, m, t, FIRST, POLAR_EFT, d == 2 ? 128 : 256>(c, s)  \
+                     : launch_fused_t<d, m, t, FIRST, POLAR_EFT, 256>(c, s);
   CASE(2, 0, 0) CASE(2, 0, 1) CASE(2, 1, 0) CASE(2, 1, 1) CASE(2, 2, 0) CASE(2, 2, 1)
   CASE(3, 0, 0) CASE(3, 0, 1)
 #undef CASE
 #define CASE3(m, t)                                                                                              \
   if (D == 3 && M == m && T == t)                                                                               \
-    return c->polar_eft ? launch_fused_t<3, m, t, FIRST, POLAR_EFT>(c, s) : launch_fused_t<3, m, t, FIRST, POLAR_FP64>(c, s);
+    return c->polar_eft ? launch_fused_t<3, m, t, FIRST, POLAR_EFT, 256>(c, s)                                   \
+                        : launch_fused_t<3, m, t, FIRST, POLAR_FP64, 256>(c, s);
   CASE3(1, 0) CASE3(1, 1) CASE3(2, 0) CASE3(2, 1)
 #undef CASE3
   return set_error(MPM_EINVAL, "unsupported (dim, material, transfer)");
@@ -1156,7 +1185,8 @@ mpm_status launch_fused(mpm_ctx* c, cudaStream_t s) {
 
 mpm_status launch_scan_permute(mpm_ctx* c, cudaStream_t s, bool clear_consumed) {
   MPM_CUDA_TRY(launch_pdl(mpm_scan, c->n_scan_tiles, kScanTile, 0, s, c->n_keys, c->P, c->counts, c->offsets, c->cursor,
-                          c->work, c->n_work, c->max_work, c->tile_state, c->status));
+                          c->work, c->n_work, c->max_work, c->item_cap, c->nb, c->nblk, c->D, c->tile_state,
+                          c->status));
   int blocks = std::max(1, std::min(ceil_div(c->P, 256), c->n_sm * 8));
   float4* gclr = clear_consumed ? c->grid[c->g] : nullptr;
   uint8_t* tclr = clear_consumed ? c->touched[c->g] : nullptr;
@@ -1272,7 +1302,13 @@ mpm_status mpm_init(const mpm_config* cfg, mpm_ctx** out) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
-  c->max_work = ceil_div(c->P, kItem) + std::min(c->n_keys, c->P) + 1;
+  // work items small enough that every SM has about two (an item's latency, not its work, sets the
+  // time of a small context): 84,915 plastic particles in 3D, 20 steps with the state's load and read,
+  // 1104 us with items of 512, 896 with 288 (two full halves of a 4^3-cell block; 1.2x more with 192)
+  // together with the rotations that the return mapping hands on
+  c->item_cap = std::min(kItem, std::max(kItemMin, (ceil_div(c->P, c->n_sm * 2) + 31) / 32 * 32));
+  c->narrow = c->D == 2 && c->P > c->n_sm * 256;
+  c->max_work = ceil_div(c->P, c->item_cap) + std::min(c->n_keys, c->P) + 1;
 
   const int D = c->D, DD = D * D;
   const size_t comps = 2 * D + 2 * DD;
@@ -1338,7 +1374,9 @@ mpm_status mpm_init(const mpm_config* cfg, mpm_ctx** out) {
   p.mu_lam = c->mu_lam;
   p.sv_lo = 1.f - cfg->plastic_compression;
   p.sv_hi = 1.f + cfg->plastic_stretch;
-  c->fused_grid = std::max(1, std::min(c->max_work, c->n_sm * 8));
+  // several CTAs per resident place, so that the hardware evens out items of different length (a CTA
+  // without an item ends at once): 16 bodies in 2D 926 us with 8 per SM, 776 with 16, 752 with 24
+  c->fused_grid = std::max(1, std::min(c->max_work, c->n_sm * 24));
   *out = c;
   return MPM_OK;
 }
@@ -1511,7 +1549,8 @@ mpm_status mpm_step_profiled(mpm_ctx* c, int n_steps, void* flush_buf, size_t fl
     c->cur = 1 - c->cur;
     cudaEventRecord(e[1], s);
     mpm_scan<<<c->n_scan_tiles, kScanTile, 0, s>>>(c->n_keys, c->P, c->counts, c->offsets, c->cursor, c->work,
-                                                   c->n_work, c->max_work, c->tile_state, c->status);
+                                                   c->n_work, c->max_work, c->item_cap, c->nb, c->nblk, c->D,
+                                                   c->tile_state, c->status);
     cudaEventRecord(e[2], s);
     int blocks = std::max(1, std::min(ceil_div(c->P, 256), c->n_sm * 8));
     if (c->D == 2)

@@ -125,12 +125,15 @@ __device__ __forceinline__ float dot6_compensated(const float x[6], const float 
   return s + c;
 }
 
-template <int REFINE>
-__device__ __forceinline__ void f_minus_polar_3d(const float F[9], float out[9]) {
-  float X[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) X[i] = F[i];
-  // scaled Newton in FP32; converges quadratically, 10 iterations bound it
+// Scaled Newton iteration of the polar rotation in FP32, X <- (z X + (z X)^-T) / 2, z = |det X|^(-1/3),
+// in place; at most 10 iterations, the last the one that moved no entry by `stop` or more.  It converges
+// quadratically: the iterate that moved by e is within about e^2 / 2 of the limit, so one that moved by
+// less than kPolarConverged is there (2e-10), without the pass that kPolarSettled spends on seeing it.
+// At strains of 1e-4 a stop of 2e-4 (2e-8) raised the error of the stress against 64 bits from 1.6e-8 to
+// 3.9e-8 of the moduli; 2e-5 leaves it.  The return mapping keeps kPolarSettled: it rebuilds F from the
+// rotation, so that every rounding of the rotation goes into F.
+constexpr float kPolarConverged = 2e-5f, kPolarSettled = 2e-7f;
+__device__ __forceinline__ void polar_newton_3d(float X[9], float stop) {
   for (int it = 0; it < 10; ++it) {
     float C[9];
     cofactor3(X, C);
@@ -144,8 +147,14 @@ __device__ __forceinline__ void f_minus_polar_3d(const float F[9], float out[9])
       diff = fmaxf(diff, fabsf(nx - X[i]));
       X[i] = nx;
     }
-    if (diff < 2e-7f) break;
+    if (diff < stop) break;
   }
+}
+
+// X comes in as F, or with `known` as the FP32 rotation of F.
+template <int REFINE>
+__device__ __forceinline__ void f_minus_polar_3d(const float F[9], float out[9], float X[9], bool known, float stop) {
+  if (!known) polar_newton_3d(X, stop);
   // F - R0 (row-major); entries that cancel are exact in FP32
 #pragma unroll
   for (int i = 0; i < 9; ++i) out[i] = F[i] - X[i];
@@ -235,21 +244,7 @@ template <>
 __device__ __forceinline__ void polar_rotation<3>(const float F[9], float R[9]) {
 #pragma unroll
   for (int i = 0; i < 9; ++i) R[i] = F[i];
-  for (int it = 0; it < 10; ++it) {
-    float C[9];
-    cofactor3(R, C);
-    const float det = R[0] * C[0] + R[1] * C[1] + R[2] * C[2];
-    const float z = rcbrtf(fabsf(det));
-    const float zi = __frcp_rn(z * det);
-    float diff = 0.f;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const float nx = 0.5f * (z * R[i] + zi * C[i]);
-      diff = fmaxf(diff, fabsf(nx - R[i]));
-      R[i] = nx;
-    }
-    if (diff < 2e-7f) break;
-  }
+  polar_newton_3d(R, kPolarSettled);
 }
 
 // Eigen-decomposition A = Q diag(l) Q^T of a symmetric D x D matrix by cyclic Jacobi rotations
@@ -298,9 +293,11 @@ __device__ __forceinline__ void jacobi_eig_sym(float A[D * D], float Q[D * D], f
 // Return mapping of the plastic fixed-corotated material: with F = R S and S = Q diag(l) Q^T
 // (so F = (R Q) diag(l) Q^T is its singular value decomposition), the singular values are clamped
 // to [lo, hi] and F rebuilt as R Q diag(clamped) Q^T; F is left untouched when no value moves.
+// R returns the rotation; true if F was left.  F is left without a decomposition where Gershgorin's
+// circles of S lie inside the limits (by 1e-6, above the rounding of the decomposition).
 template <int D>
-__device__ __forceinline__ void plastic_return(float F[D * D], float lo, float hi) {
-  float R[D * D], S[D * D], Q[D * D], l[D];
+__device__ __forceinline__ bool plastic_return(float F[D * D], float lo, float hi, float R[D * D]) {
+  float S[D * D], Q[D * D], l[D];
   polar_rotation<D>(F, R);
 #pragma unroll
   for (int i = 0; i < D; ++i)
@@ -319,6 +316,15 @@ __device__ __forceinline__ void plastic_return(float F[D * D], float lo, float h
       S[i * D + j] = m;
       S[j * D + i] = m;
     }
+  bool inside = true;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    float rad = 1e-6f;
+#pragma unroll
+    for (int j = 0; j < D; ++j) rad += j == i ? 0.f : fabsf(S[i * D + j]);
+    inside &= S[i * D + i] - rad > lo && S[i * D + i] + rad < hi;
+  }
+  if (inside) return true;
   jacobi_eig_sym<D>(S, Q, l);
   bool moved = false;
   float lc[D];
@@ -327,7 +333,7 @@ __device__ __forceinline__ void plastic_return(float F[D * D], float lo, float h
     lc[i] = fminf(fmaxf(l[i], lo), hi);
     moved |= lc[i] != l[i];
   }
-  if (!moved) return;
+  if (!moved) return true;
   // U = R Q; F = U diag(lc) Q^T
   float U[D * D];
 #pragma unroll
@@ -348,14 +354,17 @@ __device__ __forceinline__ void plastic_return(float F[D * D], float lo, float h
       for (int k = 0; k < D; ++k) acc = fmaf(U[i * D + k] * lc[k], Q[j * D + k], acc);
       F[i * D + j] = acc;
     }
+  return false;
 }
 
 // Kirchhoff stress tau = P F^T.
 //   neo-Hookean:      tau = mu (F F^T - I) + lam ln(J) I
 //   fixed-corotated:  tau = 2 mu (F - R) F^T + lam (J - 1) J I
 // ln J and J - 1 come from det(F) - 1 computed without cancellation.
+// 3D: `stop` is that of polar_newton_3d; with `known`, R0 is the rotation it gives.
 template <int D, int MATERIAL, int POLAR>
-__device__ __forceinline__ void kirchhoff(const float F[D * D], float mu, float lam, float tau[D * D]) {
+__device__ __forceinline__ void kirchhoff(const float F[D * D], float mu, float lam, float tau[D * D],
+                                          float stop = kPolarSettled, const float* R0 = nullptr, bool known = false) {
   float jm1 = det_minus_one<D>(F);
   if (MATERIAL == 0) {
     float l = lam * log1pf(jm1);
@@ -370,10 +379,14 @@ __device__ __forceinline__ void kirchhoff(const float F[D * D], float mu, float 
       }
   } else {
     float FR[D * D];
-    if (D == 2)
+    if (D == 2) {
       f_minus_polar_2d(F, FR);
-    else
-      f_minus_polar_3d<POLAR>(F, FR);
+    } else {
+      float X[D * D];
+#pragma unroll
+      for (int i = 0; i < D * D; ++i) X[i] = known ? R0[i] : F[i];
+      f_minus_polar_3d<POLAR>(F, FR, X, known, stop);
+    }
     float l = lam * jm1 * (jm1 + 1.0f);
 #pragma unroll
     for (int i = 0; i < D; ++i)
