@@ -1100,129 +1100,123 @@ __device__ bool chol_solve(double* A, double* b, int r) {
   return !s_bad;
 }
 
-// Solve of the same SPD system by an FP32 Cholesky factor with iterative refinement in FP64
-// (the first warp; FP64 arithmetic has a ~65-cycle dependent latency on this GPU, FP32 ~5): the
-// correction of each sweep solves L L^T d = b - A x with the FP32 factor, the residual is formed in
-// FP64 from the unmodified A, and the sweeps stop once the correction is below 2^-40 of x (the
-// entries of A and b, assembled by compensated FP32 sums, carry about that relative accuracy).
-// Converges when cond(A) is well below 1 / FP32 epsilon; returns false (A and b untouched) if the
-// FP32 factorisation breaks down or 8 sweeps do not converge, and the caller falls back to
-// chol_solve.  On success b holds the solution.
-// The factor lives in registers: lane i holds row i of L (KR >= r entries, unrolled loops with
-// compile-time bounds), the columns pass between lanes by shuffles, and a copy of L in shared
-// memory gives each lane its column for the back substitution.
-template <int KR>
-__device__ bool chol_solve_refined_reg(const double* A, double* b, int r) {
-  __shared__ float Lsm[kMaxRl * (kMaxRl + 1)];
-  __shared__ double s_x[kMaxRl];
+// Solve of the same SPD system by an FP32 inverse with iterative refinement in FP64: the correction of
+// each sweep is d = B (b - A x) with B the FP32 inverse, the residual is formed in FP64 from the
+// unmodified A, and the sweeps stop once the correction is below 2^-40 of x (the entries of A and b,
+// assembled by compensated FP32 sums, carry about that relative accuracy).  Converges when cond(A) is
+// well below 1 / FP32 epsilon; returns false (A and b untouched) if a pivot is not positive or 8 sweeps
+// do not converge, and the caller falls back to chol_solve.  On success b holds the solution.
+//
+// One CTA solves while the chip waits, so what counts is the chain of dependent operations and the
+// instructions fetched on the way.  The inverse (the symmetric sweep operator, Goodnight 1979: pivot k
+// maps a_ij to a_ij - a_ik a_kj / a_kk, row and column k to a_ik / a_kk, a_kk to -1 / a_kk; after all
+// pivots the matrix is -A^-1) has one element per thread (four for r > 16) in registers and one
+// published column and barrier per pivot, and a sweep's correction is then one matrix-vector product
+// instead of 2 r dependent substitution steps.  Kernel cycles at r = 16 (r = 32): a Cholesky factor
+// held by one warp in unrolled code 10,900 (40,000), its two or three sweeps 14,000 to 18,000
+// (37,000 to 48,000).
+template <int RP>
+__device__ bool spd_solve_refined(const double* A, double* b, int r) {
+  constexpr int NE = RP * RP > kNormBlock ? RP * RP / kNormBlock : 1;   // elements per thread
+  constexpr int LD = RP + 1;
+  static_assert(NE * kNormBlock == RP * RP, "one pass of the threads covers the matrix");
+  __shared__ float s_col[2][RP];
+  __shared__ float s_inv[RP * LD];
+  __shared__ float s_v[RP];
+  __shared__ double s_x[RP];
   __shared__ int s_ok;
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    float Lr[KR];
+  const int t = threadIdx.x;
+  const int j = t % RP, i0 = t / RP;              // element (i0 + q kNormBlock / RP, j)
+  float a[NE];
 #pragma unroll
-    for (int k = 0; k < KR; ++k) Lr[k] = (lane < r && k < r) ? (float)A[lane * r + k] : 0.f;
-    float rd = 0.f;   // 1 / L[lane][lane]
-    bool ok = true;
-#pragma unroll
-    for (int j = 0; j < KR; ++j) {
-      if (j < r && ok) {
-        const float piv = __shfl_sync(0xffffffffu, Lr[j], j);
-        if (!(piv > 0.f) || !(piv < 3.0e38f)) {
-          ok = false;   // uniform: every lane sees the same pivot
-        } else {
-          const float y = rsqrtf(piv);
-          const float l = lane > j ? Lr[j] * y : 0.f;
-          if (lane == j) {
-            Lr[j] = piv * y;
-            rd = y;
-          } else if (lane > j) {
-            Lr[j] = l;
-          }
-#pragma unroll
-          for (int k = j + 1; k < KR; ++k) {
-            if (k < r) {
-              const float lk = __shfl_sync(0xffffffffu, l, k);
-              if (lane >= k) Lr[k] = fmaf(-l, lk, Lr[k]);
-            }
-          }
-        }
-      }
-    }
-    int conv = 0;
-    if (ok) {
-#pragma unroll
-      for (int k = 0; k < KR; ++k) Lsm[lane * (kMaxRl + 1) + k] = Lr[k];
-      __syncwarp();
-      float Lc[KR];   // column `lane` of L: Lc[i] = L[i][lane]
-#pragma unroll
-      for (int i = 0; i < KR; ++i) Lc[i] = Lsm[i * (kMaxRl + 1) + lane];
-      if (lane < r) s_x[lane] = 0.0;
-      float v = lane < r ? (float)b[lane] : 0.f;
-      __syncwarp();
-      for (int sweep = 0; sweep < 8 && !conv; ++sweep) {
-        // L L^T d = v (FP32), d in v: forward by columns, backward by rows of L
-#pragma unroll
-        for (int k = 0; k < KR; ++k) {
-          if (k < r) {
-            const float yk = __shfl_sync(0xffffffffu, v * rd, k);
-            if (lane == k) v = yk;
-            else if (lane > k) v = fmaf(-Lr[k], yk, v);
-          }
-        }
-#pragma unroll
-        for (int i = KR - 1; i >= 0; --i) {
-          if (i < r) {
-            const float xi = __shfl_sync(0xffffffffu, v * rd, i);
-            if (lane == i) v = xi;
-            else if (lane < i) v = fmaf(-Lc[i], xi, v);
-          }
-        }
-        // x += d; residual b - A x in FP64 (four independent partial sums per row)
-        float dmax = 0.f, xmax = 0.f;
-        if (lane < r) {
-          const double xn = s_x[lane] + (double)v;
-          s_x[lane] = xn;
-          dmax = fabsf(v);
-          xmax = fabsf((float)xn);
-        }
-        __syncwarp();
-        if (lane < r) {
-          double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
-          int jj = 0;
-          for (; jj + 3 < r; jj += 4) {
-            p0 = fma(A[lane * r + jj], s_x[jj], p0);
-            p1 = fma(A[lane * r + jj + 1], s_x[jj + 1], p1);
-            p2 = fma(A[lane * r + jj + 2], s_x[jj + 2], p2);
-            p3 = fma(A[lane * r + jj + 3], s_x[jj + 3], p3);
-          }
-          for (; jj < r; ++jj) p0 = fma(A[lane * r + jj], s_x[jj], p0);
-          v = (float)(b[lane] - ((p0 + p1) + (p2 + p3)));
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-          xmax = fmaxf(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
-        }
-        conv = dmax <= 9.1e-13f * xmax;   // 2^-40 of x: below the accuracy of the assembled system
-        __syncwarp();
-      }
-    }
-    if (conv && lane < r) b[lane] = s_x[lane];
-    if (lane == 0) s_ok = conv;
+  for (int q = 0; q < NE; ++q) {
+    const int i = i0 + q * (kNormBlock / RP);
+    a[q] = i < r && j < r ? (float)A[i * r + j] : 0.f;
+    if (j == 0) s_col[0][i] = a[q];
   }
   __syncthreads();
-  return s_ok != 0;
-}
-
-__device__ bool chol_solve_refined(const double* A, double* b, int r) {
-  if (r <= 8) return chol_solve_refined_reg<8>(A, b, r);
-  if (r <= 16) return chol_solve_refined_reg<16>(A, b, r);
-  return chol_solve_refined_reg<kMaxRl>(A, b, r);
+  bool ok = true;                                 // uniform: every thread sees the same pivots
+  for (int k = 0; k < r; ++k) {
+    const float* col = s_col[k & 1];
+    const float piv = col[k], aj = col[j];
+    if (!(piv > 0.f) || !(piv < 3.0e38f)) {
+      ok = false;
+      break;
+    }
+    const float ip = __frcp_rn(piv);
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      const int i = i0 + q * (kNormBlock / RP);
+      const float ai = col[i], si = ai * ip, sj = aj * ip;
+      const float up = i < j ? fmaf(-si, aj, a[q]) : fmaf(-sj, ai, a[q]);   // equal at (i, j) and (j, i)
+      a[q] = i == k ? (j == k ? -ip : sj) : (j == k ? si : up);
+      if (j == k + 1) s_col[(k + 1) & 1][i] = a[q];
+    }
+    __syncthreads();
+  }
+  if (ok) {
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      const int i = i0 + q * (kNormBlock / RP);
+      s_inv[i * LD + j] = -a[q];                  // rows and columns past r are zero
+    }
+    __syncthreads();
+    if (t < 32) {
+      // lanes (half h, row i): r <= 16 splits a row's products over the two half warps
+      constexpr int H = RP <= 16 ? 2 : 1;
+      constexpr int NC = RP / H;                  // columns per lane
+      const int i = t % RP < r ? t % RP : r - 1, c0 = H == 2 ? (t / RP) * NC : 0;
+      const bool row = t < r;
+      float inv[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) inv[c] = s_inv[i * LD + c0 + c];
+      const double bi = b[i];
+      double x = 0.0, res = bi;
+      int conv = 0;
+      for (int sweep = 0; sweep < 8 && !conv; ++sweep) {
+        if (t < RP) s_v[t] = t < r ? (float)res : 0.f;
+        __syncwarp();
+        float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+        for (int c = 0; c < NC; c += 2) {
+          d0 = fmaf(inv[c], s_v[c0 + c], d0);
+          d1 = fmaf(inv[c + 1], s_v[c0 + c + 1], d1);
+        }
+        float d = d0 + d1;
+        if (H == 2) d += __shfl_xor_sync(0xffffffffu, d, 16);
+        x += (double)d;
+        // largest correction and largest entry (bit patterns of non-negative floats are ordered)
+        const unsigned dm = __reduce_max_sync(0xffffffffu, row ? __float_as_uint(fabsf(d)) : 0u);
+        const unsigned xm = __reduce_max_sync(0xffffffffu, row ? __float_as_uint(fabsf((float)x)) : 0u);
+        conv = __uint_as_float(dm) <= 9.1e-13f * __uint_as_float(xm) && __uint_as_float(xm) < 3.0e38f;   // 2^-40 of x
+        if (conv) break;
+        if (t < RP) s_x[t] = x;
+        __syncwarp();
+        double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
+#pragma unroll
+        for (int c = 0; c < NC; c += 4) {
+          const int cc = c0 + c;
+          if (cc < r) p0 = fma(A[cc * r + i], s_x[cc], p0);
+          if (cc + 1 < r) p1 = fma(A[(cc + 1) * r + i], s_x[cc + 1], p1);
+          if (cc + 2 < r) p2 = fma(A[(cc + 2) * r + i], s_x[cc + 2], p2);
+          if (cc + 3 < r) p3 = fma(A[(cc + 3) * r + i], s_x[cc + 3], p3);
+        }
+        double p = (p0 + p1) + (p2 + p3);
+        if (H == 2) p += __shfl_xor_sync(0xffffffffu, p, 16);
+        res = bi - p;
+      }
+      if (conv && row) b[t] = x;
+      if (t == 0) s_ok = conv;
+    }
+    __syncthreads();
+    ok = s_ok != 0;
+  }
+  return ok;
 }
 
 __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, const float* __restrict__ dec,
                                                          int64_t cap, int mode, const float* __restrict__ target,
-                                                         int projection, int n_rows_override, float ridge) {
+                                                         int projection, int n_rows_override, float ridge, double inv_r) {
   const int d = R.d, r = R.r;
   const int nP = n_rows_override > 0 ? n_rows_override : R.counts[0];
   const int rows = nP * d;
@@ -1233,6 +1227,27 @@ __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, c
   __shared__ bool s_last;
   // hi / lo FP32 split of vhat_n (FP64) for the velocity right-hand side
   __shared__ float s_vh_hi[kMaxRl], s_vh_lo[kMaxRl];
+  // element e = threadIdx.x + q kNormBlock of the accumulators as (row, column) of the upper triangle of
+  // J^T J; column r: J^T b, row and column r: b^T b
+  constexpr int kAcc = (kMaxRl * (kMaxRl + 1) / 2 + kMaxRl + 1 + kNormBlock - 1) / kNormBlock;
+  int ei[kAcc], ej[kAcc];
+#pragma unroll
+  for (int q = 0; q < kAcc; ++q) {
+    const int e = threadIdx.x + q * kNormBlock;
+    int i = 0, rem = e;
+    if (e < n_mat) {
+      while (rem >= r - i) {
+        rem -= r - i;
+        ++i;
+      }
+      rem += i;
+    } else {
+      i = e - n_mat;
+      rem = r;
+    }
+    ei[q] = i;
+    ej[q] = rem;
+  }
   if (mode == NE_VEL && threadIdx.x < r) {
     const double v = S.vh[threadIdx.x];
     const float hi = (float)v;
@@ -1252,15 +1267,7 @@ __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, c
       const int row = row0 + rr, p = row / d, a = row % d;
       float b;
       if (mode == NE_VEL) {
-        // right-hand side of the velocity increment: v_trial - J vhat_n, J vhat_n by a compensated
-        // dot product of the FP32 row with the hi / lo parts of vhat_n
-        float sh = 0.f, sc = 0.f;
-        for (int c = 0; c < r; ++c) {
-          const float x = dec[((size_t)(1 + c) * cap + p) * d + a];
-          dot2_term(x, s_vh_hi[c], sh, sc);
-          dot2_term(x, s_vh_lo[c], sh, sc);
-        }
-        b = (R.v_trial[(size_t)p * d + a] - sh) - sc;
+        b = R.v_trial[(size_t)p * d + a];   // minus J vhat_n, below
       } else if (mode == NE_GN) {
         b = dec[((size_t)(1 + r) * cap + p) * d + a] + R.dt * R.v_trial[(size_t)p * d + a];
       } else {
@@ -1269,26 +1276,34 @@ __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, c
       sb[rr] = b;
     }
     __syncthreads();
+    if (mode == NE_VEL) {
+      // right-hand side of the velocity increment: v_trial - J vhat_n, J vhat_n by a compensated
+      // dot product of the FP32 row with the hi / lo parts of vhat_n
+      if (threadIdx.x < nr) {
+        float sh = 0.f, sc = 0.f;
+        for (int c = 0; c < r; ++c) {
+          const float x = sJ[threadIdx.x][c];
+          dot2_term(x, s_vh_hi[c], sh, sc);
+          dot2_term(x, s_vh_lo[c], sh, sc);
+        }
+        sb[threadIdx.x] = (sb[threadIdx.x] - sh) - sc;
+      }
+      __syncthreads();
+    }
     // entries of J^T J (upper triangle), J^T b and b^T b over this tile's rows: compensated FP32
     // dot products (Dot2: exact products by FMA, error-free sums), added in FP64
-    for (int e = threadIdx.x; e < n_acc; e += blockDim.x) {
-      float sh = 0.f, sc = 0.f;
-      if (e < n_mat) {
-        // upper-triangle index e -> (i, j), i <= j
-        int i = 0, rem = e;
-        while (rem >= r - i) {
-          rem -= r - i;
-          ++i;
-        }
-        const int j = i + rem;
-        for (int q = 0; q < nr; ++q) dot2_term(sJ[q][i], sJ[q][j], sh, sc);
-      } else if (e < n_mat + r) {
-        const int i = e - n_mat;
-        for (int q = 0; q < nr; ++q) dot2_term(sJ[q][i], sb[q], sh, sc);
-      } else {
-        for (int q = 0; q < nr; ++q) dot2_term(sb[q], sb[q], sh, sc);
+#pragma unroll
+    for (int q = 0; q < kAcc; ++q) {
+      const int e = threadIdx.x + q * kNormBlock;
+      if (e < n_acc) {
+        float sh = 0.f, sc = 0.f;
+        const float* u = ei[q] < r ? &sJ[0][ei[q]] : sb;
+        const float* w = ej[q] < r ? &sJ[0][ej[q]] : sb;
+        const int su = ei[q] < r ? kMaxRl + 1 : 1, sw = ej[q] < r ? kMaxRl + 1 : 1;
+#pragma unroll 4
+        for (int k = 0; k < nr; ++k) dot2_term(u[k * su], w[k * sw], sh, sc);
+        atomicAdd(&S.acc[e], (double)sh + (double)sc);
       }
-      atomicAdd(&S.acc[e], (double)sh + (double)sc);
     }
     __syncthreads();
   }
@@ -1303,26 +1318,25 @@ __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, c
   __shared__ double bvec[kMaxRl];
   __shared__ double s_rhs[kMaxRl];
   __shared__ double s_bb, s_shift;
-  for (int e = threadIdx.x; e < n_mat; e += blockDim.x) {
-    int i = 0, rem = e;
-    while (rem >= r - i) {
-      rem -= r - i;
-      ++i;
+  // (the accumulators live in L2: written by atomics, read past L1)
+#pragma unroll
+  for (int q = 0; q < kAcc; ++q) {
+    const int e = threadIdx.x + q * kNormBlock;
+    if (e < n_acc) {
+      const double v = __ldcg(&S.acc[e]);
+      const int i = ei[q], j = ej[q];
+      if (j < r) {
+        A_keep[i * r + j] = v;
+        A_keep[j * r + i] = v;
+      } else if (i < r) {
+        bvec[i] = v;
+        s_rhs[i] = v;
+      } else {
+        s_bb = v;
+      }
+      S.acc[e] = 0.0;
     }
-    const int j = i + rem;
-    const double v = atomicAdd(&S.acc[e], 0.0);
-    A[i * r + j] = v;
-    A[j * r + i] = v;
-    A_keep[i * r + j] = v;
-    A_keep[j * r + i] = v;
   }
-  for (int i = threadIdx.x; i < r; i += blockDim.x) {
-    bvec[i] = atomicAdd(&S.acc[n_mat + i], 0.0);
-    s_rhs[i] = bvec[i];
-  }
-  if (threadIdx.x == 0) s_bb = atomicAdd(&S.acc[n_mat + r], 0.0);
-  __syncthreads();
-  for (int e = threadIdx.x; e < n_acc; e += blockDim.x) S.acc[e] = 0.0;
   if (threadIdx.x == 0) S.counter[0] = 0u;
   __syncthreads();
   // Ridge rho tr(A) / r (rho = max(ridge, 1e-10)): the regularised least
@@ -1336,7 +1350,7 @@ __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, c
     double tr = threadIdx.x < r ? A_keep[threadIdx.x * r + threadIdx.x] : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-    if (threadIdx.x == 0) s_shift = (tr > 0 ? tr : 1.0) / r;
+    if (threadIdx.x == 0) s_shift = (tr > 0 ? tr : 1.0) * inv_r;
   }
   __syncthreads();
   bool ok = false;
@@ -1346,7 +1360,7 @@ __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, c
     for (int e = threadIdx.x; e < r * r; e += blockDim.x) A[e] = A_keep[e] + ((e / r) == (e % r) ? ridge_abs : 0.0);
     for (int i = threadIdx.x; i < r; i += blockDim.x) bvec[i] = s_rhs[i];
     __syncthreads();
-    ok = chol_solve_refined(A, bvec, r) || chol_solve(A, bvec, r);
+    ok = (r <= 16 ? spd_solve_refined<16>(A, bvec, r) : spd_solve_refined<kMaxRl>(A, bvec, r)) || chol_solve(A, bvec, r);
   }
   if (!ok) {
     if (threadIdx.x == 0) raise_status(R.status, STATUS_CHOLESKY);
@@ -1370,33 +1384,29 @@ __global__ void __launch_bounds__(kNormBlock) rom_normal(RomDev R, RomSolve S, c
       }
     }
   } else {
-    // GN step: J^T J delta = J^T b with b = -residual
-    __shared__ double s_slope, s_dn;
-    if (threadIdx.x < 32) {
-      double sl = threadIdx.x < r ? s_rhs[threadIdx.x] * bvec[threadIdx.x] : 0.0;
-      double dn = threadIdx.x < r ? bvec[threadIdx.x] * bvec[threadIdx.x] : 0.0;
+    // GN step: J^T J delta = J^T b with b = -residual.  Warp 0 and warp 1 form the slope and the
+    // length of the step while the others lay out the line search's trials.
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < 2) {
+      double sum = lane < r ? (warp == 0 ? s_rhs[lane] : bvec[lane]) * bvec[lane] : 0.0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sl += __shfl_xor_sync(0xffffffffu, sl, o);
-        dn += __shfl_xor_sync(0xffffffffu, dn, o);
-      }
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       if (threadIdx.x == 0) {
-        s_slope = -2.0 * sl;   // d/dalpha |res + alpha J delta|^2 at 0 = 2 res^T J delta = -2 b^T J delta
-        s_dn = sqrt(dn);
-        S.scal[0] = s_bb;      // f0 = |res|^2
-        S.scal[1] = s_slope;
-        S.scal[2] = s_dn;
+        S.scal[0] = s_bb;          // f0 = |res|^2
+        S.scal[1] = -2.0 * sum;    // d/dalpha |res + alpha J delta|^2 at 0 = 2 res^T J delta = -2 b^T J delta
+      } else if (threadIdx.x == 32) {
+        S.scal[2] = sqrt(sum);
       }
-    }
-    for (int i = threadIdx.x; i < r; i += blockDim.x) S.delta[i] = bvec[i];
-    __syncthreads();
-    const float* base32 = (mode == NE_FIT) ? S.xk32 : S.xh32;
-    for (int e = threadIdx.x; e < kLS * r; e += blockDim.x) {
-      const int m = e / r, i = e % r;
-      const double alpha = ldexp(1.0, -m);
-      const double basev = (mode == NE_FIT) ? S.xk[i] : S.xh[i];
-      S.ls_base32[e] = base32[i];
-      S.ls_dir32[e] = (float)((S.xk[i] - basev) + alpha * bvec[i]);
+      if (warp == 1 && lane < r) S.delta[lane] = bvec[lane];
+    } else {
+      const float* base32 = (mode == NE_FIT) ? S.xk32 : S.xh32;
+      for (int e = threadIdx.x - 64; e < kLS * r; e += kNormBlock - 64) {
+        const int m = e / r, i = e % r;
+        const double alpha = __hiloint2double((1023 - m) << 20, 0);   // 2^-m
+        const double basev = (mode == NE_FIT) ? S.xk[i] : S.xh[i];
+        S.ls_base32[e] = base32[i];
+        S.ls_dir32[e] = (float)((S.xk[i] - basev) + alpha * bvec[i]);
+      }
     }
   }
 }
@@ -1454,7 +1464,7 @@ __global__ void __launch_bounds__(kNormBlock) rom_linesearch(RomDev R, RomSolve 
     int pick = -1;
     for (int m = 0; m < kLS; ++m) {
       const double f = *((volatile double*)&S.fls[m]);
-      if (f <= f0 + armijo_c * ldexp(1.0, -m) * slope) {
+      if (f <= f0 + armijo_c * __hiloint2double((1023 - m) << 20, 0) * slope) {
         pick = m;
         break;
       }
@@ -1463,10 +1473,11 @@ __global__ void __launch_bounds__(kNormBlock) rom_linesearch(RomDev R, RomSolve 
     // negligible and the linear model promised a decrease well above the FP32
     // resolution of the objective (-slope / 2 = |J delta|^2 > 1e-3 f0);
     // otherwise the iterate has converged
-    double xn = 0;
-    for (int i = 0; i < r; ++i) xn += S.xk[i] * S.xk[i];
-    if (pick < 0 && dn > 1e-8 * (1.0 + sqrt(xn)) && -0.5 * slope > 1e-3 * f0)
-      raise_status(R.status, STATUS_GN_NO_DECREASE);
+    if (pick < 0) {
+      double xn = 0;
+      for (int i = 0; i < r; ++i) xn += S.xk[i] * S.xk[i];
+      if (dn > 1e-8 * (1.0 + sqrt(xn)) && -0.5 * slope > 1e-3 * f0) raise_status(R.status, STATUS_GN_NO_DECREASE);
+    }
     if (iter >= 0 && iter < kMaxGnIters) S.picks[iter] = pick;
     s_pick = pick;
   }
@@ -1474,7 +1485,7 @@ __global__ void __launch_bounds__(kNormBlock) rom_linesearch(RomDev R, RomSolve 
   const int pick = s_pick;
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
     double xk = S.xk[i];
-    if (pick >= 0) xk += ldexp(1.0, -pick) * S.delta[i];
+    if (pick >= 0) xk += __hiloint2double((1023 - pick) << 20, 0) * S.delta[i];
     S.xk[i] = xk;
     S.xk32[i] = (float)xk;
     const double basev = (mode == NE_FIT) ? xk : S.xh[i];
@@ -1744,7 +1755,7 @@ mpm_status rom_launch_step(rom_ctx* c, cudaStream_t s) {
     if (st != MPM_OK) return st;
   }
   rom_normal<<<b_ne, kNormBlock, 0, s>>>(c->dv, c->sv, c->outS, c->k_cap, NE_VEL, nullptr, c->cfg.projection, 0,
-                                         c->cfg.ridge);
+                                         c->cfg.ridge, 1.0 / c->dv.r);
   MPM_CUDA_TRY(cudaGetLastError());
   if (c->cfg.projection == 1) {
     rom_commit_velocity_only<<<1, 64, 0, s>>>(c->dv, c->sv);
@@ -1760,7 +1771,7 @@ mpm_status rom_launch_step(rom_ctx* c, cudaStream_t s) {
     st = decoder_launch_dev(c->dec, c->X, c->qlist, c->counts + 0, 1, c->k_cap, c->sv.xk32, c->sv.dk32, ks, r + 2,
                             c->outS, s);
     if (st != MPM_OK) return st;
-    rom_normal<<<b_ne, kNormBlock, 0, s>>>(c->dv, c->sv, c->outS, c->k_cap, NE_GN, nullptr, 0, 0, c->cfg.ridge);
+    rom_normal<<<b_ne, kNormBlock, 0, s>>>(c->dv, c->sv, c->outS, c->k_cap, NE_GN, nullptr, 0, 0, c->cfg.ridge, 1.0 / c->dv.r);
     MPM_CUDA_TRY(cudaGetLastError());
     st = decoder_launch_dev(c->dec, c->X, c->qlist, c->counts + 0, 1, c->k_cap, c->sv.ls_base32, c->sv.ls_dir32, kls,
                             1 + kLS, c->outLS, s);
@@ -2447,7 +2458,7 @@ mpm_status rom_fit_initial(rom_ctx* c, const float* target, const float* V0, int
   for (int it = 0; it < iters && st == MPM_OK; ++it) {
     st = decoder_launch_dev(c->dec, c->X, nullptr, c->nP_all, 1, P, c->sv.xk32, nullptr, ks, r + 1, c->outS, s);
     if (st != MPM_OK) break;
-    rom_normal<<<b_ne, kNormBlock, 0, s>>>(c->dv, c->sv, c->outS, P, NE_FIT, tgt, 0, P, 0.f);
+    rom_normal<<<b_ne, kNormBlock, 0, s>>>(c->dv, c->sv, c->outS, P, NE_FIT, tgt, 0, P, 0.f, 1.0 / c->dv.r);
     // trials: secant from the iterate; base rows hold the iterate
     st = decoder_launch_dev(c->dec, c->X, nullptr, c->nP_all, 1, P, c->sv.ls_base32, c->sv.ls_dir32, kls, 1 + kLS,
                             c->outLS, s);
@@ -2464,7 +2475,7 @@ mpm_status rom_fit_initial(rom_ctx* c, const float* target, const float* V0, int
     MPM_CUDA_TRY(cudaMemsetAsync(c->sv.vh, 0, sizeof(double) * r, s));
     // solve J^T J vhat = J^T V0 (projection flag 1 keeps xk: the commit below sets the state)
     MPM_CUDA_TRY(cudaMemcpyAsync(c->sv.xh, c->sv.xk, sizeof(double) * r, cudaMemcpyDeviceToDevice, s));
-    rom_normal<<<b_ne, kNormBlock, 0, s>>>(c->dv, c->sv, c->outS, P, NE_VEL, nullptr, 1, P, 0.f);
+    rom_normal<<<b_ne, kNormBlock, 0, s>>>(c->dv, c->sv, c->outS, P, NE_VEL, nullptr, 1, P, 0.f, 1.0 / c->dv.r);
   }
   cudaFree(tgt);
   cudaFree(vel);
