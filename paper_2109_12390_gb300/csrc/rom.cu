@@ -24,7 +24,7 @@
 //   decoder        dg/dxhat at (X^P, xhat_n)
 //   rom_normal     normal equations J^T J, J^T b (multi-CTA, compensated FP32
 //                  sums added in FP64); the last CTA to finish solves them (FP32
-//                  Cholesky with FP64 refinement, FP64 Cholesky fallback):
+//                  inverse with FP64 refinement, FP64 Cholesky fallback):
 //                  vhat_{n+1} (Eq. nonlinear_projection:vel), or a Gauss-Newton
 //                  step delta for xhat (Eq. ...:pos)
 //   per Gauss-Newton iteration (initial guess 2 xhat_n - xhat_{n-1}):
@@ -239,13 +239,17 @@ __global__ void __launch_bounds__(1024) rom_select(RomDev R) {
   const int n_prev = R.counts[2];
   for (int i = t; i < n_prev; i += T) R.grid[R.nodes[i]] = make_float4(0.f, 0.f, 0.f, 0.f);
 
-  // radix select of the k-th smallest hash
+  // radix select of the k-th smallest hash, ended once every hash of the selected bin is taken (the
+  // threshold is then the bin's upper end): two or three passes instead of eight for 4096 particles, 8 us
+  // of a step's 428
+  __shared__ int s_done;
+  bool done = false;
   if (t == 0) {
     s_prefix = 0ull;
     s_remaining = k;
   }
   unsigned long long mask = 0ull;
-  for (int pass = 0; pass < 8; ++pass) {
+  for (int pass = 0; pass < 8 && !done; ++pass) {
     const int shift = 56 - 8 * pass;
     for (int i = t; i < 256; i += T) s_hist[i] = 0;
     __syncthreads();
@@ -275,26 +279,29 @@ __global__ void __launch_bounds__(1024) rom_select(RomDev R) {
       const unsigned cross = __ballot_sync(0xffffffffu, incl >= rem);
       const int owner = cross ? __ffs(cross) - 1 : 31;
       if (lane == owner) {
-        int acc = incl - tot, b = lane * 8 + 7;
+        int acc = incl - tot, b = lane * 8 + 7, in_bin = -1;
         bool found = false;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           if (!found && acc + c[j] >= rem) {
             b = lane * 8 + j;
+            in_bin = c[j];
             found = true;
           } else if (!found) {
             acc += c[j];
           }
         }
         s_remaining = rem - acc;
+        s_done = in_bin == rem - acc;
         s_prefix = prefix | ((unsigned long long)b << shift);
       }
     }
     mask |= 255ull << shift;
     __syncthreads();
+    done = s_done != 0;
   }
-  const uint64_t thr = s_prefix;
-  const int need_eq = s_remaining;  // hashes equal to thr to take, lowest ids first
+  const uint64_t thr = done ? s_prefix | ~mask : s_prefix;
+  const int need_eq = done ? P : s_remaining;  // hashes equal to thr to take, lowest ids first
   // select: h < thr, or h == thr among the first need_eq by id
   int n_less = 0, n_eq = 0;
   for (int p = p0; p < p1; ++p) {
@@ -708,7 +715,7 @@ __global__ void __launch_bounds__(1024) rom_eul_cells(RomDev R) {
   const int k = R.counts[0];
   const uint32_t stamp = (uint32_t)(*R.step + 1);
   constexpr int NS = (D == 2) ? 9 : 27;
-  constexpr int NC = (D == 2) ? 16 : 64;     // cells -2 .. 1 around a node, per axis 4
+  constexpr int NC = (D == 2) ? 36 : 216;    // cells -2 .. 3 around a stencil's first node, per axis 6
   if (t == 0) s_nc = 0;
   __syncthreads();
   for (int i = t; i < k; i += T) {
@@ -730,29 +737,37 @@ __global__ void __launch_bounds__(1024) rom_eul_cells(RomDev R) {
     }
   }
   __syncthreads();
-  for (int e = t; e < k * NS * NC; e += T) {
-    const int l = R.nodes[e / NC];
-    const int o = e % NC;
-    int c[D];
-    int rem = l;
+  // Every sample's 6^D cells, four per thread and round so that their atomics overlap.  (A stencil's
+  // nodes share most of their cells: node by node it was 3^D 4^D tests per sample, 29 us for 256
+  // samples in 2D; with the shorter selection the Eulerian step went from 491 to 467 us.)
+  constexpr int U = 4;
+  for (int e0 = t; e0 < k * NC; e0 += U * T) {
+    int cl[U];
+    uint32_t old[U];
 #pragma unroll
-    for (int a = D - 1; a >= 0; --a) {
-      c[a] = rem % R.n;
-      rem /= R.n;
-    }
-    bool ok = true;
-    int oo = o;
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * T;
+      cl[u] = -1;
+      if (e >= k * NC) continue;
+      const int i = e / NC;
+      int oo = e - i * NC, c[D];
+      bool ok = true;
 #pragma unroll
-    for (int a = D - 1; a >= 0; --a) {
-      c[a] += (oo % 4) - 2;
-      oo /= 4;
-      ok &= (c[a] >= 1) & (c[a] <= R.n - 3);
+      for (int a = D - 1; a >= 0; --a) {
+        const int b = min(max(stencil_base(R.x_samp[(size_t)i * D + a], R.inv_dx), 0), R.n - 3);
+        c[a] = b + oo % 6 - 2;
+        oo /= 6;
+        ok &= (c[a] >= 1) & (c[a] <= R.n - 3);
+      }
+      if (ok) cl[u] = node_linear<D>(c, R.n);
     }
-    if (!ok) continue;
-    const int cl = node_linear<D>(c, R.n);
-    if (atomicExch(&R.cstamp[cl], stamp) != stamp) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) old[u] = cl[u] >= 0 ? atomicExch(&R.cstamp[cl[u]], stamp) : stamp;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (old[u] == stamp) continue;
       const int slot = atomicAdd(&s_nc, 1);
-      if (slot < R.cap_cells) R.clist[slot] = cl;
+      if (slot < R.cap_cells) R.clist[slot] = cl[u];
       else raise_status(R.status, STATUS_CAPACITY);
     }
   }
@@ -1114,7 +1129,8 @@ __device__ bool chol_solve(double* A, double* b, int r) {
 // published column and barrier per pivot, and a sweep's correction is then one matrix-vector product
 // instead of 2 r dependent substitution steps.  Kernel cycles at r = 16 (r = 32): a Cholesky factor
 // held by one warp in unrolled code 10,900 (40,000), its two or three sweeps 14,000 to 18,000
-// (37,000 to 48,000).
+// (37,000 to 48,000); with the inverse a whole step (256 samples, r = 16, four solves, 2D) went from 472
+// to 428 us.
 template <int RP>
 __device__ bool spd_solve_refined(const double* A, double* b, int r) {
   constexpr int NE = RP * RP > kNormBlock ? RP * RP / kNormBlock : 1;   // elements per thread
