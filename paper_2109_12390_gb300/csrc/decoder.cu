@@ -540,14 +540,6 @@ constexpr int kF32Threads = 512;
 constexpr int kF32Rows = 64;              // largest tile (row slots)
 constexpr int kF32In = 41;                // staged input row stride (d + r <= 40)
 
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)),
-               "l"(gmem_src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
 // ELU for the FP32 path: exp(z) - 1 with the fast exponential (absolute error at the FP32 ulp of
 // values near 1, far below the parity tolerance)
 __device__ __forceinline__ float act_f32path(int act, float z) {

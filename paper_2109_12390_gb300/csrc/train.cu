@@ -149,14 +149,6 @@ constexpr int kExchRows = 104;
 constexpr int kBwdMaxR = 5;           // rows per point in training: primal, d <= 3 tangents, JVP
 constexpr int kChunkStride = 33;      // padded row stride of one 32-feature chunk: distinct banks
 
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)),
-               "l"(gmem_src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_groups() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
 // 256 threads: warps w and w + 4 read the same tensor-memory lane group; thread
 // t owns tile row rw = 32 (w % 4) + lane and the feature half h = w / 4
 // (features 64 h .. 64 h + 63) of every layer.
@@ -228,7 +220,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_tc(BwdArgs a) {
         const __nv_bfloat16* src = (act ? a.astore : a.dstore) + ((int64_t)lz * kW + fg) * a.rows_total + row0 + 8 * c8;
         cp_async16((act ? sA : sD) + fl * 128 + 8 * c8, src);
       }
-      cp_async_commit_group();
+      cp_async_commit();
     };
     prefetch_z(a.n_hidden - 1, 0);
     // ---- output layer: residual adjoints ybar (FP32)
@@ -297,7 +289,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_tc(BwdArgs a) {
         mma_phase ^= 1u;
         tc::tc_fence_after();
       }
-      cp_async_wait_groups();   // this thread's staging copies of the step have landed
+      cp_async_wait_all();   // this thread's staging copies of the step have landed
       __syncthreads();
       if (tail->abort) break;
       for (int i2 = 0; i2 < 2; ++i2) {
@@ -384,7 +376,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_tc(BwdArgs a) {
 #pragma unroll
           for (int i = 0; i < 32; ++i) zs[(int64_t)(ch * 32 + i) * a.rows_total] = zb[i];
         }
-        if (i2 == 0) cp_async_wait_groups();   // the next chunk's staging has landed
+        if (i2 == 0) cp_async_wait_all();   // the next chunk's staging has landed
         __syncthreads();
       }
       // bias gradient of layer l (sbias was filled before the last barrier)
@@ -428,7 +420,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_tc(BwdArgs a) {
     for (int w = 0; w < kBwdThreads / 32; ++w) tot += s_loss[w];
     atomicAdd(a.loss, tot);
   }
-  cp_async_wait_groups();   // no staging copy outlives the CTA (an aborted sweep)
+  cp_async_wait_all();   // no staging copy outlives the CTA (an aborted sweep)
   tc::tc_fence_after();
   if (warp == 0) tc::tmem_free<kW>(tmem);
 }
@@ -972,9 +964,7 @@ __global__ void __launch_bounds__(128, 2) train_dw_gemm_image(const __nv_bfloat1
 constexpr int kMaxIn = 40;
 constexpr int kDw0Stride = 132;       // floats per staged feature row (128 rows + pad; float4 aligned)
 constexpr int kDw0MaxPt = 64;         // points per tile (R >= 2)
-// ROWMAJOR: zbar0 is stored row-major in decoder_bf16's row order (whole points of R = D + 2 consecutive
-// rows, floor(32 / R) points per 32 rows) and staged [row][feature].
-template <int D, bool ROWMAJOR>
+template <int D>
 __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t rows_total, Batch b, int r, int Pt,
                                                      const float* norm, const float* W0, float* gW0, float* g_lat_pt,
                                                      float* g_u_pt) {
@@ -1003,11 +993,7 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
     const int64_t row0 = tile * 128;
     __syncthreads();   // the previous tile's staged values are consumed
     // zbar0 rows of the tile: warp w stages features w, w + 8, ..., one float4 per lane
-    for (int rr = warp; ROWMAJOR && rr < 128; rr += 8) {
-      const float4 v = *reinterpret_cast<const float4*>(zb0 + (row0 + rr) * kW + 4 * lane);
-      *reinterpret_cast<float4*>(sz + rr * kDw0Stride + 4 * lane) = v;
-    }
-    for (int ff = warp; !ROWMAJOR && ff < kW; ff += 8) {
+    for (int ff = warp; ff < kW; ff += 8) {
       const float4 v = *reinterpret_cast<const float4*>(zb0 + (int64_t)ff * rows_total + row0 + 4 * lane);
       *reinterpret_cast<float4*>(sz + ff * kDw0Stride + 4 * lane) = v;
     }
@@ -1030,12 +1016,7 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
     // four points at a time with float4 reads of the staged adjoints where the rows allow it (a
     // quarter warp's 16-byte reads then fall in distinct banks; the scalar reads of lanes 132
     // floats apart conflict 4 ways)
-    const bool vec4 = !ROWMAJOR && (Pt & 3) == 0 && (q_lo & 3) == 0 && (q_hi & 3) == 0;
-    // a point's adjoint of feature f in row kind k
-    constexpr int R = D + 2, ppg = 32 / R;
-    auto zrow = [&](int q, int k) {
-      return ROWMAJOR ? sz[((q / ppg) * 32 + (q % ppg) * R + k) * kDw0Stride + f] : zf[k * Pt + q];
-    };
+    const bool vec4 = (Pt & 3) == 0 && (q_lo & 3) == 0 && (q_hi & 3) == 0;
     for (int q4 = q_lo; vec4 && q4 < q_hi; q4 += 4) {
       const float4 zp4 = *reinterpret_cast<const float4*>(zf + q4);
       float4 zt4[D];
@@ -1077,7 +1058,7 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
       }
     }
     for (int q = q_lo; !vec4 && q < q_hi; ++q) {
-      const float zp = zrow(q, 0);                   // primal row
+      const float zp = zf[q];                   // primal row
       const float* in = sin0 + q * kMaxIn;
 #pragma unroll
       for (int j = 0; j < kMaxIn; j += 4) {
@@ -1091,8 +1072,8 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
       }
 #pragma unroll
       for (int a2 = 0; a2 < D; ++a2)                 // X-tangent rows: one input each
-        acc[a2] = fmaf(zrow(q, 1 + a2), inv_range[a2], acc[a2]);
-      const float zj = zrow(q, D + 1);               // JVP row: [0, u] (u zero-padded to 32)
+        acc[a2] = fmaf(zf[(1 + a2) * Pt + q], inv_range[a2], acc[a2]);
+      const float zj = zf[(D + 1) * Pt + q];               // JVP row: [0, u] (u zero-padded to 32)
       const float* uq = su + q * 32;
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
@@ -1111,11 +1092,11 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
       const int g = o % n_groups, rr = o / n_groups;
       const int q = rr % Pt, jvp = rr / Pt;
       const int64_t pnt = tile * Pt + q;
-      const int row = ROWMAJOR ? (q / ppg) * 32 + (q % ppg) * R + (jvp ? d + 1 : 0) : (jvp ? d + 1 : 0) * Pt + q;
+      const int row = (jvp ? d + 1 : 0) * Pt + q;
       float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
 #pragma unroll 8
       for (int ff = 0; ff < kW; ++ff) {
-        const float z = ROWMAJOR ? sz[row * kDw0Stride + ff] : sz[ff * kDw0Stride + row];
+        const float z = sz[ff * kDw0Stride + row];
         const float4 w = *reinterpret_cast<const float4*>(sWl + ff * 36 + 4 * g);
         v0 = fmaf(z, w.x, v0);
         v1 = fmaf(z, w.y, v1);
@@ -1149,6 +1130,194 @@ __global__ void __launch_bounds__(256) train_dw0_lat(const float* zb0, int64_t r
 
 size_t dw0_smem_bytes() {
   return (size_t)(kW * kDw0Stride + kDw0MaxPt * kMaxIn + kDw0MaxPt * 32 + kW * 36) * sizeof(float);
+}
+
+// The same gradients from zbar0 as train_bwd_pipe stores it: row-major in decoder_bf16's row order (R = D + 2
+// consecutive rows per point, floor(32 / R) points per 32 rows), so that a tile is 64 consecutive KB.  One
+// CTA per SM; tile i + 1 arrives by asynchronous copies (its inputs in registers) under the arithmetic of tile
+// i.  Thread (feature pair, point group) sums the weight gradients: one shared read of an input then serves
+// two features, and the eight groups' sums meet once per CTA.  The latent adjoints take (point, 4 latents,
+// quarter of the features) per thread, both rows of the point at once, and four shuffled sums.  Bound by the
+// latency of the shared-memory reads (16 warps); 65,536 points, r = 16, 2D: 132 us with one staged tile per CTA and one
+// row or feature per thread, 94 us like this.
+constexpr int kDw0Threads = 512;
+constexpr int kDw0In = 32;            // d + r <= 31 on this path
+
+template <int D>
+__global__ void __launch_bounds__(kDw0Threads, 1) train_dw0_pipe(const float* __restrict__ zb0, int64_t rows_total,
+                                                                 Batch b, int r, const float* norm, const float* W0,
+                                                                 float* gW0, float* g_lat_pt, float* g_u_pt) {
+  constexpr int R = D + 2, PPG = 32 / R, PT = 4 * PPG;             // points per lane group and per tile
+  constexpr int NI = (PT * kDw0In + kDw0Threads - 1) / kDw0Threads;  // staged inputs per thread
+  constexpr int NG = kDw0Threads / (kW / 2);                       // point groups
+  extern __shared__ __align__(16) float dsm[];
+  float* sz = dsm;                                   // two tiles [128 rows][kDw0Stride]
+  float* sin0 = sz + 2 * 128 * kDw0Stride;           // [PT][32]: primal inputs of the points
+  float* su = sin0 + PT * kDw0In;                    // [PT][32]: JVP directions
+  float* sWl = su + PT * kDw0In;                     // [128][36]: latent columns of W0
+  const int t = threadIdx.x, lane = t & 31;
+  const int K = D + r;
+  for (int e = t; e < kW * 36; e += kDw0Threads) {
+    const int ff = e / 36, j = e % 36;
+    sWl[e] = j < r ? W0[ff * K + D + j] : 0.f;
+  }
+  float inv_range[D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) inv_range[a] = 1.f / norm[D + a];
+  const float lo = lane < D ? norm[lane] : 0.f, range = lane < D ? norm[D + lane] : 1.f;
+  const int64_t n_tiles = rows_total / 128;
+  auto fetch = [&](int64_t tile, int buf) {
+    const float* src = zb0 + tile * 128 * kW;
+    float* dst = sz + buf * 128 * kDw0Stride;
+#pragma unroll
+    for (int i = 0; i < 128 * kW / 4 / kDw0Threads; ++i) {
+      const int e = t + i * kDw0Threads, row = e >> 5, c = 4 * (e & 31);
+      cp_async16(dst + row * kDw0Stride + c, src + row * kW + c);
+    }
+    cp_async_commit();
+  };
+  float vi[NI], vu[NI];
+  // input `lane` of points t / 32, ... of a tile: X or xhat, and u
+  auto load_inputs = [&](int64_t tile) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int q = (t + i * kDw0Threads) >> 5;
+      const int64_t pnt = tile * PT + q;
+      const bool in = q < PT && pnt < b.B;
+      vi[i] = in && lane < K ? (lane < D ? b.X[pnt * D + lane] : b.xh[pnt * r + (lane - D)]) : 0.f;
+      vu[i] = in && lane < r ? b.u[pnt * r + lane] : 0.f;
+    }
+  };
+  const int fp = t & (kW / 2 - 1), pg = t / (kW / 2);
+  float acc[2][kDw0In];
+#pragma unroll
+  for (int j = 0; j < kDw0In; ++j) acc[0][j] = acc[1][j] = 0.f;
+  int64_t tile = blockIdx.x;
+  if (tile < n_tiles) {
+    fetch(tile, 0);
+    load_inputs(tile);
+  }
+  for (int buf = 0; tile < n_tiles; buf ^= 1) {
+    const int64_t next = tile + gridDim.x;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int e = t + i * kDw0Threads;
+      const bool valid = tile * PT + (e >> 5) < b.B;
+      if (e < PT * kDw0In) {
+        sin0[e] = lane < D ? (valid ? (vi[i] - lo) / range : 0.f) : vi[i];
+        su[e] = vu[i];
+      }
+    }
+    if (next < n_tiles) {
+      fetch(next, buf ^ 1);
+      cp_async_wait_but_one();
+    } else {
+      cp_async_wait_all();
+    }
+    __syncthreads();
+    if (next < n_tiles) load_inputs(next);
+    const float* z = sz + buf * 128 * kDw0Stride;
+    // (a) weight gradients of features 2 fp, 2 fp + 1 over this thread's points (rows of points past the batch are 0)
+#pragma unroll
+    for (int i = 0; i < (PT + NG - 1) / NG; ++i) {
+      const int q = pg + i * NG;
+      if (PT % NG != 0 && q >= PT) break;
+      const float* zq = z + ((q / PPG) * 32 + (q % PPG) * R) * kDw0Stride + 2 * fp;
+      const float2 zp = *reinterpret_cast<const float2*>(zq);
+      const float2 zj = *reinterpret_cast<const float2*>(zq + (D + 1) * kDw0Stride);
+      const float* in = sin0 + q * kDw0In;
+#pragma unroll
+      for (int j = 0; j < kDw0In; j += 4) {
+        if (j < K) {
+          const float4 v = *reinterpret_cast<const float4*>(in + j);
+          fma2(acc[0][j], acc[0][j + 1], v.x, v.y, zp.x);
+          fma2(acc[0][j + 2], acc[0][j + 3], v.z, v.w, zp.x);
+          fma2(acc[1][j], acc[1][j + 1], v.x, v.y, zp.y);
+          fma2(acc[1][j + 2], acc[1][j + 3], v.z, v.w, zp.y);
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < D; ++a) {                  // X-tangent rows: one input each
+        const float2 zt = *reinterpret_cast<const float2*>(zq + (1 + a) * kDw0Stride);
+        acc[0][a] = fmaf(zt.x, inv_range[a], acc[0][a]);
+        acc[1][a] = fmaf(zt.y, inv_range[a], acc[1][a]);
+      }
+      const float* uq = su + q * kDw0In;             // JVP row: [0, u]
+#pragma unroll
+      for (int j = 0; j + D < kDw0In; j += 4) {
+        if (j < r) {
+          const float4 v = *reinterpret_cast<const float4*>(uq + j);
+          const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (j + c + D < kDw0In) {
+              acc[0][D + j + c] = fmaf(zj.x, vv[c], acc[0][D + j + c]);
+              acc[1][D + j + c] = fmaf(zj.y, vv[c], acc[1][D + j + c]);
+            }
+        }
+      }
+    }
+    // (b) latent adjoints of the primal and the JVP row of each point: lanes (point, 4 latents, features 16 i + 4 part ..)
+    const int G = (r + 3) / 4, tasks = PT * G * 4;
+    for (int o0 = t - lane; o0 < tasks; o0 += kDw0Threads) {
+      const int o = min(o0 + lane, tasks - 1);
+      const int part = o & 3, g = (o >> 2) % G, q = (o >> 2) / G;
+      const float* zp = z + ((q / PPG) * 32 + (q % PPG) * R) * kDw0Stride + 4 * part;
+      const float* zj = zp + (D + 1) * kDw0Stride;
+      const float* w = sWl + 4 * part * 36 + 4 * g;
+      float vp[4] = {0.f, 0.f, 0.f, 0.f}, vj[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int i = 0; i < kW / 16; ++i) {
+        const float4 p4 = *reinterpret_cast<const float4*>(zp + 16 * i);
+        const float4 j4 = *reinterpret_cast<const float4*>(zj + 16 * i);
+        const float pa[4] = {p4.x, p4.y, p4.z, p4.w}, ja[4] = {j4.x, j4.y, j4.z, j4.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float4 w4 = *reinterpret_cast<const float4*>(w + (16 * i + c) * 36);
+          fma2(vp[0], vp[1], w4.x, w4.y, pa[c]);
+          fma2(vp[2], vp[3], w4.z, w4.w, pa[c]);
+          fma2(vj[0], vj[1], w4.x, w4.y, ja[c]);
+          fma2(vj[2], vj[3], w4.z, w4.w, ja[c]);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        vp[c] += __shfl_xor_sync(0xffffffffu, vp[c], 1);
+        vj[c] += __shfl_xor_sync(0xffffffffu, vj[c], 1);
+        vp[c] += __shfl_xor_sync(0xffffffffu, vp[c], 2);
+        vj[c] += __shfl_xor_sync(0xffffffffu, vj[c], 2);
+      }
+      const int64_t pnt = tile * PT + q;
+      if (part < 2 && o0 + lane < tasks && pnt < b.B) {
+        float* dst = (part ? g_u_pt : g_lat_pt) + pnt * r + 4 * g;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (4 * g + c < r) dst[c] = part ? vj[c] : vp[c];
+      }
+    }
+    __syncthreads();
+    tile = next;
+  }
+  // the point groups' sums, then one atomic per weight
+  constexpr int LD = kDw0In + 1;
+  static_assert(NG * LD <= 2 * kDw0Stride, "the sums fit the tile buffers");
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int j = 0; j < kDw0In; ++j) sz[(pg * kW + 2 * fp + h) * LD + j] = acc[h][j];
+  __syncthreads();
+  for (int e = t; e < kW * K; e += kDw0Threads) {
+    const int f = e / K, j = e - f * K;
+    float sum = 0.f;
+#pragma unroll
+    for (int g = 0; g < NG; ++g) sum += sz[(g * kW + f) * LD + j];
+    atomicAdd(&gW0[e], sum);
+  }
+}
+
+template <int D>
+constexpr size_t dw0_pipe_smem_bytes() {
+  return (size_t)(2 * 128 * kDw0Stride + 2 * 4 * (32 / (D + 2)) * kDw0In + kW * 36) * sizeof(float);
 }
 
 __global__ void train_lat_scatter(Batch b, int r, const float* g_lat_pt, const float* g_u_pt, float dt_snap,
@@ -1448,11 +1617,21 @@ mpm_status train_launch_step(trainer_ctx* c, cudaStream_t s, int update) {
       train_dw_gemm<<<g, 128, 0, s>>>(c->zbstore, c->astore, c->rows_total, kps, c->gparams, c->d_w_off, c->status);
     MPM_CUDA_TRY(cudaGetLastError());
   }
-  auto* dw0 = d == 2 ? (c->pipe ? train_dw0_lat<2, true> : train_dw0_lat<2, false>)
-                     : (c->pipe ? train_dw0_lat<3, true> : train_dw0_lat<3, false>);
-  dw0<<<c->n_sm * 2, 256, dw0_smem_bytes(), s>>>(c->zb0, c->rows_total, c->b, r, c->Pt, dec->norm,
-                                                 dec->params + dec->w_off[0], c->gparams + dec->w_off[0], c->g_lat_pt,
-                                                 c->g_u_pt);
+  const float* W0 = dec->params + dec->w_off[0];
+  float* gW0 = c->gparams + dec->w_off[0];
+  if (c->pipe) {
+    const int g0 = (int)std::min<int64_t>(c->n_sm, c->rows_total / 128);
+    if (d == 2)
+      train_dw0_pipe<2><<<g0, kDw0Threads, dw0_pipe_smem_bytes<2>(), s>>>(c->zb0, c->rows_total, c->b, r, dec->norm, W0,
+                                                                          gW0, c->g_lat_pt, c->g_u_pt);
+    else
+      train_dw0_pipe<3><<<g0, kDw0Threads, dw0_pipe_smem_bytes<3>(), s>>>(c->zb0, c->rows_total, c->b, r, dec->norm, W0,
+                                                                          gW0, c->g_lat_pt, c->g_u_pt);
+  } else {
+    auto* dw0 = d == 2 ? train_dw0_lat<2> : train_dw0_lat<3>;
+    dw0<<<c->n_sm * 2, 256, dw0_smem_bytes(), s>>>(c->zb0, c->rows_total, c->b, r, c->Pt, dec->norm, W0, gW0,
+                                                   c->g_lat_pt, c->g_u_pt);
+  }
   MPM_CUDA_TRY(cudaGetLastError());
   train_lat_scatter<<<blocks, 256, 0, s>>>(c->b, r, c->g_lat_pt, c->g_u_pt, c->cfg.dt_snap, c->g_lat);
   MPM_CUDA_TRY(cudaGetLastError());
@@ -1740,8 +1919,12 @@ mpm_status trainer_create(mpm_decoder* dec, const train_config* cfg, const snaps
     MPM_CUDA_TRY(cudaFuncSetAttribute(train_dw_gemm_image, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)dw_image_smem_bytes()));
   }
-  for (auto* f : {train_dw0_lat<2, true>, train_dw0_lat<2, false>, train_dw0_lat<3, true>, train_dw0_lat<3, false>})
+  for (auto* f : {train_dw0_lat<2>, train_dw0_lat<3>})
     MPM_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw0_smem_bytes()));
+  MPM_CUDA_TRY(cudaFuncSetAttribute(train_dw0_pipe<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)dw0_pipe_smem_bytes<2>()));
+  MPM_CUDA_TRY(cudaFuncSetAttribute(train_dw0_pipe<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)dw0_pipe_smem_bytes<3>()));
   train_pack_transposed<<<std::max(1, dec->n_tc * 64), 256>>>(dec->params, c->d_w_off, dec->n_tc, c->wtimg);
   MPM_CUDA_TRY(cudaGetLastError());
   MPM_CUDA_TRY(cudaDeviceSynchronize());
