@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
       }
       // training: the previous layer's activations leave the operand tile while the tensor core
       // reads it (both are reads; the barrier after the wait orders them before the next writes)
-      if (!SPLIT && a.astore && l > (l0_tc ? -1 : 0))
+      if (!SPLIT && a.astore && l >= 0)
         copy_out_tile(a.astore + (int64_t)l * kW * a.rows_total, a.rows_total, atile, tile, t);
       if (!tc::mbar_wait(&tail->bar_mma, mma_phase)) {
         raise_status(a.status, STATUS_TIMEOUT);

@@ -1,5 +1,6 @@
 """Minibatch gradients at the edges of the training kernels' tiles (32 or 24 points in 2D and 3D, eight or six per
-lane group), below and above two tiles per SM, at the largest latent dimension of the pipelined kernels (28) and with the linear activation, against the FP64 oracle.
+lane group), below and above two tiles per SM, at the largest latent dimension of the pipelined kernels (28) and
+the smallest of the feature-major ones (29), and with the linear activation, against the FP64 oracle.
 Bounds: 2e-2 norm-wise as tests/test_gpu_train.py; 5e-2 for the batches below 512 points, where the roundings of
 the operands to BF16 (2^-9 each, six layers forward and back: 2.3e-2 if none cancel) are hardly averaged."""
 import numpy as np
@@ -26,9 +27,9 @@ def _store(d, J, seed):
 
 
 @pytest.mark.parametrize("d,r,batch,act", [(2, 8, 1, OD.ELU), (2, 16, 31, OD.ELU), (2, 5, 33, OD.ELU),
-                                           (2, 28, 1000, OD.ELU), (2, 16, 9729, OD.ELU),
+                                           (2, 28, 1000, OD.ELU), (2, 29, 1000, OD.ELU), (2, 16, 9729, OD.ELU),
                                            (2, 16, 700, OD.IDENTITY), (3, 1, 23, OD.ELU), (3, 16, 25, OD.ELU),
-                                           (3, 28, 601, OD.ELU), (3, 7, 8000, OD.IDENTITY)])
+                                           (3, 28, 601, OD.ELU), (3, 29, 601, OD.ELU), (3, 7, 8000, OD.IDENTITY)])
 def test_gradients(d, r, batch, act):
     from paper_2109_12390_gb300.decoder import Decoder
     from paper_2109_12390_gb300.train import Trainer
