@@ -258,7 +258,7 @@ ROM_TRAIN_INSTANCES = 32
 ROM_TESTS = 4
 ENCODER_SUBSET = 1024
 ROM_SETTINGS = dict(n_samples=256, gn_iters=3, projection=0, ridge=1e-1, affine=0, f_reference=1)
-ROM_DECODER_FP32 = True     # reduced-step decoder calls in FP32 on the CUDA cores (training stays BF16)
+ROM_DECODER_FP32 = True     # reduced-step decoder calls in FP32 (training stays BF16)
 
 
 def _rom_tests(steps, n_tests=ROM_TESTS):
@@ -459,9 +459,9 @@ def rom_batch_serving(dec16, snaps, n_inst=384, steps=40, n_recon_inst=64):
             "setup_seconds": setup_s,
             "reading": "the reduced step is throughput-bound on its FP32 decoder work (the batch step takes about "
                        "the sum of the instances' steps): one launch serves them all, it does not add concurrency",
-            "autotune": {"chosen_precision": {1: "FP32 CUDA cores", 2: "split BF16 tensor cores"}[best_prec],
+            "autotune": {"chosen_precision": {1: "FP32", 2: "split BF16 tensor cores"}[best_prec],
                          "chosen_concurrency": best_k, "ms_per_batch_step": tune,
-                         "what": "precision/concurrency: square-layer arithmetic (1 FP32 CUDA cores, 2 split "
+                         "what": "precision/concurrency: square-layer arithmetic (1 FP32, 2 split "
                                  "BF16 tensor cores) and decoder_set_concurrency (FP32 tiles per call), timed"},
             "how": "one CUDA graph launch per step: every instance's step graph a parallel branch",
             "decoders": "r = 16 trained; r = 8 and 32 untrained (Xavier, same scaling), timing only",
@@ -618,7 +618,7 @@ def rom_leg(r=16, train_steps=None, steps=None):
                        f"at_{steps}_steps_{steps * 5e-5:.2f}s": bool(err_full <= 1e-2)},
         "paper_plain_settings": plain,
         "per_test": per_test,
-        "settings": dict(ROM_SETTINGS, latent_dim=r, decoder="FP32 CUDA cores" if ROM_DECODER_FP32 else "BF16 tcgen05"),
+        "settings": dict(ROM_SETTINGS, latent_dim=r, decoder="FP32" if ROM_DECODER_FP32 else "BF16 tcgen05"),
         "gain": {"trained": per_test[0]["rel_error_at_checkpoint"], "untrained_xavier": e_untrained,
                  "trained_linear_manifold": e_linear, "linear_training_steps": max(1, train_steps // 4),
                  "steps": ck},

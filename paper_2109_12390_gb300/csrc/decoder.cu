@@ -20,6 +20,10 @@
 // the BF16 rounding of the two absolute evaluations (the Gauss-Newton
 // residual needs differences far below BF16 resolution).
 //
+// This describes decoder_tc, the general kernel (mixed rows, r > 28, split BF16);
+// decoder_bf16 and decoder_tc3 take the other BF16 and FP32 calls with rows in
+// (point, kind) order, decoder_f32 the FP32 calls left (see each kernel).
+//
 // Per tile: layer 0 (K = d + r <= 35) and the output layer (N = d) run in
 // FP32 on the CUDA cores; each square 128 x 128 layer is one M=128, N=128,
 // K=128 tcgen05.mma chain (BF16 operands from shared memory in the 128-byte

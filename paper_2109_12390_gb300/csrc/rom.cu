@@ -240,8 +240,8 @@ __global__ void __launch_bounds__(1024) rom_select(RomDev R) {
   for (int i = t; i < n_prev; i += T) R.grid[R.nodes[i]] = make_float4(0.f, 0.f, 0.f, 0.f);
 
   // radix select of the k-th smallest hash, ended once every hash of the selected bin is taken (the
-  // threshold is then the bin's upper end): two or three passes instead of eight for 4096 particles, 8 us
-  // of a step's 428
+  // threshold is then the bin's upper end): two or three passes instead of eight for 4096 particles, 25 ->
+  // 18 us for the kernel
   __shared__ int s_done;
   bool done = false;
   if (t == 0) {
@@ -1130,7 +1130,7 @@ __device__ bool chol_solve(double* A, double* b, int r) {
 // instead of 2 r dependent substitution steps.  Kernel cycles at r = 16 (r = 32): a Cholesky factor
 // held by one warp in unrolled code 10,900 (40,000), its two or three sweeps 14,000 to 18,000
 // (37,000 to 48,000); with the inverse a whole step (256 samples, r = 16, four solves, 2D) went from 472
-// to 428 us.
+// to 428 us, the kernel from 30 to 15.
 template <int RP>
 __device__ bool spd_solve_refined(const double* A, double* b, int r) {
   constexpr int NE = RP * RP > kNormBlock ? RP * RP / kNormBlock : 1;   // elements per thread

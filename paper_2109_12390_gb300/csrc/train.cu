@@ -5,21 +5,23 @@
 //   train_sample     counter-based draw of the pairs (SplitMix64 of
 //                    (seed, step, i), uniform over all pairs), gather of X,
 //                    latents, JVP directions and targets
-//   decoder_tc       forward (tensor cores), storing every hidden layer's
-//                    activations and the primal rows' activation slopes (BF16,
-//                    feature-major)
-//   train_bwd_tc     loss residuals and output-layer gradients (FP32), then the
+//   decoder_bf16     forward (tensor cores), storing every hidden layer's
+//                    activations (128-row tiles as MMA images) and the primal
+//                    rows' activation slopes (BF16)
+//   train_bwd_pipe   loss residuals and output-layer gradients (FP32), then the
 //                    reverse sweep: z_bar = act'(z) h_bar + act''(z) sum_j zdot_j t_bar_j
 //                    for primal rows, zdot_bar = act'(z) t_bar for tangent rows; for
 //                    ELU act''(z) zdot_j = [z < 0] a_j, the tangent row's stored
 //                    activation, so the slope record and the activations suffice
-//                    (exchanged through shared memory), next adjoint rows by a
+//                    (a point's rows sit in one warp: shuffles), next adjoint rows by a
 //                    tcgen05 GEMM with the transposed weights resident in shared
-//                    memory; layer 0 and the latent adjoints in FP32
-//   train_dw_gemm    weight gradients of the square layers, dW = Zbar^T A, as
-//                    split-K tcgen05 GEMMs over all rows (both operands stored
-//                    row-contiguous, i.e. K-major), FP32 atomics across splits
-//   train_dw0        first-layer weight gradient (K = d + r, FP32)
+//                    memory
+//   train_dw_gemm_image  weight gradients of the square layers, dW = Zbar^T A, as
+//                    split-K tcgen05 GEMMs over all rows straight from the stored
+//                    images, FP32 atomics across splits
+//   train_dw0_pipe   first-layer weight gradient (K = d + r) and latent adjoints, FP32
+//   (r > 28: decoder_tc, train_bwd_tc, train_dw_gemm and train_dw0_lat, with
+//   feature-major activations and adjoints)
 //   train_lat_scatter latent-table gradient (snapshot n gets d/dxhat_n of its
 //                    own rows and -u_bar / dt; its successor gets +u_bar / dt)
 //   train_adam       Adam on the FP32 master parameters and the latent table,

@@ -93,7 +93,7 @@ class Decoder:
 
     def set_precision(self, fp32):
         """Square-layer arithmetic of decoder_eval and of reduced-order contexts created afterwards:
-        False / 0 BF16 tensor cores, True / 1 FP32 CUDA cores, 2 split BF16 (hi + lo operands,
+        False / 0 BF16 tensor cores, True / 1 FP32, 2 split BF16 (hi + lo operands,
         three products) on the tensor cores."""
         _abi.check(_abi.lib().decoder_set_precision(self._h, int(fp32)))
 

@@ -141,7 +141,7 @@ def rom_error(decoder, scene, fom_xs, *, n_samples=256, seed=4, gn_iters=3, proj
 
 def build_serving_batch(decoders, roms, concurrency, precision=None):
     """Sets the decoders' expected concurrency (the FP32 tiling of their calls) and, if given, their
-    square-layer arithmetic (1 FP32 CUDA cores, 2 split BF16 tensor cores), then captures the batch
+    square-layer arithmetic (1 FP32, 2 split BF16 tensor cores), then captures the batch
     of reduced-order contexts (one graph launch per step for all of them)."""
     from .rom import RomBatch
     for dec in decoders:
