@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_tc(BwdArgs a) {
 // Backward over decoder_bf16's stores (train_bwd_pipe): the reverse sweep of train_bwd_tc with the same
 // arithmetic per row, on the alternating-tile pipeline.  A lane group of 32 rows holds whole points (R
 // consecutive lanes each), so a point's curvature terms reach its primal row by shuffles, in the order
-// of its tangent rows (pairwise).  Per (tile slot, layer) the slot's 32 KB activation image and its points' slope
+// of its tangent rows.  Per (tile slot, layer) the slot's 32 KB activation image and its points' slope
 // records arrive by bulk copies; a thread takes 32 columns of its row: adjoint from tensor memory (or,
 // for the last hidden layer, Wout^T ybar), and writes the new adjoint over the activation it read.
 // The image then is the MMA's operand and is stored by one bulk copy for the weight-gradient GEMM.
@@ -499,6 +499,22 @@ size_t bwd_pipe_smem_bytes() {
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// 16 columns of four neighbouring lanes' rows, transposed by blocks of four: lane j of the four gets columns
+// 4 j .. 4 j + 3, row q's at v[4 q ..].
+__device__ __forceinline__ void quad_transpose(float (&v)[16], int j) {
+#pragma unroll
+  for (int x = 1; x < 4; x <<= 1) {
+    const bool up = (j & x) != 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if ((i >> 2) & x) continue;
+      const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + 4 * x], x);
+      v[i] = up ? got : v[i];
+      v[i + 4 * x] = up ? v[i + 4 * x] : got;
+    }
+  }
+}
 
 template <int D>
 __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) {
@@ -721,24 +737,41 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
               sw[0] = v0.x, sw[1] = v0.y, sw[2] = v0.z, sw[3] = v0.w, sw[4] = v1.x, sw[5] = v1.y, sw[6] = v1.z, sw[7] = v1.w;
               aw[0] = u0.x, aw[1] = u0.y, aw[2] = u0.z, aw[3] = u0.w, aw[4] = u1.x, aw[5] = u1.y, aw[6] = u1.z, aw[7] = u1.w;
             }
+            // The sum goes in the order of the rows, as train_bwd_tc adds them: it is rounded to BF16 next, and
+            // another order falls on the other side of a rounding here and there (pairwise sums moved the
+            // latent gradients of 2,105 points by 3e-5).  R = 4: the four lanes of a point take four columns each
+            // of its primal row, 16 shuffles per 16 columns; R = 5: the primal lane adds what it is sent, a
+            // shuffle per column and tangent row.  Gradients of 65,536 points, R = 4: 635 us; 709 with the
+            // R = 5 form, whose 48 shuffles then set the time; 679 with pairwise sums.
+            float term[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const float sp = (i & 1) ? bf16_hi(sw[i / 2]) : bf16_lo(sw[i / 2]);
               const float at = (i & 1) ? bf16_hi(aw[i / 2]) : bf16_lo(aw[i / 2]);
               const float zb = (sp < 0.f ? 1.f : sp) * z[i];
-              const float term = prim ? zb : (sp >= 0.f ? at : 0.f) * z[i];
-              // (primal + first tangent) + (second + third), and with R = 5 the fourth
-              float sum = term + __shfl_down_sync(0xffffffffu, term, 1);
-              sum += __shfl_down_sync(0xffffffffu, sum, 2);
-              if (R == 5) sum += __shfl_down_sync(0xffffffffu, term, 4);
-              z[i] = prim ? sum : zb;
+              term[i] = prim ? zb : (sp >= 0.f ? at : 0.f) * z[i];
+              z[i] = zb;
+              if (R == 5) {
+                float sum = term[i];
+#pragma unroll
+                for (int j = 1; j < R; ++j) sum += __shfl_down_sync(0xffffffffu, term[i], j);
+                z[i] = prim ? sum : zb;
+              }
+            }
+            float p4[4];                                 // R = 4: columns 4 k .. 4 k + 3 of the point's primal row
+            if (R == 4) {
+              quad_transpose(term, k);
+#pragma unroll
+              for (int c = 0; c < 4; ++c) p4[c] = ((term[c] + term[4 + c]) + term[8 + c]) + term[12 + c];
             }
             // bias gradients: the primal rows' adjoints summed per column (column lane % 8, the rows
             // in four parts)
 #pragma unroll
             for (int c = 0; c < 16; c += 8) {
               __syncwarp();
-              if (prim) {
+              if (R == 4 && (k >> 1) == c / 8)
+                *reinterpret_cast<float4*>(wscratch + q * 8 + 4 * (k & 1)) = make_float4(p4[0], p4[1], p4[2], p4[3]);
+              if (R == 5 && prim) {
                 float4* o = reinterpret_cast<float4*>(wscratch + q * 8);
                 o[0] = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
                 o[1] = make_float4(z[c + 4], z[c + 5], z[c + 6], z[c + 7]);
@@ -753,39 +786,38 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
               if (lane < 8) wbias[l * 32 + (c0 & 31) + c + lane] += v;
             }
             if (l >= 1) {
-              uint32_t w[8];
+              auto pack2 = [](float v0, float v1) {
+                const __nv_bfloat162 b2 = __floats2bfloat162_rn(v0, v1);
+                return *reinterpret_cast<const uint32_t*>(&b2);
+              };
+              if (R == 5 || k > 0) {
+                uint32_t w[8];
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const __nv_bfloat162 b2 = __floats2bfloat162_rn(z[2 * j], z[2 * j + 1]);
-                w[j] = *reinterpret_cast<const uint32_t*>(&b2);
+                for (int j = 0; j < 8; ++j) w[j] = pack2(z[2 * j], z[2 * j + 1]);
+                *own0 = make_uint4(w[0], w[1], w[2], w[3]);
+                *own1 = make_uint4(w[4], w[5], w[6], w[7]);
               }
-              *own0 = make_uint4(w[0], w[1], w[2], w[3]);
-              *own1 = make_uint4(w[4], w[5], w[6], w[7]);
+              if (R == 4)   // the primal row (nothing of its columns is read after the barrier of the bias sums)
+                *reinterpret_cast<uint2*>(image + tc::sw128_offset(rw - k, c0 + 4 * k, kW)) =
+                    make_uint2(pack2(p4[0], p4[1]), pack2(p4[2], p4[3]));
+            } else if (R == 4) {
+              // first-layer adjoints (FP32, row-major): the point's four lanes exchange their 16 columns so that
+              // each store of the warp writes 64 contiguous bytes of eight rows
+              quad_transpose(z, k);
+#pragma unroll
+              for (int c = 0; c < 4; ++c) z[c] = p4[c];
+#pragma unroll
+              for (int r4 = 0; r4 < 4; ++r4)
+                *reinterpret_cast<float4*>(a.zb0 + (grow - k + r4) * kW + c0 + 4 * k) =
+                    make_float4(z[4 * r4], z[4 * r4 + 1], z[4 * r4 + 2], z[4 * r4 + 3]);
             } else {
-              // first-layer adjoints (FP32, row-major): four neighbouring lanes exchange their 16 columns
-              // so that each store of the warp writes 64 contiguous bytes of eight rows
+              // the same by four neighbouring lanes, whatever their points
               const int j = lane & 3;
-              float4 got[4];                             // after round x: columns 4 j .. of row j ^ x
+              quad_transpose(z, j);
 #pragma unroll
-              for (int x = 0; x < 4; ++x) {
-                float g4[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                  const int p = j ^ x;
-                  const float v = p == 0 ? z[c] : p == 1 ? z[4 + c] : p == 2 ? z[8 + c] : z[12 + c];
-                  g4[c] = x == 0 ? v : __shfl_xor_sync(0xffffffffu, v, x);
-                }
-                got[x] = make_float4(g4[0], g4[1], g4[2], g4[3]);
-              }
-#pragma unroll
-              for (int r4 = 0; r4 < 4; ++r4) {
-                const int x = j ^ r4;
-                float4 v = got[0];
-                if (x == 1) v = got[1];
-                if (x == 2) v = got[2];
-                if (x == 3) v = got[3];
-                *reinterpret_cast<float4*>(a.zb0 + (grow - j + r4) * kW + c0 + 4 * j) = v;
-              }
+              for (int r4 = 0; r4 < 4; ++r4)
+                *reinterpret_cast<float4*>(a.zb0 + (grow - j + r4) * kW + c0 + 4 * j) =
+                    make_float4(z[4 * r4], z[4 * r4 + 1], z[4 * r4 + 2], z[4 * r4 + 3]);
             }
           }
           tc::fence_async_smem();
