@@ -39,19 +39,10 @@
 #include <vector>
 
 #include "common.cuh"
+#include "mpm_items.cuh"
 #include "mpm_math.cuh"
 
 namespace mpmrom {
-
-// The fused kernel takes up to kItem particles per work item, kItem / CH per thread, in CTAs of CH
-// threads.  3D: grid blocks of 4^3 cells at 8 particles per cell, 512 = 256 x 2.  2D: blocks of 8^2
-// cells at 4 per cell hold about 256 particles; large contexts take them in CTAs of 128 threads, so
-// that twice as many items are in flight per SM (an item's phases are separated by barriers and
-// dependent loads): 1.03 M particles in 16 bodies 854 -> 744 us for 10 steps with the state's load and
-// read.  Small ones (less than one such block per SM) keep 256 threads, whose items have the lower
-// latency: 4096 particles 10.9 against 12.0 us per step.
-constexpr int kItem = 512;
-constexpr int kItemMin = 128;         // smallest bound of a work item (small contexts)
 
 // Dynamic shared memory of the fused kernel: per slot its P2G record (2 D + D^2 floats), its
 // position in cell order, its cell and its rank within the cell.
@@ -1302,12 +1293,9 @@ mpm_status mpm_init(const mpm_config* cfg, mpm_ctx** out) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
-  // work items small enough that every SM has about two (an item's latency, not its work, sets the
-  // time of a small context): 84,915 plastic particles in 3D, 20 steps with the state's load and read,
-  // 1104 us with items of 512, 896 with 288 (two full halves of a 4^3-cell block; 1.2x more with 192)
-  // together with the rotations that the return mapping hands on
-  c->item_cap = std::min(kItem, std::max(kItemMin, (ceil_div(c->P, c->n_sm * 2) + 31) / 32 * 32));
-  c->narrow = c->D == 2 && c->P > c->n_sm * 256;
+  const ItemRule rule = item_rule(c->D, c->P, c->n_sm);
+  c->item_cap = rule.cap;
+  c->narrow = rule.narrow;
   c->max_work = ceil_div(c->P, c->item_cap) + std::min(c->n_keys, c->P) + 1;
 
   const int D = c->D, DD = D * D;
