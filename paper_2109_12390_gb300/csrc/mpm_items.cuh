@@ -22,13 +22,24 @@ struct ItemRule {
 // measured: one body of 134,689 particles 18.2 -> 17.4, of 144,400 17.4 -> 16.8, 16 of 140,494 18.7 -> 17.4.
 inline ItemRule item_rule(int dim, long long P, int n_sm) {
   ItemRule r{kItem, dim == 2 && P > 896ll * n_sm};
-  // work items small enough that every SM has about two (an item's latency, not its work, sets the
-  // time of a small context): 84,915 plastic particles in 3D, 20 steps with the state's load and read,
-  // 1104 us with items of 512, 896 with 288 (two full halves of a 4^3-cell block; 1.2x more with 192)
-  // together with the rotations that the return mapping hands on
-  const long long two = (P + 2ll * n_sm - 1) / (2ll * n_sm);
-  const long long cap = (two + 31) / 32 * 32;
-  r.cap = (int)(cap < kItemMin ? kItemMin : cap > kItem ? kItem : cap);
+  // An item's latency, not its work, sets the time of a small context, so blocks are split over several items
+  // there; but only while all items are resident at once (3 wide CTAs per SM), since one more wave costs what the
+  // split gains.  With half a full block per item that holds while the halves fill no more than 7/8 of the places
+  // (the rest is for blocks at the bodies' surfaces).
+  const long long half = dim == 2 ? 128 : 256, places = 3ll * n_sm;
+  if (8 * P > 7 * places * half) return r;
+  if (dim == 2) {
+    // Up to 128 particles per SM one item per block; past it 3/4 of a full block, so that one of a few particles
+    // more than 256 is cut in two and not in three: one body of 9,680 particles 11.2 -> 10.9 us a step (bound 512
+    // -> 256), five of 28,125 12.9 -> 11.5, one of 50,176 12.8 -> 12.2.
+    r.cap = P > 128ll * n_sm ? 192 : 256;
+  } else {
+    // About two items per SM: 12,240 plastic particles 33 -> 24 us a step (bound 512 -> 128), 36,000 41 -> 24,
+    // 84,915 48.8 -> 37.4.  Past the line above the same bound cost up to 14 %: 123,750 particles 26.2 -> 29.5,
+    // 139,536 plastic ones 52.2 -> 60.5.
+    const long long cap = ((P + 2ll * n_sm - 1) / (2ll * n_sm) + 31) / 32 * 32;
+    r.cap = (int)(cap < kItemMin ? kItemMin : cap > kItem ? kItem : cap);
+  }
   return r;
 }
 

@@ -44,3 +44,13 @@ def test_narrow_ctas_only_past_one_wave_of_wide_ones(rule, n_sm):
     for P in _sizes():
         assert not rule(2, P, n_sm)[1] or P > 768 * n_sm
     assert rule(2, 2000 * n_sm, n_sm)[1]
+
+
+@pytest.mark.parametrize("n_sm", [132, 148, 152])
+def test_blocks_are_split_only_while_the_items_are_resident(rule, n_sm):
+    # 3 items per SM: bodies of full blocks (256 particles in 2D, 512 in 3D) and nothing else
+    for dim, full in ((2, 256), (3, 512)):
+        for P in _sizes():
+            cap, narrow = rule(dim, P, n_sm)
+            items = -(-P // full) * -(-full // cap)
+            assert cap == 512 or items <= 3 * n_sm
