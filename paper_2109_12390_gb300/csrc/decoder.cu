@@ -2005,20 +2005,21 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
   // larger latents take the FP32 kernel
   const bool f32_path = (dec->fp32 == 1 || dec->r > 40 - kTcLat) && !a.dstore;
   // FP32 calls run on the tensor cores (decoder_tc3) but for mixed rows (their partner rows are not in
-  // the row's warp), for callers that keep decoder_f32's rounding, and for a lone caller's small calls
-  // with secant rows (256 samples x 12 or 18 rows: 32 us against 40 us; without secants, 256 x 17
-  // rows, 31 us against 24 us the other way; 4096 x 4 rows 98 against 25 us)
+  // the row's warp), for callers that keep decoder_f32's rounding, and for calls with secant rows that fit one of
+  // decoder_f32's small tiles per SM of the caller's share (256 samples x 12 or 18 rows of a lone caller: 32 us
+  // against 40 us; 16 x 12 rows of one of eight callers 33.6 against 41.9, 64 x 12, past it, 55 against 41; without
+  // secants, 256 x 17 rows, 31 us against 24 us the other way; 4096 x 4 rows 98 against 25 us)
+  const int share = std::max(1, dec->n_sm / std::max(1, dec->concurrency));
   bool secants = false;
   for (int k = 0; k < R; ++k) secants |= kind_class(kinds[k]) == 2;
   const bool pipe = !has_mixed && n * R < ((int64_t)1 << 31) - 4096;   // row numbers and their padding fit 32 bits
-  const bool tc3 = f32_path && pipe && !cuda_cores &&
-                   !(secants && dec->concurrency == 1 && n * R <= 31 * (int64_t)dec->n_sm);
+  const bool tc3 = f32_path && pipe && !cuda_cores && !(secants && n * R <= 31 * (int64_t)share);
   if (dec->n_tc == 0) {
     int64_t rows = n * R;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((rows + 127) / 128, dec->n_sm * 8));
     decoder_simt<<<blocks, 128, 0, s>>>(a);
   } else if (tc3) {
-    pipe_launch(a, true, n * R, dec->n_sm, std::max(1, dec->n_sm / std::max(1, dec->concurrency)), secants, s);
+    pipe_launch(a, true, n * R, dec->n_sm, share, secants, s);
   } else if (f32_path) {
     MPM_CHECK_ARG(R <= kF32Rows, "the FP32 path takes at most 64 row kinds");
     int64_t tiles;
@@ -2031,8 +2032,7 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
     } else {
       // packed tiles: about one per SM (per SM share of the concurrent callers), 32 or 64 slots
       const int64_t rows = n * R;
-      const int64_t target = std::max(1, dec->n_sm / std::max(1, dec->concurrency));
-      const int64_t U = std::max<int64_t>(1, std::min<int64_t>((rows + target - 1) / target, kF32Rows - 1));
+      const int64_t U = std::max<int64_t>(1, std::min<int64_t>((rows + share - 1) / share, kF32Rows - 1));
       a.f32_U = (int)U;
       a.Pt = 1;
       small = U + 1 <= 32;
