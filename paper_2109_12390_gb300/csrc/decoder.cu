@@ -145,7 +145,10 @@ __device__ __forceinline__ void store_operand(uint8_t* tile, int row, int col, c
 // the dropped A_lo W_lo term and the residuals of the splits being about 2^-16 of each product;
 // the two weight images of one layer at a time are streamed into shared memory while the
 // previous layer's epilogue runs, and the activations take the accurate exponential.
-template <bool SPLIT>
+// TRAIN (not with SPLIT): the activations of every layer and the primal rows' slopes are stored.  A variant
+// of its own: with the stores behind a runtime test the evaluations were 5 to 8 % slower (20,000 points x 12
+// rows with secants, r = 32: 1.14 -> 1.05 ms; split BF16, r = 16: 1.35 -> 1.28).
+template <bool SPLIT, bool TRAIN>
 __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte alignment for the swizzled operand tiles
@@ -304,7 +307,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
           const float t0 = b < a.d ? sW0[c * kW0Stride + b] / a.norm[a.d + b] : sW0[c * kW0Stride + kTcLat + b - a.d];
           hv[j] = act_d2(a.act, z[j]) * zd[j] * t0;
         }
-        if (a.dstore && ri.cls == 0)
+        if (TRAIN && ri.cls == 0)
           a.dstore[(int64_t)c * a.rows_total + tile * 128 + rw] = __float2bfloat16_rn(act_slope_record(a.act, z[j]));
       }
       store_operand<SPLIT>(atile, rw, c0, hv);
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
       }
       // training: the previous layer's activations leave the operand tile while the tensor core
       // reads it (both are reads; the barrier after the wait orders them before the next writes)
-      if (!SPLIT && a.astore && l >= 0)
+      if (TRAIN && l >= 0)
         copy_out_tile(a.astore + (int64_t)l * kW * a.rows_total, a.rows_total, atile, tile, t);
       if (!tc::mbar_wait(&tail->bar_mma, mma_phase)) {
         raise_status(a.status, STATUS_TIMEOUT);
@@ -399,7 +402,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
           // training: the primal rows' activation slopes (the backward's act' and act'' terms), from
           // the published pre-activations, spread over the half's four warps: feature = lane, 8 rows
           // per thread, one 16-byte store of 8 rows of one feature (the training calls have R > 1)
-          if (a.dstore) {
+          if (TRAIN) {
             for (int k = warp & 3; 8 * k < a.Pt; k += 4) {
               float v[8];
 #pragma unroll
@@ -424,7 +427,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
         }
         // the primal row of point q is tile row q (kind index 0)
         const float* zq = xh + ri.q * kXbStride;
-        if (a.dstore) {
+        if (TRAIN) {
           // training (primal and tangent rows only): the slope s of the primal row, e^z where z < 0
           // and -1 elsewhere, gives both activations without another exponential: ELU(z) = s - 1
           // (z where s < 0), act'(z) = s (1 where s < 0); the same values as below
@@ -470,7 +473,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
           }
         }
         // the next layer's operand tile; in training also the last layer's, for the copy-out
-        if (!last || (!SPLIT && a.astore)) {
+        if (!last || TRAIN) {
 #pragma unroll
           for (int j = 0; j < 32; j += 8) store_operand<SPLIT>(atile, rw, ch * 32 + j, acc + j);
         }
@@ -488,7 +491,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decoder_tc(DecArgs a) {
     __syncthreads();
     // training: the last layer's activations (the barrier at the end of the tile orders these
     // reads before the next tile's first operand writes)
-    if (!SPLIT && a.astore) copy_out_tile(a.astore + (int64_t)a.n_tc * kW * a.rows_total, a.rows_total, atile, tile, t);
+    if (TRAIN) copy_out_tile(a.astore + (int64_t)a.n_tc * kW * a.rows_total, a.rows_total, atile, tile, t);
     if (h == 0 && ri.cls >= 0) {
       const int kidx = rw / a.Pt;  // position of this row's kind in `kinds`
       float* o = a.out + ((int64_t)kidx * a.n + ri.p) * a.d;
@@ -1278,7 +1281,7 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
 // NS tile slots in turn, one MMA issuer warp per slot.  All weights are resident (four 32 KB layers
 // and the first layer's split image), and the A operand sits in tensor memory alone: 64 columns of
 // BF16 activations, or for the first layer 16 + 16 of the inputs' high and low parts.  The
-// arithmetic and its order are decoder_tc<false>'s, so the results are the same bits.
+// arithmetic and its order are decoder_tc's (without SPLIT), so the results are the same bits.
 //
 // TRAIN: whole points only (pipe_U = R floor(32 / R) rows per lane group, the other lanes idle); every
 // layer's operand is also stored as the tile image the MMA reads (128 rows x 128 BF16 in the 128-byte
@@ -1854,9 +1857,11 @@ mpm_status decoder_create(const decoder_desc* desc, mpm_decoder** out) {
   if (e == cudaSuccess) e = cudaMemset(dec->params, 0, sizeof(float) * dec->n_params);
   if (e == cudaSuccess) e = cudaMemset(dec->status, 0, sizeof(uint32_t));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(decoder_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec->smem);
+    e = cudaFuncSetAttribute(decoder_tc<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec->smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(decoder_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec->smem_split);
+    e = cudaFuncSetAttribute(decoder_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec->smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(decoder_tc<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec->smem_split);
   if (e == cudaSuccess) e = pipe_limits();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(decoder_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dec_f32_smem_bytes());
@@ -2064,9 +2069,11 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
     const int64_t tiles = (n + a.Pt - 1) / a.Pt;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, dec->n_sm));
     if (dec->fp32 == 2 && !a.dstore)
-      decoder_tc<true><<<blocks, kDecThreads, dec->smem_split, s>>>(a);
+      decoder_tc<true, false><<<blocks, kDecThreads, dec->smem_split, s>>>(a);
+    else if (a.dstore)
+      decoder_tc<false, true><<<blocks, kDecThreads, dec->smem, s>>>(a);
     else
-      decoder_tc<false><<<blocks, kDecThreads, dec->smem, s>>>(a);
+      decoder_tc<false, false><<<blocks, kDecThreads, dec->smem, s>>>(a);
   }
   MPM_CUDA_TRY(cudaGetLastError());
   return MPM_OK;
