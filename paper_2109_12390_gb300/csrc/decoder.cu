@@ -1591,86 +1591,82 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
   if (warp == 0) tc::tmem_free<256 * NS>(tail->tmem);
 }
 
-// Transposed FP32 copies of the square layers for the CUDA-core path:
-// WT[l][k][f] = W[l][f][k].
-__global__ void decoder_transpose(const float* W, int n_layers, float* WT) {
-  __shared__ float tileT[32][33];
-  for (int l = 0; l < n_layers; ++l) {
-    for (int b = blockIdx.x; b < 16; b += gridDim.x) {
-      const int f0 = (b / 4) * 32, k0 = (b % 4) * 32;
-      const int tx = threadIdx.x & 31, tyy = threadIdx.x >> 5;
-      for (int y = tyy; y < 32; y += blockDim.x / 32) tileT[y][tx] = W[(size_t)l * kW * kW + (f0 + y) * kW + k0 + tx];
-      __syncthreads();
-      for (int y = tyy; y < 32; y += blockDim.x / 32) WT[(size_t)l * kW * kW + (k0 + y) * kW + f0 + tx] = tileT[tx][y];
-      __syncthreads();
-    }
-  }
+// Everything the kernels read in another form than the parameter vector's, in one launch (it runs after
+// every optimisation step; as eight copies and four kernels a parameter change took 52 us, like this 14.5):
+//   bsq      the square layers' biases, contiguous
+//   wsqT     the square layers transposed, WT[l][k][f] = W[l][f][k] (decoder_f32)
+//   wimg     bf16(w), and wimg_lo bf16(w - bf16(w)), in the 128-byte swizzled K-major layout the MMA reads
+//   wstream  decoder_tc3's: per layer the low, middle and high BF16 images (w = hi + mid + lo exactly, each rounded
+//            to nearest) as atoms of 128 output rows x 64 K in the same layout: the first layer (padded
+//            inputs, at most 42) one atom per image, the square layers two
+//   w0img    the first layer for the tensor cores where its padded inputs fit 32: bf16(w) at K 0 .. 31 of a row,
+//            bf16(w - bf16(w)) at 32 .. 63 (one 16 KB atom column)
+// Padded inputs: coordinates at 0 .. 3, latents from kTcLat, zero where no input sits.
+// Blocks of 256 threads: one per 32 x 32 tile of a square layer, then kDeriveW0 for the first layer and the biases.
+constexpr int kDeriveThreads = 256, kDeriveW0 = kW * 64 / 1024;
+struct DeriveArgs {
+  const float* W0;          // (W, d + r)
+  const float* sq;          // first square layer, each kW * kW weights and kW biases
+  int d, r, n_tc;
+  float *bsq, *wsqT;
+  uint8_t *wimg, *wimg_lo, *wstream, *w0img;   // w0img may be null
+};
+
+__device__ __forceinline__ void put_bf16(uint8_t* img, size_t at, __nv_bfloat16 v) {
+  *reinterpret_cast<__nv_bfloat16*>(img + at) = v;
 }
 
-// Packs the square-layer weights (FP32, (out, in) row-major) into BF16 images
-// in the 128-byte swizzled K-major layout the MMA reads: img = bf16(w) and, when
-// img_lo is set, img_lo = bf16(w - bf16(w)) (the split operands).
-__global__ void decoder_pack(const float* W, int n_layers, int64_t stride, uint8_t* img, uint8_t* img_lo) {
-  const int64_t total = (int64_t)n_layers * kW * kW;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    int l = (int)(i / (kW * kW));
-    int rem = (int)(i % (kW * kW));
-    int row = rem / kW, k = rem % kW;
-    const float w = W[l * stride + rem];
-    const __nv_bfloat16 v = __float2bfloat16_rn(w);
-    const size_t o = (size_t)l * kLayerBytes + tc::sw128_offset(row, k, kW);
-    *reinterpret_cast<__nv_bfloat16*>(img + o) = v;
-    if (img_lo) *reinterpret_cast<__nv_bfloat16*>(img_lo + o) = __float2bfloat16_rn(w - __bfloat162float(v));
-  }
-}
-
-// Packs the first layer (FP32, (W, d + r) row-major) for the tensor cores: row c of the image
-// holds bf16(w) of the padded inputs (coordinates at 0 .. 3, latents from kTcLat) at K 0 .. 31
-// and bf16(w - bf16(w)) at K 32 .. 63, zero where no input sits, in the 128-byte swizzled
-// K-major layout (one 16 KB atom column).
-__global__ void decoder_pack_w0(const float* W0, int d, int r, uint8_t* img) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kW * 32; e += gridDim.x * blockDim.x) {
-    const int c = e / 32, ii = e % 32;
-    const int i = ii < kTcLat ? (ii < d ? ii : -1) : (ii - kTcLat < r ? d + ii - kTcLat : -1);
-    const float w = i >= 0 ? W0[c * (d + r) + i] : 0.f;
-    const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-    *reinterpret_cast<__nv_bfloat16*>(img + tc::sw128_offset(c, ii, kW)) = hi;
-    *reinterpret_cast<__nv_bfloat16*>(img + tc::sw128_offset(c, 32 + ii, kW)) =
-        __float2bfloat16_rn(w - __bfloat162float(hi));
-  }
-}
-
-// Weight stream of decoder_tc3: per layer its low, middle and high BF16 images (w = hi + mid + lo
-// exactly, each rounded to nearest), as atoms of 128 output rows x 64 K in the 128-byte swizzled
-// K-major layout: the first layer (padded inputs, at most 42) one atom per image, the square layers
-// two.
-__global__ void decoder_pack3(const float* W0, int d, int r, const float* wsq, int n_tc, uint8_t* out) {
-  const int64_t total = (int64_t)(1 + 2 * n_tc) * kW * 64;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int blk = (int)(e / (kW * 64)), rem = (int)(e % (kW * 64));
-    const int row = rem / 64, k = rem % 64;
+__global__ void __launch_bounds__(kDeriveThreads) decoder_derive(DeriveArgs a) {
+  __shared__ float tile[32][33];
+  const int t = threadIdx.x;
+  const int b = (int)blockIdx.x - 16 * a.n_tc;
+  const bool square = b < 0;
+  const int l = (int)blockIdx.x / 16, f0 = ((int)blockIdx.x / 4 % 4) * 32, k0 = ((int)blockIdx.x % 4) * 32;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    int row, k;             // output feature, input (square layers: of 128; first layer: of 64 padded)
     float w;
-    int64_t at;   // low atom, and the distance to the next image's
-    int step;
-    if (blk == 0) {
-      const int i = k < kTcLat ? (k < d ? k : -1) : (k - kTcLat < r ? d + k - kTcLat : -1);
-      w = i >= 0 ? W0[row * (d + r) + i] : 0.f;
+    size_t at, step;        // low image's atom, and the distance to the next image's
+    if (square) {
+      row = f0 + t / 32 + 8 * i;
+      k = k0 + t % 32;
+      w = a.sq[(size_t)l * (kW * kW + kW) + row * kW + k];
+      at = 3 + 6 * (size_t)l + k / 64;
+      step = 2;
+      tile[t / 32 + 8 * i][t % 32] = w;
+    } else {
+      const int e = b * 1024 + t + kDeriveThreads * i;
+      row = e / 64;
+      k = e % 64;
+      const int in = k < kTcLat ? (k < a.d ? k : -1) : (k - kTcLat < a.r ? a.d + k - kTcLat : -1);
+      w = in >= 0 ? a.W0[row * (a.d + a.r) + in] : 0.f;
       at = 0;
       step = 1;
-    } else {
-      const int l = (blk - 1) / 2, kh = (blk - 1) & 1;
-      w = wsq[((int64_t)l * kW + row) * kW + kh * 64 + k];
-      at = 3 + 6 * l + kh;
-      step = 2;
     }
     const __nv_bfloat16 hi = __float2bfloat16_rn(w);
     const float r1 = w - __bfloat162float(hi);
     const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
     const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-    uint8_t* o = out + at * kAtomBytes + tc::sw128_offset(row, k, kW);
-    *reinterpret_cast<__nv_bfloat16*>(o) = lo;
-    *reinterpret_cast<__nv_bfloat16*>(o + step * kAtomBytes) = mid;
-    *reinterpret_cast<__nv_bfloat16*>(o + 2 * step * kAtomBytes) = hi;
+    const size_t o = at * kAtomBytes + tc::sw128_offset(row, k & 63, kW);
+    put_bf16(a.wstream, o, lo);
+    put_bf16(a.wstream, o + step * kAtomBytes, mid);
+    put_bf16(a.wstream, o + 2 * step * kAtomBytes, hi);
+    if (square) {
+      const size_t q = (size_t)l * kLayerBytes + tc::sw128_offset(row, k, kW);
+      put_bf16(a.wimg, q, hi);
+      put_bf16(a.wimg_lo, q, mid);
+    } else if (a.w0img && k < 32) {
+      put_bf16(a.w0img, tc::sw128_offset(row, k, kW), hi);
+      put_bf16(a.w0img, tc::sw128_offset(row, 32 + k, kW), mid);
+    }
+  }
+  if (square) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      a.wsqT[(size_t)l * kW * kW + (k0 + t / 32 + 8 * i) * kW + f0 + t % 32] = tile[t % 32][t / 32 + 8 * i];
+  } else if (b == 0) {
+    for (int e = t; e < a.n_tc * kW; e += kDeriveThreads) a.bsq[e] = a.sq[(size_t)(e / kW) * (kW * kW + kW) + kW * kW + e % kW];
   }
 }
 
@@ -1754,25 +1750,11 @@ size_t dec_f32_smem_bytes() {
 
 mpm_status refresh_derived_impl(mpm_decoder* dec, cudaStream_t s) {
   if (dec->n_tc == 0) return MPM_OK;
-  for (int l = 0; l < dec->n_tc; ++l) {
-    MPM_CUDA_TRY(cudaMemcpyAsync(dec->wsq + (size_t)l * kW * kW, dec->params + dec->w_off[1 + l],
-                                 sizeof(float) * kW * kW, cudaMemcpyDeviceToDevice, s));
-    MPM_CUDA_TRY(cudaMemcpyAsync(dec->bsq + (size_t)l * kW, dec->params + dec->b_off[1 + l], sizeof(float) * kW,
-                                 cudaMemcpyDeviceToDevice, s));
-  }
-  decoder_pack<<<std::max(1, std::min(dec->n_sm * 4, dec->n_tc * 64)), 256, 0, s>>>(dec->wsq, dec->n_tc,
-                                                                                    (int64_t)kW * kW, dec->wimg,
-                                                                                    dec->wimg_lo);
+  const DeriveArgs a{dec->params + dec->w_off[0], dec->params + dec->w_off[1], dec->d,       dec->r,
+                     dec->n_tc,                   dec->bsq,                    dec->wsqT,    dec->wimg,
+                     dec->wimg_lo,                dec->wstream,                dec->w0img};
+  decoder_derive<<<16 * dec->n_tc + kDeriveW0, kDeriveThreads, 0, s>>>(a);
   MPM_CUDA_TRY(cudaGetLastError());
-  decoder_transpose<<<16, 256, 0, s>>>(dec->wsq, dec->n_tc, dec->wsqT);
-  MPM_CUDA_TRY(cudaGetLastError());
-  decoder_pack3<<<std::max(1, std::min(dec->n_sm * 4, (1 + 2 * dec->n_tc) * 32)), 256, 0, s>>>(
-      dec->params + dec->w_off[0], dec->d, dec->r, dec->wsq, dec->n_tc, dec->wstream);
-  MPM_CUDA_TRY(cudaGetLastError());
-  if (dec->w0img) {
-    decoder_pack_w0<<<16, 256, 0, s>>>(dec->params + dec->w_off[0], dec->d, dec->r, dec->w0img);
-    MPM_CUDA_TRY(cudaGetLastError());
-  }
   return MPM_OK;
 }
 
@@ -1836,7 +1818,7 @@ mpm_status decoder_create(const decoder_desc* desc, mpm_decoder** out) {
   const size_t sq = sizeof(float) * dec->n_tc * kW * kW, img = (size_t)dec->n_tc * kLayerBytes;
   const size_t o_params = place(sizeof(float) * dec->n_params), o_norm = place(sizeof(float) * 4 * dec->d);
   const size_t o_status = place(sizeof(uint32_t));
-  const size_t o_wsq = place(sq), o_bsq = place(sizeof(float) * dec->n_tc * kW), o_wsqT = place(sq);
+  const size_t o_bsq = place(sizeof(float) * dec->n_tc * kW), o_wsqT = place(sq);
   const size_t o_wimg = place(img), o_wimg_lo = place(img), o_w0img = place(kLayerBytes / 2);
   const size_t o_wstream = place(dec->n_tc > 0 ? (size_t)(3 + 6 * dec->n_tc) * kAtomBytes : 0);
   cudaError_t e = cudaMalloc((void**)&dec->pool, bytes);
@@ -1845,7 +1827,6 @@ mpm_status decoder_create(const decoder_desc* desc, mpm_decoder** out) {
     dec->norm = (float*)(dec->pool + o_norm);
     dec->status = (uint32_t*)(dec->pool + o_status);
     if (dec->n_tc > 0) {
-      dec->wsq = (float*)(dec->pool + o_wsq);
       dec->bsq = (float*)(dec->pool + o_bsq);
       dec->wsqT = (float*)(dec->pool + o_wsqT);
       dec->wimg = dec->pool + o_wimg;
@@ -1949,7 +1930,6 @@ static mpm_status decoder_launch(const mpm_decoder* dec, const float* X, const i
   a.wimg = dec->wimg;
   a.wimg_lo = dec->wimg_lo;
   a.w0img = dec->w0img;
-  a.wsq = dec->wsq;
   a.wstream = dec->wstream;
   a.wsqT = dec->wsqT;
   a.X = X;

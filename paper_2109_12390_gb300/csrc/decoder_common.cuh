@@ -31,10 +31,9 @@ struct DecArgs {
   // padded layout): rows = output features, hi at K 0 .. 31 and lo at K 32 .. 63 of one
   // 128-byte swizzled row; null when the first layer runs on the CUDA cores
   const uint8_t* w0img;
-  // every layer's weights as three BF16 images (decoder_pack3) in the order decoder_tc3 reads them
+  // every layer's weights as three BF16 images (decoder_derive) in the order decoder_tc3 reads them
   const uint8_t* wstream;
-  const float* wsq;   // (n_tc, W, W) FP32 square-layer weights, (out, in) row-major
-  const float* wsqT;  // (n_tc, W, W) the same transposed, (in, out) row-major
+  const float* wsqT;  // (n_tc, W, W) FP32 square-layer weights transposed, (in, out) row-major
   const float* X;
   const int32_t* lat;
   const float* latents;
@@ -358,8 +357,7 @@ struct mpm_decoder {
   uint8_t* pool = nullptr;            // the one allocation that holds the buffers below
   float* params = nullptr;            // FP32 master copy
   float* norm = nullptr;
-  float* wsq = nullptr;               // square-layer weights gathered contiguously (n_tc, W, W)
-  float* bsq = nullptr;               // their biases (n_tc, W)
+  float* bsq = nullptr;               // square-layer biases gathered contiguously (n_tc, W)
   float* wsqT = nullptr;              // transposed FP32 copies (n_tc, W, W) for the CUDA-core path
   uint8_t* wimg = nullptr;            // BF16 swizzled images
   uint8_t* wimg_lo = nullptr;         // residual images bf16(w - bf16(w)) for the split-BF16 path
