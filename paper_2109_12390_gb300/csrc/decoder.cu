@@ -995,8 +995,8 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc<256 * NS>(&tail->tmem);
-  for (int e = t; e < kW; e += tc3_threads<NS>()) sb0[e] = a.b0[e];
-  for (int e = t; e < a.n_tc * kW; e += tc3_threads<NS>()) sbh[e] = a.bh[e];
+  for (int e = t; e < kW; e += tc3_threads<NS>()) sb0[e] = finite_bias(a.b0[e]);
+  for (int e = t; e < a.n_tc * kW; e += tc3_threads<NS>()) sbh[e] = finite_bias(a.bh[e]);
   for (int e = t; e < 3 * kW; e += tc3_threads<NS>()) sWout[e] = e < a.d * kW ? a.Wout[e] : 0.f;
   if (t < 2 * a.d) snorm[t] = a.norm[t];
   tc::tc_fence_before();
@@ -1336,8 +1336,8 @@ __global__ void __launch_bounds__(bf16_threads<NS>(), 1) decoder_bf16(DecArgs a)
       tc::bulk_g2s(wsm + l * kLayerBytes, a.wimg + (size_t)l * kLayerBytes, kLayerBytes, &tail->bar_w);
   }
   if (warp == 0) tc::tmem_alloc<256 * NS>(&tail->tmem);
-  for (int e = t; e < kW; e += bf16_threads<NS>()) sb0[e] = a.b0[e];
-  for (int e = t; e < a.n_tc * kW; e += bf16_threads<NS>()) sbh[e] = a.bh[e];
+  for (int e = t; e < kW; e += bf16_threads<NS>()) sb0[e] = finite_bias(a.b0[e]);
+  for (int e = t; e < a.n_tc * kW; e += bf16_threads<NS>()) sbh[e] = finite_bias(a.bh[e]);
   for (int e = t; e < 3 * kW; e += bf16_threads<NS>()) sWout[e] = e < a.d * kW ? a.Wout[e] : 0.f;
   if (t < 2 * a.d) snorm[t] = a.norm[t];
   tc::tc_fence_before();
