@@ -867,8 +867,8 @@ __global__ void __launch_bounds__(kF32Threads, 1) decoder_f32(DecArgs a) {
 // overlapped.  262,144 points x 4 rows, r = 16: 0.63 ms (decoder_f32: 5.07 ms), distance from 64 bits
 // 4e-8 .. 7e-8 (6.5e-8); 256 points x 17 rows: 24 us (31 us); 20,000 points x 12 rows with secants:
 // 0.34 ms (1.36 ms).
-// After a wait that ran out nothing waits on the copies or MMAs any more: the pass runs to its end
-// (in bounds, its results void) with the TIMEOUT status raised.
+// After a wait that ran out nothing waits on the copies or MMAs any more and no more weights are fetched: the
+// pass runs to its end (in bounds, its results void) with the TIMEOUT status raised.
 // --------------------------------------------------------------------------
 constexpr int kRing = 9;
 template <int NS>
@@ -1013,21 +1013,20 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
   const int KS0 = (K0 + 15) / 16;                         // their K steps
   const int atoms = 3 + 6 * a.n_tc;
 
+  uint32_t fetched = 0;   // weight copies this thread started
   if (warp == kEpiThreads / 32) {
     // ---- weight stream
     if (lane == 0) {
-      uint32_t i = 0;
-      for (int it = blockIdx.x; it < n_iter; it += gridDim.x)
-        for (int j = 0; j < atoms; ++j, ++i) {
-          const uint32_t slot = i % kRing, use = i / kRing;
-          if (use > 0) pipe_wait(a.status, &tail->abort, &tail->empty[slot], (use - 1) & 1u);
-          tc::mbar_expect_tx(&tail->full[slot], (uint32_t)kAtomBytes);
-          tc::bulk_g2s(ring + slot * kAtomBytes, a.wstream + (size_t)j * kAtomBytes, kAtomBytes, &tail->full[slot]);
-        }
-      // the last copies land before the CTA exits (only a timed-out pass leaves any in flight)
-      if (*(volatile int*)&tail->abort)
-        for (uint32_t k = i > kRing ? i - kRing : 0; k < i; ++k)
-          (void)tc::mbar_wait(&tail->full[k % kRing], (k / kRing) & 1u);
+      const uint32_t passes = (int)blockIdx.x < n_iter ? (uint32_t)(n_iter - 1 - (int)blockIdx.x) / gridDim.x + 1 : 0;
+      int j = 0;   // atom of the pass
+      fetched = ring_fill<kRing>(
+          passes * (uint32_t)atoms,
+          [&](uint32_t slot, uint32_t phase) { return pipe_wait(a.status, &tail->abort, &tail->empty[slot], phase); },
+          [&](uint32_t slot, uint32_t) {
+            tc::mbar_expect_tx(&tail->full[slot], (uint32_t)kAtomBytes);
+            tc::bulk_g2s(ring + slot * kAtomBytes, a.wstream + (size_t)j * kAtomBytes, kAtomBytes, &tail->full[slot]);
+            j = j + 1 < atoms ? j + 1 : 0;
+          });
     }
     __syncwarp();
   } else if (warp > kEpiThreads / 32) {
@@ -1271,6 +1270,9 @@ __global__ void __launch_bounds__(tc3_threads<NS>(), 1) decoder_tc3(DecArgs a) {
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  // after a timeout the last copies land before the CTA exits
+  if (fetched > 0 && *(volatile int*)&tail->abort)
+    ring_land<kRing>(fetched, [&](uint32_t slot, uint32_t phase) { (void)tc::mbar_wait(&tail->full[slot], phase); });
   if (warp == 0) tc::tmem_free<256 * NS>(tail->tmem);
 }
 

@@ -4,19 +4,20 @@
 #pragma once
 
 #include "decoder_common.cuh"
+#include "ring.cuh"
 
 namespace mpmrom {
 
 constexpr int kEpiThreads = 512;          // epilogue threads
 constexpr int kAtomBytes = kW * 128;      // 128 rows x 64 BF16
 
-// Bounded wait; after a timeout anywhere in the CTA no further waits are made.
-__device__ __forceinline__ void pipe_wait(uint32_t* status, int* abort, uint64_t* bar, uint32_t phase) {
-  if (*(volatile int*)abort) return;
-  if (!tc::mbar_wait(bar, phase)) {
-    raise_status(status, STATUS_TIMEOUT);
-    atomicExch(abort, 1);
-  }
+// Bounded wait; after a timeout anywhere in the CTA no further waits are made.  Whether the phase was seen complete.
+__device__ __forceinline__ bool pipe_wait(uint32_t* status, int* abort, uint64_t* bar, uint32_t phase) {
+  if (*(volatile int*)abort) return false;
+  if (tc::mbar_wait(bar, phase)) return true;
+  raise_status(status, STATUS_TIMEOUT);
+  atomicExch(abort, 1);
+  return false;
 }
 
 // Barriers 1 + s: the epilogue warps arrive when slot s's next operand is complete (and its

@@ -566,9 +566,11 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
     const uint32_t w_desc = tc::smem_desc_sw128_lo(tc::smem_addr(wt));
     constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW);
     const uint32_t slope_bytes = (uint32_t)(4 * ppg * 256);
-    uint32_t mma_phase = 0, full_phase = 0;
+    uint32_t mma_phase = 0;
+    Refill fill;                                         // the slot's fetches (the same in every lane)
     // activations and slopes of layer l of a tile into the slot
     auto fetch = [&](int tile, int l) {
+      if (!fill.start() || !leader) return;
       tc::mbar_expect_tx(&tail->full[s], (uint32_t)kLayerBytes + slope_bytes);
       tc::bulk_g2s(image, a.astore + ((int64_t)l * a.rows_total + (int64_t)tile * 128) * kW, kLayerBytes,
                    &tail->full[s]);
@@ -577,17 +579,14 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
     };
     pipe_wait(a.status, &tail->abort, &tail->bar_w, 0);
     __syncwarp();
-    bool first = true;
     for (int it = blockIdx.x; it < n_iter; it += gridDim.x) {
       const int tile = it * NT + s;
       if (s >= NT || tile >= n_tiles) continue;
-      if (first && leader) fetch(tile, a.n_hidden - 1);
-      first = false;
+      if (fill.n == 0) fetch(tile, a.n_hidden - 1);
       for (int l = a.n_hidden - 1; l >= 0; --l) {
         __syncwarp();
-        pipe_wait(a.status, &tail->abort, &tail->full[s], full_phase);
-        full_phase ^= 1u;
-        __syncwarp();
+        const bool landed = fill.live && pipe_wait(a.status, &tail->abort, &tail->full[s], fill.last_phase());
+        fill.seen(__all_sync(0xffffffffu, landed));
         tc::tc_fence_after();
         tc::tc_fence_before();
         pipe_arrive(3 + s);                              // data and (below the last layer) adjoints are there
@@ -604,11 +603,9 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
           __syncwarp();
           pipe_wait(a.status, &tail->abort, &tail->bar_mma[s], mma_phase);
           mma_phase ^= 1u;
-          if (leader) {
-            tc::bulk_wait_read();
-            fetch(tile, l - 1);
-          }
-        } else if (leader) {
+          if (leader) tc::bulk_wait_read();
+          fetch(tile, l - 1);
+        } else {
           const int next = (it + (int)gridDim.x) * NT + s;
           if (it + (int)gridDim.x < n_iter && next < n_tiles) fetch(next, a.n_hidden - 1);
         }
@@ -622,10 +619,8 @@ __global__ void __launch_bounds__(kBwdPipeThreads, 1) train_bwd_pipe(BwdArgs a) 
     }
     __syncwarp();
     (void)tc::mbar_wait(&tail->drain, 0);
-    if (*(volatile int*)&tail->abort) {
-      (void)tc::mbar_wait(&tail->bar_w, 0);
-      if (!first) (void)tc::mbar_wait(&tail->full[s], full_phase ^ 1u);
-    }
+    if (*(volatile int*)&tail->abort) (void)tc::mbar_wait(&tail->bar_w, 0);
+    if (!fill.live) (void)tc::mbar_wait(&tail->full[s], fill.last_phase());
     __syncwarp();
   } else {
     const int h = warp >> 2, lg = warp & 3;
@@ -976,22 +971,21 @@ __global__ void __launch_bounds__(128, 2) train_dw_gemm_image(const __nv_bfloat1
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem = tslot;
+  uint32_t fetched = 0;   // stages this thread started to fill
   if (t == 0) {
-    for (int b = 0; b < n_blk; ++b) {
-      const int st = b % kDwStages;
-      if (b >= kDwStages) pipe_wait(status, &abort_flag, &empty[st], (uint32_t)((b / kDwStages - 1) & 1));
-      const int64_t row = k0 + 64 * (int64_t)b;
-      const int64_t at = (row >> 7) * kLayerBytes + (row & 64) * 128;   // half of 64 features: 16 KB apart
-      uint8_t* dst = stages + st * kDwStageBytes;
-      tc::mbar_expect_tx(&full[st], (uint32_t)kDwStageBytes);
-      tc::bulk_g2s(dst, Z + at, 8192, &full[st]);
-      tc::bulk_g2s(dst + 8192, Z + at + kLayerBytes / 2, 8192, &full[st]);
-      tc::bulk_g2s(dst + 16384, A + at, 8192, &full[st]);
-      tc::bulk_g2s(dst + 24576, A + at + kLayerBytes / 2, 8192, &full[st]);
-    }
-    if (*(volatile int*)&abort_flag)   // after a timeout the last copies land before the CTA exits
-      for (int b = max(0, n_blk - kDwStages); b < n_blk; ++b)
-        (void)tc::mbar_wait(&full[b % kDwStages], (uint32_t)((b / kDwStages) & 1));
+    fetched = ring_fill<kDwStages>(
+        (uint32_t)n_blk,
+        [&](uint32_t st, uint32_t phase) { return pipe_wait(status, &abort_flag, &empty[st], phase); },
+        [&](uint32_t st, uint32_t b) {
+          const int64_t row = k0 + 64 * (int64_t)b;
+          const int64_t at = (row >> 7) * kLayerBytes + (row & 64) * 128;   // half of 64 features: 16 KB apart
+          uint8_t* dst = stages + st * kDwStageBytes;
+          tc::mbar_expect_tx(&full[st], (uint32_t)kDwStageBytes);
+          tc::bulk_g2s(dst, Z + at, 8192, &full[st]);
+          tc::bulk_g2s(dst + 8192, Z + at + kLayerBytes / 2, 8192, &full[st]);
+          tc::bulk_g2s(dst + 16384, A + at, 8192, &full[st]);
+          tc::bulk_g2s(dst + 24576, A + at + kLayerBytes / 2, 8192, &full[st]);
+        });
   }
   if (t == 32) {
     constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kW) | (1u << 15) | (1u << 16);   // both operands transposed
@@ -1024,6 +1018,8 @@ __global__ void __launch_bounds__(128, 2) train_dw_gemm_image(const __nv_bfloat1
   }
   tc::tc_fence_before();
   __syncthreads();
+  if (fetched > 0 && *(volatile int*)&abort_flag)   // after a timeout the last copies land before the CTA exits
+    ring_land<kDwStages>(fetched, [&](uint32_t st, uint32_t phase) { (void)tc::mbar_wait(&full[st], phase); });
   tc::tc_fence_after();
   if (warp == 0) tc::tmem_free<kW>(tmem);
 }
