@@ -374,15 +374,18 @@ mpm_status decoder_status_word(mpm_decoder* dec, uint32_t* out, int clear, void*
  * the FP32 master weights, on the tensor cores with every operand the exact sum
  * of three BF16 numbers (six products, FP32 accumulation), or as FP32 GEMMs on
  * the CUDA cores where those are faster or their rounding is kept (mixed rows,
- * a lone caller's small calls with secant rows, gradients measured against a
- * reference configuration); it removes the BF16 rounding of positions and
- * gradients.  fp32 = 2:
+ * calls with secant rows of at most 31 rows per SM of the caller's share,
+ * gradients measured against a reference configuration); it removes the BF16
+ * rounding of positions and gradients.  Finite values: an infinite activation
+ * gives NaN on the tensor cores (an infinite bias is taken as the largest finite
+ * number).  fp32 = 2:
  * split BF16 on the tensor cores: activations and weights are each the sum of
  * two BF16 numbers (hi = bf16(v), lo = bf16(v - hi)) and every product is
  * A_hi W_hi + A_hi W_lo + A_lo W_hi accumulated in FP32, so each product keeps
  * about 16 bits (relative error near 2^-16 against 2^-24 for FP32, against
- * 2^-8 for BF16) at tensor-core throughput: for many concurrent reduced-order
- * instances.  The output layer is FP32 in every mode, the first layer FP32 in
+ * 2^-8 for BF16): for large calls with mixed rows, which fp32 = 1 takes on the
+ * CUDA cores; others are nearer and faster with fp32 = 1 (20,000 points x 12 rows
+ * with secants 0.32 against 1.28 ms).  The output layer is FP32 in every mode, the first layer FP32 in
  * modes 1 and 2 and split BF16 in mode 0 (FP32 there when r > 28).  Takes effect
  * for reduced-order contexts created afterwards.  Errors: MPM_EINVAL.
  */

@@ -1875,7 +1875,7 @@ mpm_status decoder_set_concurrency(mpm_decoder* dec, int k) {
 
 mpm_status decoder_set_precision(mpm_decoder* dec, int fp32) {
   MPM_CHECK_ARG(dec, "null decoder");
-  MPM_CHECK_ARG(fp32 >= 0 && fp32 <= 2, "precision: 0 BF16, 1 FP32 CUDA cores, 2 split BF16 tensor cores");
+  MPM_CHECK_ARG(fp32 >= 0 && fp32 <= 2, "precision: 0 BF16, 1 FP32, 2 split BF16");
   dec->fp32 = fp32;
   return MPM_OK;
 }

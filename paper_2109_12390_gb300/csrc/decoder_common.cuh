@@ -367,7 +367,7 @@ struct mpm_decoder {
   int n_sm = 0;
   size_t smem = 0;
   size_t smem_split = 0;
-  int fp32 = 0;                       // square layers: 0 BF16 tensor cores, 1 FP32 CUDA cores, 2 split BF16 tensor cores
+  int fp32 = 0;                       // square layers: 0 BF16, 1 FP32 (tensor or CUDA cores), 2 split BF16
   int concurrency = 1;                // expected concurrent calls (FP32 tiling)
 };
 

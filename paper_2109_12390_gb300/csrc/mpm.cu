@@ -1380,8 +1380,10 @@ mpm_status mpm_init(const mpm_config* cfg, mpm_ctx** out) {
   p.mu_lam = c->mu_lam;
   p.sv_lo = 1.f - cfg->plastic_compression;
   p.sv_hi = 1.f + cfg->plastic_stretch;
-  // several CTAs per resident place, so that the hardware evens out items of different length (a CTA
-  // without an item ends at once): 16 bodies in 2D 926 us with 8 per SM, 776 with 16, 752 with 24
+  // several CTAs per resident place, so that the hardware evens out items of different length: 16 bodies
+  // in 2D 926 us with 8 per SM, 776 with 16, 752 with 24.  max_work counts every grid block, so on a large, mostly
+  // empty grid most of them find no item and end at once: 10,000 particles in 16 bodies on 512^2 cells each 52.1 us
+  // a step with 8 per SM, 52.2 with 24; 57,600 there 21.5 and 20.3
   c->fused_grid = std::max(1, std::min(c->max_work, c->n_sm * 24));
   *out = c;
   return MPM_OK;
@@ -1809,6 +1811,8 @@ mpm_status mpm_step_noalloc(const mpm_config* cfg, float* x, float* v, float* F,
   p.mu_lam = c.mu_lam;
   p.sv_lo = 1.f - cfg->plastic_compression;
   p.sv_hi = 1.f + cfg->plastic_stretch;
+  // (items and CTAs stay at the sizes that item_rule starts from: smaller items would need a longer work list,
+  // and a configuration that just fits the scratch would be refused)
   c.fused_grid = std::max(1, std::min(c.max_work, c.n_sm * 8));
   // load the caller's state, bin it and transfer it to the grid, then step
   c.cur = 0;

@@ -153,8 +153,8 @@ def build_serving_batch(decoders, roms, concurrency, precision=None):
 
 def autotune_serving(decoders, roms, candidates=(1, 8, 32, 128, 512), precisions=(1, 2), trial_steps=4):
     """Decoder arithmetic and tiling for batched serving, chosen by measurement: for the FP32
-    CUDA-core arithmetic each candidate concurrency k (how many decoder calls are expected to run
-    at once, which sets how many SMs one call's tiles spread over), and the split-BF16 tensor-core
+    arithmetic each candidate concurrency k (how many decoder calls are expected to run
+    at once, which sets how many SMs one call's tiles spread over), and the split-BF16
     arithmetic (128-row tiles, no tiling choice); each configuration's batch is captured and
     `trial_steps` batch steps are timed on the device.  Returns ((precision, k) of the fastest,
     {"precision/k": ms per batch step}).  The trial steps advance the contexts."""
